@@ -249,9 +249,8 @@ hd_status hd_encode(const uint32_t *data_bits, uint32_t n, uint64_t num_codeword
     if (!data_bits || !stream) return HD_ERR_NULL;
     if (!aligned16(data_bits) || !aligned16(stream)) return HD_ERR_ALIGN;
     const uint32_t k = n - (uint32_t)m;
-    if (launch_encode_generic(data_bits, words_for_bits(num_codewords * k), n, num_codewords, stream,
-                              words_for_bits(num_codewords * n), static_cast<cudaStream_t>(cuda_stream)) !=
-        cudaSuccess)
+    if (launch_encode(data_bits, words_for_bits(num_codewords * k), n, num_codewords, stream,
+                      words_for_bits(num_codewords * n), static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return HD_ERR_CUDA;
     return HD_OK;
 }

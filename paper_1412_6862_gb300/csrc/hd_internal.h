@@ -46,8 +46,13 @@ inline int decode_grid(uint64_t want, uint64_t cap)
 cudaError_t launch_decode_generic(const uint32_t *in, uint64_t in_words, uint32_t n, uint64_t num_cw,
                                   uint64_t tile_begin, uint64_t tile_end, uint32_t *out, uint64_t out_words,
                                   void *syn, int syn_type, unsigned long long *err, cudaStream_t st);
-cudaError_t launch_encode_generic(const uint32_t *data, uint64_t data_words, uint32_t n, uint64_t num_cw,
-                                  uint32_t *stream, uint64_t stream_words, cudaStream_t st);
+
+// The encoders (any supported n, any length): data_words / stream_words are the
+// buffers' lengths; launched as programmatic dependents of the kernel ahead.
+cudaError_t launch_encode(const uint32_t *data, uint64_t data_words, uint32_t n, uint64_t num_cw, uint32_t *stream,
+                          uint64_t stream_words, cudaStream_t st);
+cudaError_t launch_encode_secded(const uint32_t *data, uint64_t data_words, uint32_t n, uint64_t num_cw,
+                                 uint32_t *stream, cudaStream_t st);
 
 // Launch `kern` on `st`, as the programmatic dependent of the kernel ahead of
 // it in the stream when pdl is set (it may then start before that kernel has

@@ -89,52 +89,6 @@ __global__ void __launch_bounds__(kTailWarps * 32)
     }
 }
 
-// One thread per codeword, bit-serial (builds inputs; not timed).  The stream must be zero.
-__global__ void k_encode_secded(const uint32_t *__restrict__ data, uint64_t data_words, uint32_t n, uint32_t m,
-                                uint64_t num_cw, uint32_t *__restrict__ stream)
-{
-    const uint32_t k = n - m, L = n + 1;
-    for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < num_cw;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t s = 0, par = 0, d = 0, win = 0;
-        for (uint32_t p = 3; p <= n; ++p) {  // checksum vector and parity of the data positions
-            if ((p & (p - 1u)) == 0) continue;
-            if ((d & 31u) == 0) win = load_window(data, data_words, (int64_t)(c * k + d));
-            if ((win >> (d & 31u)) & 1u) {
-                s ^= p;
-                par ^= 1u;
-            }
-            ++d;
-        }
-        par ^= __popc(s) & 1u;  // the checksum bits set to s
-        const uint64_t b0 = c * L, b1 = b0 + L;
-        uint32_t acc = 0;
-        d = 0;
-        for (uint32_t p = 0; p <= n; ++p) {
-            uint32_t bit;
-            if (p == 0) {
-                bit = par;
-            } else if ((p & (p - 1u)) == 0) {
-                bit = (s >> (31u - __clz(p))) & 1u;
-            } else {
-                if ((d & 31u) == 0) win = load_window(data, data_words, (int64_t)(c * k + d));
-                bit = (win >> (d & 31u)) & 1u;
-                ++d;
-            }
-            const uint64_t b = b0 + p;
-            acc |= bit << (b & 31u);
-            if ((b & 31u) == 31u || p == n) {
-                const uint64_t w = b >> 5;
-                if ((w << 5) >= b0 && (w << 5) + 32 <= b1)
-                    stream[w] = acc;
-                else if (acc)
-                    atomicOr(&stream[w], acc);
-                acc = 0;
-            }
-        }
-    }
-}
-
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -192,13 +146,9 @@ hd_status hd_encode_secded(const uint32_t *data_bits, uint32_t n, uint64_t num_c
     if (!aligned16(data_bits) || !aligned16(stream)) return HD_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const uint32_t k = n - (uint32_t)m;
-    if (cudaMemsetAsync(stream, 0, words_for_bits(num_codewords * (n + 1u)) * 4, st) != cudaSuccess)
-        return HD_ERR_CUDA;
-    const uint64_t want = (num_codewords + 255) / 256, cap = (uint64_t)num_sms() * 16;
-    k_encode_secded<<<(int)std::min(want, cap), 256, 0, st>>>(data_bits, words_for_bits(num_codewords * k), n,
-                                                              (uint32_t)m, num_codewords, stream);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? HD_OK : HD_ERR_CUDA;
+    return launch_encode_secded(data_bits, words_for_bits(num_codewords * k), n, num_codewords, stream, st) == cudaSuccess
+               ? HD_OK
+               : HD_ERR_CUDA;
 }
 
 }  // extern "C"
