@@ -54,6 +54,13 @@ cudaError_t launch_encode(const uint32_t *data, uint64_t data_words, uint32_t n,
 cudaError_t launch_encode_secded(const uint32_t *data, uint64_t data_words, uint32_t n, uint64_t num_cw,
                                  uint32_t *stream, cudaStream_t st);
 
+cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, uint64_t num_cw, uint32_t *stream,
+                                cudaStream_t st);
+
+// Resident CTAs per SM of a kernel with `smem` bytes of dynamic shared memory
+// (opted in to on first use), cached per device; <= 0 on failure.
+int stream_blocks_per_sm(const void *kernel, int threads, uint32_t smem);
+
 // Launch `kern` on `st`, as the programmatic dependent of the kernel ahead of
 // it in the stream when pdl is set (it may then start before that kernel has
 // finished, and must wait for it before touching what that kernel writes).

@@ -23,8 +23,7 @@
 //    long codewords, the few words that hold a checksum position.
 //  * k_short_small (n <= 255): warp tiles of 32 codewords straight from global
 //    memory, one codeword per lane, like the generic full-length kernel.
-// The encoder (k_encode_short) is bit-serial, one thread per codeword: it is
-// used to build inputs, not timed.
+// The encoder is in hd_short_encode.cu.
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
@@ -501,52 +500,6 @@ __global__ void __launch_bounds__(kSmallWarps * 32)
         grid_dep_wait();  // the counters' clear ahead of a programmatic dependent launch
         if (err && errs) atomicAdd(err, (unsigned long long)errs);
         if (det && dets) atomicAdd(det, (unsigned long long)dets);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Encoder: one thread per codeword, bit-serial.  The stream must be zero.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ bool is_pow2(uint32_t p) { return (p & (p - 1u)) == 0; }
-
-__global__ void k_encode_short(const uint32_t *__restrict__ data, uint64_t data_words, uint32_t n, uint32_t r,
-                               uint64_t num_cw, uint32_t *__restrict__ stream)
-{
-    const uint32_t k = n - r;
-    for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < num_cw;
-         c += (uint64_t)gridDim.x * blockDim.x) {
-        // checksum vector of the message placed at the data positions
-        uint32_t s = 0, d = 0, win = 0;
-        for (uint32_t p = 3; p <= n; ++p) {
-            if (is_pow2(p)) continue;
-            if ((d & 31u) == 0) win = load_window(data, data_words, (int64_t)(c * k + d));
-            if ((win >> (d & 31u)) & 1u) s ^= p;
-            ++d;
-        }
-        // write positions 1..n: checksum bit j at position 2^j makes the syndrome 0
-        const uint64_t b0 = c * n, b1 = b0 + n;
-        uint32_t acc = 0;
-        d = 0;
-        for (uint32_t p = 1; p <= n; ++p) {
-            uint32_t bit;
-            if (is_pow2(p)) {
-                bit = (s >> (31u - __clz(p))) & 1u;
-            } else {
-                if ((d & 31u) == 0) win = load_window(data, data_words, (int64_t)(c * k + d));
-                bit = (win >> (d & 31u)) & 1u;
-                ++d;
-            }
-            const uint64_t b = b0 + p - 1;
-            acc |= bit << (b & 31u);
-            if ((b & 31u) == 31u || p == n) {
-                const uint64_t w = b >> 5;
-                if ((w << 5) >= b0 && (w << 5) + 32 <= b1)
-                    stream[w] = acc;
-                else if (acc)
-                    atomicOr(&stream[w], acc);
-                acc = 0;
-            }
-        }
     }
 }
 
@@ -1080,12 +1033,7 @@ hd_status hd_encode_short(const uint32_t *data_bits, uint32_t n, uint64_t num_co
     if (!aligned16(data_bits) || !aligned16(stream)) return HD_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const uint32_t r = short_r(n), k = n - r;
-    if (cudaMemsetAsync(stream, 0, words_for_bits(num_codewords * n) * 4, st) != cudaSuccess) return HD_ERR_CUDA;
-    const uint64_t want = (num_codewords + 255) / 256, cap = (uint64_t)num_sms() * 16;
-    k_encode_short<<<(int)std::min(want, cap), 256, 0, st>>>(data_bits, words_for_bits(num_codewords * k), n, r,
-                                                             num_codewords, stream);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? HD_OK : HD_ERR_CUDA;
+    return launch_encode_short(data_bits, n, k, num_codewords, stream, st) == cudaSuccess ? HD_OK : HD_ERR_CUDA;
 }
 
 hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, void *cuda_stream, int32_t *chosen)

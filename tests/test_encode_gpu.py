@@ -59,3 +59,31 @@ def test_lane_path_edges(n, secded):
 def test_streaming_path_and_tail(n, cap):
     for N in (311_296, 311_297, 327_680, 327_680 + 1021):  # 311,296: the last one-codeword-per-lane size on 152 SMs
         _check(n, N, False, cap)
+
+
+# Segments of any length: below a word (a stream word holds several), at the
+# words' and the checksum positions' edges, the paper's lengths and the longest;
+# counts from one segment to several tiles per warp.
+@pytest.mark.parametrize("n,N", [
+    (3, 1), (3, 700_001), (4, 33), (7, 100_003), (16, 200_001), (30, 99_999), (31, 4097), (32, 4097), (33, 150_001),
+    (62, 5), (63, 9999), (64, 9999), (65, 120_007), (95, 3001), (96, 3001), (128, 70_001), (129, 2), (544, 60_001),
+    (1023, 777), (1024, 777), (1025, 20_011), (3212, 15_013), (8013, 3001), (16383, 7), (16384, 500), (16415, 501),
+    (32752, 3), (32767, 1), (32767, 1201)])
+@pytest.mark.parametrize("cap", [0, 3])
+def test_encode_short_paths(n, N, cap):
+    import torch
+    r, k = hd.hd_short_params(n)
+    data = synth.random_words(n * 3 + N, N * k)
+    want = gc.oracle_encode_parallel(oracle.encode_short, data, n, N, k, n)
+    if (N * k) % 32:
+        data = data.copy()
+        data[-1] |= np.uint32((0xFFFFFFFF << ((N * k) % 32)) & 0xFFFFFFFF)
+    out = torch.full((hd.words_for(N * n) + 8,), -1, dtype=torch.int32, device="cuda")
+    hd.hd_set_max_ctas(cap)
+    hd.encode_short(gc.to_device(data), n, N, out=out)
+    torch.cuda.synchronize()
+    hd.hd_set_max_ctas(0)
+    got = gc.host_u32(out)
+    bad = np.nonzero(got[:want.size] != want)[0]
+    assert bad.size == 0, f"n={n} N={N}: {bad.size} words differ, first {bad[:4]}"
+    assert (got[want.size:] == 0xFFFFFFFF).all()
