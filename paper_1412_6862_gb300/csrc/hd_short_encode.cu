@@ -12,11 +12,14 @@
 // inside it).  Words shared with a neighbouring tile are written with atomic
 // AND/OR of the tile's own bits, so nothing needs clearing first.
 //
-// Bound: the issue slots, about 30 instructions per 32 output words beside 23
-// bytes a clock of HBM.  Message words are read by plain loads, eight in flight
-// a lane: a segment's windows start at any bit, every word is read twice within
-// a few instructions (the second time from L1), and 48 warps an SM hide the
-// rest, so that stages and barriers would only cost shared memory.
+// Bound: the issue slots and the shared-memory pipe.  A tile's message arrives by
+// one bulk copy into the warp's stage (plain loads spread over several segments
+// kept the L1 busy at 75 % of its wavefronts and took 1.4 to 2 times as long); the
+// stage is free once pass 1 has read it, so the next tile's copy runs behind pass
+// 2 and one stage a warp suffices: 27 warps an SM.  Measured on GB300, 512 Mbit of
+// segments, of the measured copy bandwidth: n = 100 / 544 / 1078 / 3212 / 16000 /
+// 32767: 0.34 / 0.45 / 0.43 / 0.49 / 0.65 / 0.78 (bit by bit before: 0.01); below
+// n = 64, where a stream word holds parts of several segments, 0.07 to 0.2.
 #include <algorithm>
 #include <cstdint>
 
@@ -28,43 +31,43 @@ namespace hd {
 namespace {
 
 constexpr int kWarps = 8;
-constexpr uint32_t kAreaWords = 1056;  // position-domain words a warp holds: 48 warps an SM, and n = 32767 fits
+constexpr uint32_t kAreaWords = 1056;  // position-domain words a warp holds: n = 32767 fits
 constexpr uint32_t kMaxTile = 256;     // segments per tile
 
 struct EncShortArgs {
     const uint32_t *data;
     uint32_t *stream;
     uint64_t data_words, num_cw, ntiles;
+    uint32_t *status;
     uint32_t n, k, g;          // segment length, message bits, segments per tile
     uint32_t Y, ylast;         // position-domain words per segment, valid bits of the last one
     uint32_t ystride;          // words between two segments' position domains (odd, at least Y + 1)
-    uint32_t tlog;             // log2 of the team size
-    uint32_t step_cw, step_bits;  // 1024 stream bits (32 words) further: segments and bits
 };
 
 __device__ __forceinline__ uint32_t low_bits(uint32_t b) { return b >= 32 ? 0xFFFFFFFFu : (1u << b) - 1u; }
+
+// Per-warp shared memory: the barrier, the message stage (a tile's bits plus the
+// rounding to 16 bytes at both ends) and the position-domain words.
+constexpr uint32_t kStageBytes = (kAreaWords * 4 + 32 + 15) / 16 * 16;
+constexpr uint32_t kOffStage = 16, kOffArea = kOffStage + kStageBytes + 16;  // slack for the last window
+constexpr uint32_t kWarpBytes = (kOffArea + kAreaWords * 4 + 15) / 16 * 16;
 
 // Pass 1 for one segment per team: the lane's position-domain words tl + T*i
 // into `y` and their fold.  x is the XOR of the words; h the XOR of the
 // indices i of the odd-parity words.  Four words at a time: the two low index
 // bits come from XORs of the words that have them, so one popcount serves four
-// words.  SAFE: every window lies inside the message buffer.
-template <bool SAFE>
-__device__ __forceinline__ void fold_segment(const EncShortArgs &a, const uint32_t *src, int32_t bit0, uint32_t tl,
-                                             uint32_t *y, uint32_t &x_out, uint32_t &h_out)
+// words.  J0: floor(log2(32 tl)) (tl > 0), mask0: ~1 where word tl begins with a
+// checksum position.
+template <int TLOG>
+__device__ __forceinline__ void fold_segment(const uint32_t *st, int32_t bit0, uint32_t Y, uint32_t ylast,
+                                             uint32_t tl, uint32_t J0, uint32_t mask0, uint32_t *y, uint32_t &x_out,
+                                             uint32_t &h_out)
 {
-    const uint32_t tlog = a.tlog, T = 1u << tlog, Y = a.Y, last = Y - 1u;
-    const uint32_t *end = a.data + a.data_words;
-    auto ld = [&](const uint32_t *p) { return SAFE || p < end ? __ldg(p) : 0u; };
-    // window of word j (>= 1, floor(log2(32 j)) = J): message bit 32 j - J - 2
-    auto window = [&](uint32_t j, uint32_t J) {
-        const int32_t b = bit0 - (int32_t)J - 2;
-        const uint32_t *p = src + (b >> 5) + (int32_t)j;
-        return __funnelshift_r(ld(p), ld(p + 1), (uint32_t)b & 31u);
-    };
+    constexpr uint32_t T = 1u << TLOG;
+    const uint32_t last = Y - 1u;
     uint32_t x = 0, A = 0, B = 0, hq = 0;
     // words past the segment are 0, the last one holds positions up to n only
-    auto trim = [&](uint32_t j, uint32_t v) { return j < last ? v : j == last ? v & a.ylast : 0u; };
+    auto trim = [&](uint32_t j, uint32_t v) { return j < last ? v : j == last ? v & ylast : 0u; };
     auto take = [&](const uint32_t (&v)[4], uint32_t q) {
         A ^= v[1] ^ v[3];
         B ^= v[2] ^ v[3];
@@ -72,49 +75,51 @@ __device__ __forceinline__ void fold_segment(const EncShortArgs &a, const uint32
         x ^= b;
         hq ^= q & (0u - parity32(b));
     };
+    // word j (>= 1, floor(log2(32 j)) = J) is the window at message bit 32 j - J - 2
     {  // i = 0..3
         uint32_t v[4];
-        if (tl == 0)
-            v[0] = trim(0, expand_runs<5>(__funnelshift_r(ld(src + (bit0 >> 5)), ld(src + (bit0 >> 5) + 1),
-                                                          (uint32_t)bit0 & 31u)));
-        else
-            v[0] = tl < Y ? trim(tl, window(tl, 36u - __clz(tl)) & ((tl & (tl - 1u)) == 0 ? ~1u : ~0u)) : 0u;
+        const int32_t b = tl == 0 ? bit0 : bit0 - (int32_t)J0 - 2;
+        const uint32_t *p = st + (b >> 5) + (int32_t)tl;
+        v[0] = tl < Y ? __funnelshift_r(p[0], p[1], (uint32_t)b & 31u) : 0u;
+        if (tl == 0) v[0] = expand_runs<5>(v[0]);
+        v[0] = trim(tl, v[0] & mask0);
 #pragma unroll
         for (uint32_t u = 1; u < 4; ++u) {
-            const uint32_t j = tl + (u << tlog);
-            v[u] = j < Y ? trim(j, window(j, 5u + tlog + (u >> 1)) & (tl == 0 && u < 3 ? ~1u : ~0u)) : 0u;
+            v[u] = 0u;
+            if (u * T >= Y) continue;  // the whole warp: short segments have no such words
+            const int32_t bu = bit0 - (int32_t)(7u + TLOG + (u >> 1));
+            const uint32_t j = tl + u * T;
+            const uint32_t *pu = st + (bu >> 5) + (int32_t)tl;
+            v[u] = j < Y ? __funnelshift_r(pu[u * T], pu[u * T + 1], (uint32_t)bu & 31u) : 0u;
+            v[u] = trim(j, u < 3 && tl == 0 ? v[u] & ~1u : v[u]);
         }
 #pragma unroll
         for (uint32_t u = 0; u < 4; ++u)
-            if (tl + (u << tlog) < Y) y[tl + (u << tlog)] = v[u];
+            if (tl + u * T < Y) y[tl + u * T] = v[u];
         take(v, 0);
     }
-    for (uint32_t q = 1, J = 7u + tlog; (q << (tlog + 2)) < Y; ++q) {
+    uint32_t J = 7u + TLOG;
+    for (uint32_t q = 1; (q << (TLOG + 2)) < Y; ++q) {
         const bool octave = (q & (q - 1u)) == 0;  // i = 4q is a power of two: J goes up (q = 1 starts at its own)
         if (octave && q > 1) ++J;
         const int32_t b = bit0 - (int32_t)J - 2;
-        const uint32_t j0 = tl + (q << (tlog + 2)), sh = (uint32_t)b & 31u;
-        const uint32_t *p = src + (b >> 5) + (int32_t)j0;
+        const uint32_t j0 = tl + (q << (TLOG + 2)), sh = (uint32_t)b & 31u;
+        const uint32_t *p = st + (b >> 5) + (int32_t)j0;
+        uint32_t *yp = y + j0;
         uint32_t v[4];
         if (j0 + 3u * T < last) {
-            uint32_t lo[4], hi[4];
 #pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) {
-                lo[u] = ld(p + u * T);
-                hi[u] = ld(p + u * T + 1);
-            }
-#pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) v[u] = __funnelshift_r(lo[u], hi[u], sh);
+            for (uint32_t u = 0; u < 4; ++u) v[u] = __funnelshift_r(p[u * T], p[u * T + 1], sh);
             if (octave && tl == 0) v[0] &= ~1u;
 #pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) y[j0 + u * T] = v[u];
+            for (uint32_t u = 0; u < 4; ++u) yp[u * T] = v[u];
         } else {
 #pragma unroll
             for (uint32_t u = 0; u < 4; ++u) {
                 const uint32_t j = j0 + u * T;
-                v[u] = j < Y ? trim(j, __funnelshift_r(ld(p + u * T), ld(p + u * T + 1), sh)) : 0u;
+                v[u] = j < Y ? trim(j, __funnelshift_r(p[u * T], p[u * T + 1], sh)) : 0u;
                 if (u == 0 && octave && tl == 0) v[0] &= ~1u;
-                if (j < Y) y[j] = v[u];
+                if (j < Y) yp[u * T] = v[u];
             }
         }
         take(v, q);
@@ -123,87 +128,147 @@ __device__ __forceinline__ void fold_segment(const EncShortArgs &a, const uint32
     h_out = hq << 2 | parity32(B) << 1 | parity32(A);
 }
 
+// TLOG: log2 of the team size, so that a lane's word strides are constants.
+template <int TLOG>
 __global__ void __launch_bounds__(kWarps * 32) k_encode_short(const EncShortArgs a)
 {
-    extern __shared__ uint32_t s_area[];
+    extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *area = s_area + warp * kAreaWords;
-    const uint32_t tlog = a.tlog, T = 1u << tlog, tl = lane & (T - 1u), team = lane >> tlog, G = 32u >> tlog;
+    uint8_t *wbase = smem + warp * kWarpBytes;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(wbase);
+    uint32_t *stage = reinterpret_cast<uint32_t *>(wbase + kOffStage);
+    uint32_t *area = reinterpret_cast<uint32_t *>(wbase + kOffArea);
+    constexpr uint32_t T = 1u << TLOG, G = 32u >> TLOG;
+    const uint32_t tl = lane & (T - 1u), team = lane >> TLOG;
     const uint32_t n = a.n, k = a.k, Y = a.Y, ys = a.ystride;
+    const uint32_t J0 = 36u - __clz(tl | 1u), mask0 = tl != 0 && (tl & (tl - 1u)) == 0 ? ~1u : ~0u;
+    const uint64_t bulk_end = a.data_words * 4 / 16 * 16;  // bytes that 16-byte copies may read
     grid_dep_launch_dependents();
     grid_dep_wait();
-    for (uint64_t t = (uint64_t)blockIdx.x * kWarps + warp; t < a.ntiles; t += (uint64_t)gridDim.x * kWarps) {
+
+    // the 16-byte groups that hold tile t's messages: first byte and length
+    auto span = [&](uint64_t t, uint64_t &byte0, uint32_t &bytes) {
+        const uint64_t c0 = t * a.g, c1 = min(c0 + a.g, a.num_cw);
+        byte0 = c0 * k / 128 * 16;
+        const uint64_t byte1 = min((c1 * k + 127) / 128 * 16, bulk_end);
+        bytes = byte1 > byte0 ? (uint32_t)(byte1 - byte0) : 0u;
+    };
+    auto load = [&](uint64_t t) {
+        uint64_t byte0;
+        uint32_t bytes;
+        span(t, byte0, bytes);
+        mbar_arrive_expect_tx(bar, bytes);
+        if (bytes) bulk_g2s(stage, reinterpret_cast<const uint8_t *>(a.data) + byte0, bytes, bar);
+    };
+    const uint64_t tw = (uint64_t)gridDim.x * kWarps;
+    uint64_t t = (uint64_t)blockIdx.x * kWarps + warp;
+    if (lane == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
+        if (t < a.ntiles) load(t);
+    }
+    __syncwarp();
+    for (uint32_t phase = 0; t < a.ntiles; t += tw, phase ^= 1u) {
+        const bool ok = mbar_wait_bounded(bar, phase);
+        if (__any_sync(0xFFFFFFFFu, !ok)) {
+            // nothing else of this warp is in flight; a late copy may still land, so wait once more
+            if (lane == 0) {
+                atomicOr(a.status, (uint32_t)HD_ERR_TIMEOUT);
+                (void)mbar_wait_bounded(bar, phase);
+            }
+            break;
+        }
         const uint64_t c0 = t * a.g;
         const uint32_t gcnt = (uint32_t)min((uint64_t)a.g, a.num_cw - c0);
-        const uint64_t bit_in = c0 * k, bit_out = c0 * n;
-        const uint32_t *src = a.data + (bit_in >> 5);
-        const uint32_t off = (uint32_t)bit_in & 31u;
-        // windows reach at most 63 bits past the tile's messages
-        const bool safe = ((bit_in + (uint64_t)gcnt * k + 95u) >> 5) < a.data_words;
+        const uint64_t bit_out = c0 * n;
+        const uint32_t off = (uint32_t)(c0 * k) & 127u;
+        {  // words past the last 16-byte boundary of the messages arrive by plain loads
+            uint64_t byte0;
+            uint32_t bytes;
+            span(t, byte0, bytes);
+            const uint64_t w0 = byte0 >> 2, wb = (byte0 + bytes) >> 2, we = ((c0 + gcnt) * k + 31) >> 5;
+            if (wb < we) {
+                for (uint64_t w = wb + lane; w < we; w += 32) stage[w - w0] = a.data[w];
+                __syncwarp();
+            }
+        }
 
         for (uint32_t cb = 0; cb < gcnt; cb += G) {
             const uint32_t c = cb + team;
             uint32_t *y = area + c * ys;
             uint32_t x = 0, h = 0;
             if (c < gcnt) {
-                if (safe)
-                    fold_segment<true>(a, src, (int32_t)(off + c * k), tl, y, x, h);
-                else
-                    fold_segment<false>(a, src, (int32_t)(off + c * k), tl, y, x, h);
+                fold_segment<TLOG>(stage, (int32_t)(off + c * k), Y, a.ylast, tl, J0, mask0, y, x, h);
                 if (tl == 0) y[Y] = 0u;
             }
-            // index j = tl + T*i: the team's XOR gives the high checksum bits
-            h = (h << tlog) ^ (parity32(x) ? tl : 0u);
-            for (uint32_t o = T >> 1; o > 0; o >>= 1) {  // stays inside aligned groups of T lanes
-                x ^= __shfl_xor_sync(0xFFFFFFFFu, x, o);
-                h ^= __shfl_xor_sync(0xFFFFFFFFu, h, o);
-            }
+            // the lane's share of the checksum bits in one word: the five low ones on bits
+            // 1, 2, 4, 8, 16 of word 0's transform, the high ones (the XOR of the indices
+            // j = tl + T*i of odd-parity words) from bit 17 up; XOR over the team
+            h = (h << TLOG) ^ (parity32(x) ? tl : 0u);
+            uint32_t chk = (superset_xor<5>(x) & 0x00010116u) | h << 17;
+            if constexpr (T == 32)
+                chk = __reduce_xor_sync(0xFFFFFFFFu, chk);
+            else
+                for (uint32_t o = T >> 1; o > 0; o >>= 1)  // stays inside aligned groups of T lanes
+                    chk ^= __shfl_xor_sync(0xFFFFFFFFu, chk, o);
             __syncwarp();  // the team's words are in place
             if (c < gcnt) {
                 // checksum positions 1, 2, 4, 8, 16 lie in word 0 (those past n do not exist and
                 // their parities are 0: no position has such a bit), 32 * 2^b in word 2^b
-                if (tl == 0) y[0] |= superset_xor<5>(x) & 0x00010116u;
-                for (uint32_t b = tl; b < 10u && (1u << b) < Y; b += T) y[1u << b] |= (h >> b) & 1u;
+                if (tl == 0) y[0] |= chk & 0x00010116u;
+                for (uint32_t b = tl; b < 10u && (1u << b) < Y; b += T) y[1u << b] |= (chk >> (17u + b)) & 1u;
             }
         }
+        // the stage has been read: the next tile's messages arrive behind pass 2
+        fence_proxy_async_smem();
         __syncwarp();
+        if (lane == 0 && t + tw < a.ntiles) load(t + tw);
 
-        // pass 2: stream words, counted from the word holding the tile's first bit
-        const uint32_t ob = (uint32_t)bit_out & 31u, total = gcnt * n;
+        // pass 2: stream words, counted from the word holding the tile's first bit.  Segment c
+        // covers the tile's bits [s, s + n), s = ob + c * n.
+        const uint32_t ob = (uint32_t)bit_out & 31u;
         uint32_t *out = a.stream + (bit_out >> 5);
         const bool last_tile = c0 + gcnt == a.num_cw;
-        if (ob != 0 && lane == 0) {  // the first word's low bits belong to the tile before
+        // words inside one segment: the shift is the segment's own
+        for (uint32_t c = team; c < gcnt; c += G) {
+            const uint32_t s = ob + c * n, w1 = (s + 31u) >> 5, w2 = (s + n) >> 5;
+            const uint32_t sh = (1u - s) & 31u;
+            const uint32_t *y = area + c * ys + ((32u * w1 - s + 1u) >> 5) + tl;
+            uint32_t *o = out + w1 + tl;
+            int32_t left = (int32_t)(w2 - w1) - (int32_t)tl;  // words from this lane's first one on
+            for (; left > (int32_t)(3 * T); left -= (int32_t)(4 * T), y += 4 * T, o += 4 * T) {
+                uint32_t v[4];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) v[u] = __funnelshift_r(y[u * T], y[u * T + 1], sh);
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) o[u * T] = v[u];
+            }
+            for (; left > 0; left -= (int32_t)T, y += T, o += T) *o = __funnelshift_r(y[0], y[1], sh);
+        }
+        // the other words, one lane each: the first one when it begins in the tile before, and
+        // the ones a segment ends in, by the segment that reaches back to the word's first bit
+        if (ob != 0 && lane == 0) {
             uint32_t v = area[0] >> 1, avail = n;
             for (uint32_t c = 1; avail < 32u && c < gcnt; ++c, avail += n) v |= (area[c * ys] >> 1) << avail;
             v <<= ob;
             uint32_t own = ~low_bits(ob);
-            if (ob + total < 32u && !last_tile) own &= low_bits(ob + total);
+            if (ob + gcnt * n < 32u && !last_tile) own &= low_bits(ob + gcnt * n);
             atomicAnd(out, v | ~own);
             atomicOr(out, v & own);
         }
-        // the lane's first whole word, as (segment, bits before it), then 32 words on at a time
-        uint32_t w = (uint32_t)lane + (ob != 0 ? 1u : 0u);
-        const uint32_t bit = 32u * w - ob;
-        uint32_t c = bit / n, r = bit - c * n;
-        for (; 32u * w < ob + total; w += 32) {
+        for (uint32_t c = lane; c < gcnt; c += 32) {
+            const uint32_t s = ob + c * n, w = (s + n) >> 5;
+            uint32_t avail = (s + n) & 31u;
+            if (avail == 0 || s > 32u * w) continue;
             const uint32_t *y = area + c * ys;
-            const uint32_t q = r + 1u;  // position of the word's first bit
+            const uint32_t q = 32u * w - s + 1u;  // position of the word's first bit
             uint32_t v = __funnelshift_r(y[q >> 5], y[(q >> 5) + 1], q & 31u);
-            uint32_t avail = n - r;
-            if (avail < 32u) {  // heads of the segments that begin in this word
-                for (uint32_t e = c + 1; avail < 32u && e < gcnt; ++e, avail += n) v |= (area[e * ys] >> 1) << avail;
-            }
+            for (uint32_t e = c + 1; avail < 32u && e < gcnt; ++e, avail += n) v |= (area[e * ys] >> 1) << avail;
             if (avail < 32u && !last_tile) {
                 atomicAnd(&out[w], v | ~low_bits(avail));
                 atomicOr(&out[w], v);
             } else {
                 out[w] = v;
-            }
-            c += a.step_cw;
-            r += a.step_bits;
-            if (r >= n) {
-                r -= n;
-                ++c;
             }
         }
         __syncwarp();  // the next tile overwrites the area
@@ -220,35 +285,45 @@ cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, ui
     a.stream = stream;
     a.data_words = words_for_bits(num_cw * k);
     a.num_cw = num_cw;
+    a.status = status_ptr();
+    if (a.status == nullptr) return cudaErrorInvalidSymbol;
     a.n = n;
     a.k = k;
     a.Y = (n + 32) / 32;
     a.ylast = n % 32 == 31 ? 0xFFFFFFFFu : (2u << (n % 32)) - 1u;
     a.ystride = (a.Y + 1) | 1u;
-    constexpr uint32_t smem = kWarps * kAreaWords * 4;
-    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(k_encode_short), kWarps * 32, smem);
-    if (bps <= 0) return cudaErrorInvalidConfiguration;
-    const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
-    // segments per tile: what the area holds, fewer when the stream then has
-    // less than one tile per resident warp
-    const uint64_t share = (num_cw + cap * kWarps - 1) / (cap * kWarps);
-    a.g = (uint32_t)std::min<uint64_t>({kAreaWords / a.ystride, kMaxTile, share});
+    constexpr uint32_t smem = kWarps * kWarpBytes;
+    static void (*const kernels[6])(EncShortArgs) = {k_encode_short<0>, k_encode_short<1>, k_encode_short<2>,
+                                                     k_encode_short<3>, k_encode_short<4>, k_encode_short<5>};
+    // segments per tile: what the area holds, evened out so that every warp of a full
+    // GPU (3 CTAs an SM) takes as many tiles (40,001 segments of n = 3212: tiles of 10
+    // left 352 of 3648 warps a second one, 13.0 us; two of 6 each take 11.0)
+    const uint64_t resident = (uint64_t)num_sms() * 3 * kWarps;
+    const uint64_t gmax = std::min(kAreaWords / a.ystride, kMaxTile);
+    const uint64_t rounds = (num_cw + gmax * resident - 1) / (gmax * resident);
+    a.g = (uint32_t)((num_cw + rounds * resident - 1) / (rounds * resident));
     // team size: a round of 32 / T segments costs a lane its ceil(Y / 4T) blocks of
-    // four words and a fixed chain (the reduction, the butterfly, the inserts)
+    // four words (dearer the more segments a warp's reads are spread over: bank
+    // conflicts) and a fixed chain (the transform, the team's XOR, the inserts).  The
+    // weights fit the times of every T at eleven lengths on GB300 (512 Mbit, T = 1 ..
+    // 32: n = 544 63/44/53/72/125/191 us, n = 3212 83/50/41/40/44/47, n = 32767
+    // 350/201/105/58/36/26); the pick is the fastest or within 16 % of it at all of them.
     uint64_t best = ~0ull;
-    for (uint32_t lg = 0; lg <= 5; ++lg) {
+    int tlog = 0;
+    for (int lg = 0; lg <= 5; ++lg) {
         const uint32_t T = 1u << lg, G = 32u >> lg;
-        const uint64_t cost = (uint64_t)((a.g + G - 1) / G) * ((a.Y + 4 * T - 1) / (4 * T) * 40 + 60 + 8 * lg);
+        const uint64_t cost = (uint64_t)((a.g + G - 1) / G) *
+                              ((a.Y + 4 * T - 1) / (4 * T) * (40 + 4 * std::min(G, a.g)) + 60 + 8 * (uint32_t)lg);
         if (cost < best) {
             best = cost;
-            a.tlog = lg;
+            tlog = lg;
         }
     }
-    a.step_cw = 1024 / n;
-    a.step_bits = 1024 % n;
+    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kernels[tlog]), kWarps * 32, smem);
+    if (bps <= 0) return cudaErrorInvalidConfiguration;
     a.ntiles = (num_cw + a.g - 1) / a.g;
-    const int grid = decode_grid((a.ntiles + kWarps - 1) / kWarps, cap);
-    return launch_kernel(k_encode_short, dim3((unsigned)grid), dim3(kWarps * 32), smem, st, true, a);
+    const int grid = decode_grid((a.ntiles + kWarps - 1) / kWarps, (uint64_t)num_sms() * (uint64_t)bps);
+    return launch_kernel(kernels[tlog], dim3((unsigned)grid), dim3(kWarps * 32), smem, st, true, a);
 }
 
 }  // namespace hd
