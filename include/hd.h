@@ -71,6 +71,9 @@ typedef enum {
  * Two errors in one codeword give syndrome p XOR q and the decoder flips that
  * third position, as any single-error-correcting Hamming decoder does.
  * num_codewords == 0 is HD_OK; it only zeroes *err_count.
+ * Short streams (up to about 300,000 codewords, fewer for the long codes) are
+ * decoded one codeword per lane, without a configuration, unless one is pinned
+ * with hd_variant_select().
  * For n = 7 and 15 the chosen configuration may decode through a table of
  * 2^n entries (data bits and syndrome per codeword value) kept in static
  * device memory; the first such call on a device fills it with a kernel on
@@ -302,7 +305,7 @@ hd_status hd_variant_info_get(uint32_t n, hd_syn_type syn_type, uint32_t ordinal
  * ordinal < 0 restores the built-in choice. */
 hd_status hd_variant_select(uint32_t n, hd_syn_type syn_type, int32_t ordinal);
 
-/* The configuration hd_decode() uses now for (n, syn_type). */
+/* The configuration hd_decode() uses now for long streams of (n, syn_type). */
 hd_status hd_variant_current(uint32_t n, hd_syn_type syn_type, hd_variant_info *info);
 
 /* Time every configuration of (n, syn_type) on `num_codewords` codewords of

@@ -90,28 +90,11 @@ hd_status check_decode_args(const uint32_t *stream, uint64_t in_bits, uint32_t n
     return HD_OK;
 }
 
-// The decode of one checked stream (num_codewords > 0) on `st`, counters
-// already cleared; pdl: the streaming kernel is the programmatic dependent of
-// the clear just enqueued on `st`.
-hd_status enqueue_decode(const uint32_t *stream, uint64_t in_bits, uint32_t n, uint64_t num_codewords,
-                         uint32_t *out_bits, void *syndromes, hd_syn_type syn_type, unsigned long long *err_count,
-                         cudaStream_t st, bool pdl)
+DecodeJob decode_job(const uint32_t *stream, uint32_t n, uint64_t num_codewords, uint32_t *out_bits, void *syndromes,
+                     hd_syn_type syn_type, unsigned long long *err_count)
 {
-    const uint32_t k = n - (uint32_t)code_m(n);
-    const uint64_t in_words = words_for_bits(in_bits);
-    const uint64_t out_words = words_for_bits(num_codewords * k);
-    const int syn = syndromes ? (int)syn_type : 0;
-    uint64_t covered = 0;
-    if (launch_decode_fast(stream, n, num_codewords, out_bits, syndromes, syn, err_count, st, &covered, pdl) !=
-        cudaSuccess)
-        return HD_ERR_CUDA;
-    if (covered < num_codewords) {
-        const uint64_t tile_begin = covered / 32, tile_end = (num_codewords + 31) / 32;
-        if (launch_decode_generic(stream, in_words, n, num_codewords, tile_begin, tile_end, out_bits, out_words,
-                                  syndromes, syn, err_count, st) != cudaSuccess)
-            return HD_ERR_CUDA;
-    }
-    return HD_OK;
+    return DecodeJob{stream, n, num_codewords, out_bits, syndromes, syndromes ? (int)syn_type : 0, err_count, nullptr,
+                     false};
 }
 
 }  // namespace
@@ -174,11 +157,15 @@ hd_status hd_decode(const uint32_t *stream, uint64_t in_bits, uint32_t n, uint64
         if (err_count && cudaMemsetAsync(err_count, 0, sizeof(*err_count), st) != cudaSuccess) return HD_ERR_CUDA;
         return HD_OK;
     }
+    const DecodeJob j = decode_job(stream, n, num_codewords, out_bits, syndromes, syn_type, err_count);
+    // one CTA's work overwrites the count itself: no clear
+    if (lanes_one_cta(num_codewords) && !variant_pinned(n, j.syn_type))
+        return launch_decode_lanes(j, true, st, true) == cudaSuccess ? HD_OK : HD_ERR_CUDA;
     // the clear and the decode both chained (programmatic dependent launch):
     // the clear may start while the kernel ahead drains and waits for it
     // before writing; the decode waits for the clear before touching memory
     if (err_count && launch_zero_counts(err_count, nullptr, st, true) != cudaSuccess) return HD_ERR_CUDA;
-    return enqueue_decode(stream, in_bits, n, num_codewords, out_bits, syndromes, syn_type, err_count, st, true);
+    return launch_decode(j, st, true) == cudaSuccess ? HD_OK : HD_ERR_CUDA;
 }
 
 hd_status hd_decode_streams(const hd_stream_job *jobs, uint32_t num_jobs, void *cuda_stream)
@@ -227,10 +214,10 @@ hd_status hd_decode_streams(const hd_stream_job *jobs, uint32_t num_jobs, void *
     for (uint32_t r = 0; r < num_jobs; ++r) {
         const hd_stream_job &j = jobs[order[r]];
         if (j.num_codewords == 0) continue;
-        const hd_status rc = enqueue_decode(j.stream, (uint64_t)j.n * j.num_codewords, j.n, j.num_codewords,
-                                            j.out_bits, j.syndromes, static_cast<hd_syn_type>(j.syn_type),
-                                            j.err_count, pool.s[r % kPoolStreams], false);
-        if (rc != HD_OK) return rc;
+        if (launch_decode(decode_job(j.stream, j.n, j.num_codewords, j.out_bits, j.syndromes,
+                                     static_cast<hd_syn_type>(j.syn_type), j.err_count),
+                          pool.s[r % kPoolStreams], false) != cudaSuccess)
+            return HD_ERR_CUDA;
     }
     for (int i = 0; i < used; ++i)
         if (cudaEventRecord(pool.join[i], pool.s[i]) != cudaSuccess ||

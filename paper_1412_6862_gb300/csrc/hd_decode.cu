@@ -6,6 +6,8 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
+#include <tuple>
 #include <vector>
 
 #include "hd_internal.h"
@@ -17,6 +19,7 @@ void register_stream_a(std::vector<StreamVariant> &v);
 void register_stream_b(std::vector<StreamVariant> &v);
 void register_stream_c(std::vector<StreamVariant> &v);
 void register_stream_secded(std::vector<StreamVariant> &v);
+void register_stream_n3(std::vector<StreamVariant> &v);
 
 namespace {
 
@@ -69,6 +72,8 @@ int current_device()
 std::map<std::pair<int, const void *>, int> g_bps;
 // (device, n, syn) -> chosen variant index (autotuner or explicit selection)
 std::map<std::tuple<int, uint32_t, int>, int> g_choice;
+// (device, n, syn) whose choice the caller pinned
+std::set<std::tuple<int, uint32_t, int>> g_pinned;
 // (device, n, syn) -> pinned SECDED configuration (index into secded_variants())
 std::map<std::tuple<int, uint32_t, int>, int> g_secded_choice;
 // device -> address of g_hd_status
@@ -159,65 +164,98 @@ uint32_t read_clear_status_decode()
     return v;
 }
 
-cudaError_t launch_decode_fast(const uint32_t *in, uint32_t n, uint64_t num_cw, uint32_t *out, void *syn,
-                               int syn_type, unsigned long long *err, cudaStream_t st, uint64_t *covered, bool pdl)
+namespace {
+
+// Whole chunks of configuration v, and the ragged tail in the same launch.
+StreamArgs stream_args(const StreamVariant &v, const DecodeJob &j, uint32_t *status, const uint16_t *lut)
 {
-    *covered = 0;
-    const int idx = chosen_variant(n, syn_type);
-    if (idx < 0) return cudaSuccess;
-    const StreamVariant &v = variants()[idx];
-    const uint64_t nchunks = num_cw / v.chunk_cw;
-    if (nchunks == 0) return cudaSuccess;
-    uint32_t *status = status_ptr();
-    if (status == nullptr) return cudaErrorInvalidSymbol;
-    const uint16_t *lut = nullptr;
-    if (v.lut) {
-        lut = lut_ptr(n, st);
-        if (lut == nullptr) return cudaSuccess;  // no table yet (first call inside a capture): generic path
-    }
-    *covered = nchunks * v.chunk_cw;
-    return v.launch(v, in, nchunks, out, syn, err, status, st, nullptr, lut, pdl);
+    const uint64_t nchunks = j.num_cw / v.chunk_cw;
+    return StreamArgs{j.in,    j.out,    j.syn_type != 0 ? j.syn : nullptr,
+                      j.err,   j.det,    status,
+                      lut,     nchunks,  j.num_cw,
+                      words_for_bits(j.num_cw * (j.n + (j.xh ? 1u : 0u))), words_for_bits(j.num_cw * (j.n - (uint32_t)code_m(j.n))),
+                      nchunks * v.chunk_cw / 32, (j.num_cw + 31) / 32};
 }
 
-// SECDED: the streaming kernel with codewords of n + 1 bits, compiled in the
-// built-in configuration of n for each syndrome type.
-cudaError_t launch_decode_fast_secded(const uint32_t *in, uint32_t n, uint64_t num_cw, uint32_t *out, void *syn,
-                                      int syn_type, unsigned long long *err, unsigned long long *det, cudaStream_t st,
-                                      uint64_t *covered, bool pdl)
+// n = 3 (a codeword is three copies of its bit) has one streaming configuration,
+// outside the selectable ones.
+const StreamVariant *variant_n3(int syn)
 {
-    *covered = 0;
+    static const std::vector<StreamVariant> v = [] {
+        std::vector<StreamVariant> a;
+        register_stream_n3(a);
+        return a;
+    }();
+    for (const StreamVariant &x : v)
+        if (x.syn == syn) return &x;
+    return nullptr;
+}
+
+}  // namespace
+
+bool variant_pinned(uint32_t n, int syn)
+{
+    std::lock_guard<std::mutex> lk(g_mu);
+    return g_pinned.count({current_device(), n, syn}) != 0;
+}
+
+bool secded_variant_pinned(uint32_t n, int syn)
+{
+    std::lock_guard<std::mutex> lk(g_mu);
+    return g_secded_choice.count({current_device(), n, syn}) != 0;
+}
+
+cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl)
+{
+    if (!variant_pinned(j.n, j.syn_type) && lanes_suffice(j.n, j.xh, j.num_cw)) return launch_decode_lanes(j, false, st, pdl);
+    const StreamVariant *v = nullptr;
+    if (j.n == 3) {
+        v = variant_n3(j.syn_type);
+    } else {
+        const int idx = chosen_variant(j.n, j.syn_type);
+        if (idx >= 0) v = &variants()[idx];
+    }
+    const uint16_t *lut = v != nullptr && v->lut ? lut_ptr(j.n, st) : nullptr;
+    // no whole chunk, or no table yet (first call inside a capture)
+    if (v == nullptr || j.num_cw < v->chunk_cw || (v->lut && lut == nullptr)) return launch_decode_lanes(j, false, st, pdl);
+    uint32_t *status = status_ptr();
+    if (status == nullptr) return cudaErrorInvalidSymbol;
+    return v->launch(stream_args(*v, j, status, lut), st, pdl);
+}
+
+// SECDED: the streaming kernel with codewords of n + 1 bits.
+cudaError_t launch_decode_secded(const DecodeJob &j, cudaStream_t st, bool pdl)
+{
+    int pinned = -1;
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        auto it = g_secded_choice.find({current_device(), j.n, j.syn_type});
+        if (it != g_secded_choice.end()) pinned = it->second;
+    }
+    if (pinned < 0 && lanes_suffice(j.n, j.xh, j.num_cw)) return launch_decode_lanes(j, false, st, pdl);
     // a pinned configuration (hd_secded_variant_select), else the table
     // configuration when its table is filled (not while `st` captures before
     // the first fill), else the arithmetic one
     const StreamVariant *v = nullptr, *vt = nullptr;
     for (const StreamVariant &x : secded_variants())
-        if (x.n == n && x.syn == syn_type) {
+        if (x.n == j.n && x.syn == j.syn_type) {
             if (!x.lut) {
                 if (v == nullptr) v = &x;
             } else if (vt == nullptr) {
                 vt = &x;
             }
         }
-    int pinned = -1;
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        auto it = g_secded_choice.find({current_device(), n, syn_type});
-        if (it != g_secded_choice.end()) pinned = it->second;
-    }
     if (pinned >= 0) {
         const StreamVariant &x = secded_variants()[pinned];
         if (x.lut) vt = &x;
         else v = &x, vt = nullptr;
     }
-    const uint16_t *lut = vt != nullptr ? lut_ptr(n, st, true) : nullptr;
+    const uint16_t *lut = vt != nullptr ? lut_ptr(j.n, st, true) : nullptr;
     if (lut != nullptr) v = vt;
-    if (v == nullptr) return cudaSuccess;
-    const uint64_t nchunks = num_cw / v->chunk_cw;
-    if (nchunks == 0) return cudaSuccess;
+    if (v == nullptr || j.num_cw < v->chunk_cw) return launch_decode_lanes(j, false, st, pdl);
     uint32_t *status = status_ptr();
     if (status == nullptr) return cudaErrorInvalidSymbol;
-    *covered = nchunks * v->chunk_cw;
-    return v->launch(*v, in, nchunks, out, syn, err, status, st, det, v->lut ? lut : nullptr, pdl);
+    return v->launch(stream_args(*v, j, status, v->lut ? lut : nullptr), st, pdl);
 }
 
 // ---------------------------------------------------------------------------
@@ -284,6 +322,7 @@ hd_status hd_variant_select(uint32_t n, hd_syn_type syn_type, int32_t ordinal)
     std::lock_guard<std::mutex> lk(g_mu);
     if (ordinal < 0) {
         g_choice.erase({dev, n, (int)syn_type});
+        g_pinned.erase({dev, n, (int)syn_type});
         return HD_OK;
     }
     int32_t c = 0;
@@ -292,6 +331,7 @@ hd_status hd_variant_select(uint32_t n, hd_syn_type syn_type, int32_t ordinal)
         if (v[i].n == n && v[i].syn == (int)syn_type) {
             if (c == ordinal) {
                 g_choice[{dev, n, (int)syn_type}] = (int)i;
+                g_pinned.insert({dev, n, (int)syn_type});
                 return HD_OK;
             }
             ++c;
@@ -427,6 +467,18 @@ hd_status hd_autotune(uint32_t n, hd_syn_type syn_type, uint64_t num_codewords, 
     std::vector<Cand> cands;
     const auto &vs = variants();
     auto *er = static_cast<unsigned long long *>(derr);
+    // the whole chunks of buffer set i (no tail: the chunked prefix differs per configuration)
+    auto set_args = [&](const StreamVariant &v, int i, const uint16_t *lut) {
+        DecodeJob j{};
+        j.in = static_cast<const uint32_t *>(din[i]);
+        j.n = n;
+        j.num_cw = num_codewords / v.chunk_cw * v.chunk_cw;
+        j.out = static_cast<uint32_t *>(dout[i]);
+        j.syn = dsyn[i];
+        j.syn_type = (int)syn_type;
+        j.err = er;
+        return stream_args(v, j, status, lut);
+    };
     for (size_t i = 0; rc == HD_OK && i < vs.size(); ++i) {
         const StreamVariant &v = vs[i];
         if (v.n != n || v.syn != (int)syn_type) continue;
@@ -435,8 +487,7 @@ hd_status hd_autotune(uint32_t n, hd_syn_type syn_type, uint64_t num_codewords, 
         if (stream_blocks_per_sm(v.kernel, v.T, v.smem) <= 0) continue;
         const uint16_t *lut = v.lut ? lut_ptr(n, st) : nullptr;
         if (v.lut && lut == nullptr) continue;
-        if (v.launch(v, static_cast<const uint32_t *>(din[0]), nchunks, static_cast<uint32_t *>(dout[0]),
-                     syn_type == HD_SYN_NONE ? nullptr : dsyn[0], er, status, st, nullptr, lut, false) != cudaSuccess) {
+        if (v.launch(set_args(v, 0, lut), st, false) != cudaSuccess) {
             rc = HD_ERR_CUDA;
             break;
         }
@@ -449,8 +500,7 @@ hd_status hd_autotune(uint32_t n, hd_syn_type syn_type, uint64_t num_codewords, 
             const StreamVariant &v = vs[c.idx];
             cudaEventRecord(e0, st);
             for (int i = 0; i < nsets; ++i)
-                v.launch(v, static_cast<const uint32_t *>(din[i]), c.nchunks, static_cast<uint32_t *>(dout[i]),
-                         syn_type == HD_SYN_NONE ? nullptr : dsyn[i], er, status, st, nullptr, c.lut, false);
+                v.launch(set_args(v, i, c.lut), st, false);
             cudaEventRecord(e1, st);
             if (cudaEventSynchronize(e1) != cudaSuccess) {
                 rc = HD_ERR_CUDA;
@@ -494,6 +544,7 @@ hd_status hd_autotune(uint32_t n, hd_syn_type syn_type, uint64_t num_codewords, 
     {
         std::lock_guard<std::mutex> lk(g_mu);
         g_choice[{current_device(), n, (int)syn_type}] = best;
+        g_pinned.erase({current_device(), n, (int)syn_type});
     }
     if (chosen) {
         hd_variant_current(n, syn_type, chosen);

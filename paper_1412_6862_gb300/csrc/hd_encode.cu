@@ -185,12 +185,15 @@ cudaError_t launch_encode_stream(EncArgs a, cudaStream_t st)
 {
     using Cfg = EncCfg<N_, T, S, G, CH>;
     a.tile_end = (a.num_cw + 31) / 32;
-    const uint64_t lane_cap = (uint64_t)num_sms() * (64 / kLaneWarps);
-    // One round of tiles, at most: on GB300 (152 SMs: 311,296 codewords) the two
-    // paths cross there.  n = 31, lanes against chunks: 1.4 against 2.9 us at
+    const int lane_bps =
+        stream_blocks_per_sm(reinterpret_cast<const void *>(k_encode_lanes<N_>), kLaneWarps * 32, 0);
+    const uint64_t lane_cap = (uint64_t)num_sms() * (uint64_t)std::max(lane_bps, 1);
+    // At most one round of tiles on the CTAs the device holds at once (152 SMs:
+    // 311,296 codewords, fewer for the long codes' wider kernels): the two paths cross
+    // about there on GB300.  n = 31, lanes against chunks: 1.4 against 2.9 us at
     // 20,000 codewords, 2.6 against 3.1 at 300,000, 3.9 against 3.3 at 600,000;
-    // n = 127: 3.8 against 3.6 at 300,000; n = 7: 3.6 against 3.2.
-    if (a.tile_end <= lane_cap * kLaneWarps) {
+    // n = 255: 2.8 against 3.6 at 100,000, 4.8 against 4.4 at 200,000.
+    if (a.tile_end <= (uint64_t)decode_grid(lane_cap, lane_cap) * kLaneWarps) {
         const int grid = decode_grid((a.tile_end + kLaneWarps - 1) / kLaneWarps, lane_cap);
         return launch_kernel(k_encode_lanes<N_>, dim3((unsigned)grid), dim3(kLaneWarps * 32), 0, st, true, a);
     }

@@ -41,11 +41,26 @@ inline int decode_grid(uint64_t want, uint64_t cap)
     return (int)(g > 0 ? g : 1);
 }
 
-// Generic warp-tile kernels (any supported n).  Warp tile t covers codewords
-// [32t, 32t+32); the launch covers warp tiles [tile_begin, tile_end).
-cudaError_t launch_decode_generic(const uint32_t *in, uint64_t in_words, uint32_t n, uint64_t num_cw,
-                                  uint64_t tile_begin, uint64_t tile_end, uint32_t *out, uint64_t out_words,
-                                  void *syn, int syn_type, unsigned long long *err, cudaStream_t st);
+// One stream to decode: plain code of length n, or with xh its SECDED extension
+// (codewords of n + 1 bits).  syn_type 0 stores no syndromes; err / det may be null.
+struct DecodeJob {
+    const uint32_t *in;
+    uint32_t n;
+    uint64_t num_cw;
+    uint32_t *out;
+    void *syn;
+    int syn_type;
+    unsigned long long *err, *det;
+    bool xh;
+};
+
+// The one-codeword-per-lane decoder, for any stream length.  direct: the whole
+// stream is one CTA's work (lanes_one_cta) and *err / *det are overwritten, so
+// that nothing needs clearing ahead; else they are added to.
+cudaError_t launch_decode_lanes(const DecodeJob &j, bool direct, cudaStream_t st, bool pdl);
+bool lanes_one_cta(uint64_t num_cw);
+// Whether a stream is short enough that one codeword per lane beats whole chunks.
+bool lanes_suffice(uint32_t n, bool xh, uint64_t num_cw);
 
 // The encoders (any supported n, any length): data_words / stream_words are the
 // buffers' lengths; launched as programmatic dependents of the kernel ahead.
@@ -102,19 +117,16 @@ cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
 // first global access.
 cudaError_t launch_zero_counts(unsigned long long *a, unsigned long long *b, cudaStream_t st, bool chained = false);
 
-// Specialised streaming decoder.  Decodes the longest prefix of whole chunks
-// it supports and returns the number of codewords covered in *covered (0 when
-// n has no specialised kernel).  pdl: launched as the programmatic dependent
-// of a launch_zero_counts() just enqueued on `st`.
-cudaError_t launch_decode_fast(const uint32_t *in, uint32_t n, uint64_t num_cw, uint32_t *out, void *syn,
-                               int syn_type, unsigned long long *err, cudaStream_t st, uint64_t *covered,
-                               bool pdl = false);
+// Decode a stream (num_cw > 0) on `st` in one launch: the streaming kernel with
+// its ragged tail, or one codeword per lane.  The counters are added to.  pdl:
+// launched as the programmatic dependent of the kernel ahead.
+cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl);
+cudaError_t launch_decode_secded(const DecodeJob &j, cudaStream_t st, bool pdl);
 
-// The SECDED streaming decoder (codewords of n + 1 bits): whole chunks, as
-// launch_decode_fast; `det` (or nullptr) receives the detected double errors.
-cudaError_t launch_decode_fast_secded(const uint32_t *in, uint32_t n, uint64_t num_cw, uint32_t *out, void *syn,
-                                      int syn_type, unsigned long long *err, unsigned long long *det, cudaStream_t st,
-                                      uint64_t *covered, bool pdl = false);
+// Whether the caller pinned a configuration (hd_variant_select, not the
+// autotuner's pick; hd_secded_variant_select): short streams take it too.
+bool variant_pinned(uint32_t n, int syn);
+bool secded_variant_pinned(uint32_t n, int syn);
 
 // Decode table of n = 7 or 15 (data | s << k per codeword; with xh the SECDED
 // table of n + 1 bits, data | s << k | P << (k + m)), filled on `st` on first

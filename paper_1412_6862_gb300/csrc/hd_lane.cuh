@@ -264,4 +264,89 @@ __device__ __forceinline__ void encode_lane_tile(const uint32_t *__restrict__ da
     __syncwarp();
 }
 
+// Decode tile t (codewords 32t .. 32t + 31, those below num_cw) of the plain
+// code, or with XH of its SECDED extension (decode_part's conventions):
+// `slots` holds 32 * lane_slot_words(ceil(k / 32)) words of this warp's shared
+// memory.  syn_type 0 (none), 1 (u8) or 2 (u16); the nonzero and detected
+// syndromes of the tile are added to errs and dets (the same in every lane).
+// Every lane of the warp calls it.
+template <int N_>
+constexpr int kLaneDataSlot = lane_slot_words((Code<N_>::k + 31) / 32);
+
+template <int N_, bool XH>
+__device__ __forceinline__ void decode_lane_tile(const uint32_t *__restrict__ in, uint64_t in_words, uint64_t num_cw,
+                                                 uint64_t t, uint32_t *__restrict__ out, uint64_t out_words,
+                                                 void *__restrict__ syn, int syn_type, uint32_t *slots, int lane,
+                                                 uint32_t &errs, uint32_t &dets)
+{
+    using C = Code<N_>;
+    constexpr int L = N_ + (XH ? 1 : 0), D = (C::k + 31) / 32, SLOT = kLaneDataSlot<N_>;
+    const uint32_t *src = in + t * L;
+    const uint32_t have = (uint32_t)min((uint64_t)L, in_words - t * L);  // words of the tile
+    const uint64_t i = t * 32 + lane;
+    const bool valid = i < num_cw;
+    // position p is tile bit lane * L + p (XH), lane * L + p - 1 (lane 0's position 0 would be word -1)
+    const int32_t bit = lane * L - (XH ? 0 : 1), a = bit >> 5;
+    const uint32_t sh = (uint32_t)bit & 31u;
+    uint32_t y[C::Wy];
+    auto word = [&](int32_t w) { return valid && (uint32_t)w < have ? src[w] : 0u; };
+    uint32_t lo = word(a);
+#pragma unroll
+    for (int w = 0; w < C::Wy; ++w) {
+        // SECDED codewords never straddle a word
+        const uint32_t hi = XH ? (w + 1 < C::Wy ? word(a + w + 1) : 0u) : word(a + w + 1);
+        y[w] = XH && L >= 32 ? lo : __funnelshift_r(lo, hi, sh);
+        lo = hi;
+    }
+    if constexpr (!XH) y[0] &= ~1u;
+    if constexpr (N_ < 31) y[0] &= (2u << N_) - 1u;
+    const uint32_t s = part_syndrome<N_>(y);
+    uint32_t sf = s, val = s;
+    bool nonzero = s != 0u;
+    if constexpr (XH) {
+        uint32_t f = 0;
+#pragma unroll
+        for (int w = 0; w < C::Wy; ++w) f ^= y[w];
+        const uint32_t P = parity32(f);
+        sf = P ? s : 0xFFFFFFFFu;
+        val = s | P << C::m;
+        nonzero = val != 0u;
+        dets += __popc(__ballot_sync(0xFFFFFFFFu, valid && P == 0u && s != 0u));
+    }
+    errs += __popc(__ballot_sync(0xFFFFFFFFu, valid && nonzero));
+    if (valid) {
+        if (syn_type == 1) static_cast<uint8_t *>(syn)[i] = (uint8_t)val;
+        if (syn_type == 2) static_cast<uint16_t *>(syn)[i] = (uint16_t)val;
+    }
+#pragma unroll
+    for (int w = 0; w < C::Wy; ++w) y[w] ^= shl_clamp(1u, sf - 32u * (uint32_t)w);
+    if constexpr (N_ == 3) {
+        const uint32_t v = __ballot_sync(0xFFFFFFFFu, (y[0] >> 3) & 1u);  // one data bit each: the tile's word
+        if (lane == 0) out[t] = v;
+    } else {
+        // the data bits, packed: 26, then 31 or 32 per word
+        uint32_t d[D];
+        d[0] = compress_runs<(C::m < 5 ? C::m : 5)>(y[0]);
+        if constexpr (C::m < 5) d[0] &= (1u << C::k) - 1u;
+        int at = 26;
+#pragma unroll
+        for (int w = 1; w < C::Wy; ++w) {
+            const bool chk = (w & (w - 1)) == 0;  // position 32w is a checksum position
+            const uint32_t v = chk ? y[w] >> 1 : y[w];
+            d[at / 32] |= v << (at % 32);
+            const int end = at + (chk ? 31 : 32);
+            if (end > (at / 32 + 1) * 32 || (end == (at / 32 + 1) * 32 && at / 32 + 1 < D))
+                d[at / 32 + 1] = at % 32 == 0 ? 0u : v >> (32 - at % 32);
+            at = end;
+        }
+        uint32_t *mine = slots + lane * SLOT;
+#pragma unroll
+        for (int w = 0; w < D; ++w) mine[w] = d[w];
+        mine[D] = 0u;
+        __syncwarp();
+        merge_tile<C::k, SLOT>(slots, 0, out + t * C::k, (uint32_t)min((uint64_t)C::k, out_words - t * C::k), lane);
+        __syncwarp();
+    }
+}
+
 }  // namespace hd

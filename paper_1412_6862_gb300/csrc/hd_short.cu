@@ -22,7 +22,7 @@
 //    first 26 data bits or cross into the next codeword, per codeword.  (5) For
 //    long codewords, the few words that hold a checksum position.
 //  * k_short_small (n <= 255): warp tiles of 32 codewords straight from global
-//    memory, one codeword per lane, like the generic full-length kernel.
+//    memory, one codeword per lane.
 // The encoder is in hd_short_encode.cu.
 #include <algorithm>
 #include <cstdint>

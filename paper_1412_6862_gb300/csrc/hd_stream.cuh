@@ -20,9 +20,24 @@
 
 #include "hd_device.cuh"
 #include "hd_internal.h"
+#include "hd_lane.cuh"
 #include "hd_tile.cuh"
 
 namespace hd {
+
+// One decode: whole chunks [0, nchunks) of the stream, and the 32-codeword
+// tiles [tile_begin, tile_end) of its ragged tail.
+struct StreamArgs {
+    const uint32_t *in;
+    uint32_t *out;
+    void *syn;
+    unsigned long long *err, *det;
+    uint32_t *status;
+    const uint16_t *lut;
+    uint64_t nchunks;
+    uint64_t num_cw, in_words, out_words;
+    uint64_t tile_begin, tile_end;
+};
 
 // One compiled configuration of the streaming decoder.
 struct StreamVariant {
@@ -34,9 +49,7 @@ struct StreamVariant {
     int inplace;  // output written into the input stage
     uint32_t smem;
     uint64_t chunk_cw;  // codewords per warp iteration (32*G)
-    cudaError_t (*launch)(const StreamVariant &v, const uint32_t *in, uint64_t nchunks, uint32_t *out, void *syn,
-                          unsigned long long *err, uint32_t *status, cudaStream_t st, unsigned long long *det,
-                          const uint16_t *lut, bool pdl);
+    cudaError_t (*launch)(const StreamArgs &a, cudaStream_t st, bool pdl);
     const void *kernel;
     int xh = 0;   // SECDED: codewords of n + 1 bits with the overall parity bit at position 0
     int lut = 0;  // decode table (n = 7, 15): one shared-memory lookup per codeword
@@ -180,13 +193,40 @@ __device__ __forceinline__ void issue_chunk(const uint32_t *in, uint64_t c, uint
     }
 }
 
+// The ragged tail's tiles t0, t0 + step, ... of a stream; returns the nonzero
+// syndromes | detected ones << 16 (a tail has at most 1024 codewords).  Out of line
+// from n = 63 up: the kernel's loop then keeps the registers it has without a tail
+// (SECDED n = 63, 2^24 codewords: 50.0 us against 51.9 inline; n = 127: 26.7 against
+// 27.4); the short codes' loops are better with it inline (n = 31, 20,000,003
+// codewords: 33.5 us against 34.5).
+template <int N_, int SYN, bool XH>
+__device__ __forceinline__ uint32_t tail_tiles(const uint32_t *in, uint64_t in_words, uint64_t num_cw, uint64_t t0,
+                                               uint64_t t1, uint64_t step, uint32_t *out, uint64_t out_words,
+                                               void *syn, uint32_t *slots, int lane)
+{
+    uint32_t te = 0, td = 0;
+    for (uint64_t t = t0; t < t1; t += step)
+        decode_lane_tile<N_, XH>(in, in_words, num_cw, t, out, out_words, syn, SYN, slots, lane, te, td);
+    return te | td << 16;
+}
+
+template <int N_, int SYN, bool XH>
+__device__ __noinline__ uint32_t tail_tiles_call(const uint32_t *in, uint64_t in_words, uint64_t num_cw, uint64_t t0,
+                                                 uint64_t t1, uint64_t step, uint32_t *out, uint64_t out_words,
+                                                 void *syn, uint32_t *slots, int lane)
+{
+    return tail_tiles<N_, SYN, XH>(in, in_words, num_cw, t0, t1, step, out, out_words, syn, slots, lane);
+}
+
 template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH = false, bool LUT = false>
 __global__ void __launch_bounds__(T)
-    k_decode_stream(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, uint8_t *__restrict__ syn,
-                    unsigned long long *__restrict__ err, uint32_t *__restrict__ status, uint64_t nchunks,
-                    unsigned long long *__restrict__ det, const uint16_t *__restrict__ lut)
+    k_decode_stream(const StreamArgs args)
 {
     using Cfg = StreamCfg<N_, SYN, T, S, G, INPLACE, XH, LUT>;
+    const uint32_t *__restrict__ in = args.in;
+    uint32_t *__restrict__ out = args.out;
+    uint8_t *__restrict__ syn = static_cast<uint8_t *>(args.syn);
+    const uint64_t nchunks = args.nchunks;
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // Programmatic dependent launch, both ways: the next kernel of the stream
@@ -209,7 +249,7 @@ __global__ void __launch_bounds__(T)
             static_assert(Cfg::lut_bytes % piece == 0, "whole pieces");
 #pragma unroll
             for (uint32_t o = 0; o < Cfg::lut_bytes; o += piece)
-                bulk_g2s(smem + Cfg::off_lut + o, reinterpret_cast<const uint8_t *>(lut) + o, piece, lut_bar);
+                bulk_g2s(smem + Cfg::off_lut + o, reinterpret_cast<const uint8_t *>(args.lut) + o, piece, lut_bar);
         }
         __syncthreads();  // the barrier is initialised before any thread waits on it
     }
@@ -220,6 +260,29 @@ __global__ void __launch_bounds__(T)
     const uint64_t gw = (uint64_t)blockIdx.x * Cfg::WARPS + warp;  // global warp index
     const uint64_t tw = (uint64_t)gridDim.x * Cfg::WARPS;          // warps in the grid
     grid_dep_wait();  // the kernels ahead (the counters' clear, and what produced the input) have finished
+
+    uint32_t errs = 0, dets = 0;  // this lane's counts
+    // The ragged tail's tiles, one codeword per lane, by the grid's last warps (which
+    // hold the fewest chunks) before their first chunk: a launch of its own for them
+    // cost 4 to 5 us, the GPU drained on both sides of it.
+    if (args.tile_begin < args.tile_end) {
+        static_assert(Cfg::warp_bytes - Cfg::off_in >= 32u * kLaneDataSlot<N_> * 4u, "a tile's merge area");
+        const uint64_t t0 = args.tile_begin + (tw - 1 - gw);
+        uint32_t *slots = reinterpret_cast<uint32_t *>(s_in);
+        uint32_t c;
+        if constexpr (N_ >= 63)
+            c = tail_tiles_call<N_, SYN, XH>(in, args.in_words, args.num_cw, t0, args.tile_end, tw, out,
+                                             args.out_words, syn, slots, lane);
+        else
+            c = tail_tiles<N_, SYN, XH>(in, args.in_words, args.num_cw, t0, args.tile_end, tw, out, args.out_words,
+                                        syn, slots, lane);
+        if (lane == 0) {
+            errs = c & 0xFFFFu;
+            dets = c >> 16;
+        }
+        fence_proxy_async_smem();  // the tiles used the ring that the copies below fill
+        __syncwarp();
+    }
 
     if constexpr (!Cfg::PADDED) {
         if (lane == 0) {
@@ -250,7 +313,6 @@ __global__ void __launch_bounds__(T)
     }
     __syncwarp();
 
-    uint32_t errs = 0, dets = 0;
     uint32_t it = 0;
     bool aborted = false;
     const uint16_t *s_lut = nullptr;
@@ -329,7 +391,7 @@ __global__ void __launch_bounds__(T)
     }
     if (lane == 0) {
         if (aborted) {
-            atomicOr(status, (uint32_t)HD_ERR_TIMEOUT);
+            atomicOr(args.status, (uint32_t)HD_ERR_TIMEOUT);
             // wait (bounded) for every load still in flight into this warp's ring
             // (after the first iteration in-place refills lag one iteration, so
             // one fewer is outstanding) and for the table
@@ -349,38 +411,26 @@ __global__ void __launch_bounds__(T)
         for (int o = 16; o > 0; o >>= 1) dets += __shfl_xor_sync(0xFFFFFFFFu, dets, o);
     }
     if (lane == 0) {
-        if (err != nullptr && errs != 0) atomicAdd(err, (unsigned long long)errs);
-        if (XH && det != nullptr && dets != 0) atomicAdd(det, (unsigned long long)dets);
+        if (args.err != nullptr && errs != 0) atomicAdd(args.err, (unsigned long long)errs);
+        if (XH && args.det != nullptr && dets != 0) atomicAdd(args.det, (unsigned long long)dets);
     }
 }
 
-template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH = false, bool LUT = false>
-cudaError_t launch_stream_variant(const StreamVariant &v, const uint32_t *in, uint64_t nchunks, uint32_t *out,
-                                  void *syn, unsigned long long *err, uint32_t *status, cudaStream_t st,
-                                  unsigned long long *det, const uint16_t *lut, bool pdl);
-
-// Per-device configuration of a kernel (dynamic shared memory opt-in and the
-// number of resident CTAs per SM).
-int stream_blocks_per_sm(const void *kernel, int threads, uint32_t smem);
-
 template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH, bool LUT>
-cudaError_t launch_stream_variant(const StreamVariant &v, const uint32_t *in, uint64_t nchunks, uint32_t *out,
-                                  void *syn, unsigned long long *err, uint32_t *status, cudaStream_t st,
-                                  unsigned long long *det, const uint16_t *lut, bool pdl)
+cudaError_t launch_stream_variant(const StreamArgs &a, cudaStream_t st, bool pdl)
 {
     using Cfg = StreamCfg<N_, SYN, T, S, G, INPLACE, XH, LUT>;
-    if (LUT && lut == nullptr) return cudaErrorInvalidValue;
+    if (LUT && a.lut == nullptr) return cudaErrorInvalidValue;
     auto kern = k_decode_stream<N_, SYN, T, S, G, INPLACE, XH, LUT>;
     const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kern), T, Cfg::smem);
     if (bps <= 0) return cudaErrorInvalidConfiguration;
     const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
-    const uint64_t want = (nchunks + Cfg::WARPS - 1) / Cfg::WARPS;
+    const uint64_t want = (a.nchunks + Cfg::WARPS - 1) / Cfg::WARPS;
     const int grid = decode_grid(want, cap);
     // with pdl the launch may overlap the kernel ahead of it (the counters'
     // clear, or a decode's drain); the kernel waits for it before its first
     // access to global memory
-    return launch_kernel(kern, dim3((unsigned)grid), dim3(T), Cfg::smem, st, pdl, in, out,
-                         static_cast<uint8_t *>(syn), err, status, nchunks, det, lut);
+    return launch_kernel(kern, dim3((unsigned)grid), dim3(T), Cfg::smem, st, pdl, a);
 }
 
 template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH = false, bool LUT = false>

@@ -33,4 +33,7 @@ void register_stream_secded(std::vector<StreamVariant> &v)
     add_variants<15, 384, 2, 32, 1, true, true>(v);
 }
 
+// The plain n = 3 code (see hd_decode.cu).
+void register_stream_n3(std::vector<StreamVariant> &v) { add_variants<3, 128, 4, 32, 1>(v); }
+
 }  // namespace hd

@@ -57,7 +57,7 @@ def test_lane_path_edges(n, secded):
 @pytest.mark.parametrize("cap", [0, 6])
 @pytest.mark.parametrize("n", ALL_N)
 def test_streaming_path_and_tail(n, cap):
-    for N in (311_296, 311_297, 327_680, 327_680 + 1021):  # 311,296: the last one-codeword-per-lane size on 152 SMs
+    for N in (116_736, 194_560, 311_296, 311_297, 327_680 + 1021):  # the lane path's last sizes, chunks with a tail
         _check(n, N, False, cap)
 
 
