@@ -197,8 +197,10 @@ hd_status hd_decode_short(const uint32_t *stream, uint64_t in_bits, uint32_t n, 
 hd_status hd_encode_short(const uint32_t *data_bits, uint32_t n, uint64_t num_codewords, uint32_t *stream,
                           void *cuda_stream);
 
-/* Segments with k >= 64 are decoded by a tiled kernel that reads a per-length
- * output-word table (about 2 * (k + 2200) bytes of device memory).
+/* Segments of n < 960 are decoded one per lane (unless a tile configuration is
+ * chosen for them, see below), longer ones by a tiled kernel that reads a
+ * per-length output-word table (about 2 * (k + 2200) bytes of device memory).
+ * Every length with k >= 64 has a table, so that either kernel can run.
  * hd_decode_short() keeps these tables in a per-device cache: the first call
  * for a length n builds its table (cudaMalloc plus a synchronous copy); up to
  * 32 lengths are kept per device, and evicting the least recently used one
@@ -233,7 +235,8 @@ void hd_short_plan_destroy(hd_short_plan *plan);
  * every configuration on `num_codewords` all-zero segments of length n (reps
  * launches each, 0 = 5; it allocates its own scratch buffers and synchronises
  * `cuda_stream`) and keeps the fastest for n on the current device, returned
- * in *chosen (-1 when n has a single kernel, k < 64).  A configuration never
+ * in *chosen (-1 when n has a single kernel, k < 64); below n = 960 it is kept
+ * only if it also beats decoding one segment per lane.  A configuration never
  * changes the result, only the speed. */
 hd_status hd_short_variant_count(uint32_t *count);
 hd_status hd_short_variant_select(int32_t ordinal);

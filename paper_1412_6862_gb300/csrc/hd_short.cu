@@ -10,18 +10,17 @@
 // left as received.
 //
 // Two decoders:
-//  * k_short_tiles (k >= 64, i.e. n >= 71): each warp streams tiles of g whole
+//  * k_short_tiles (n >= 960; any k >= 64 where a configuration is chosen): each warp streams tiles of g whole
 //    codewords through a ring of shared-memory stages filled by 1-D bulk
 //    copies.  Per tile: (1) syndromes, teams of T lanes per codeword (T from a
-//    cost model, 1..32), each lane folding its position-domain words into an
-//    XOR and a parity mask, then a butterfly over the team; the corrections
-//    flip bits in the stage.  (3) Every output word from a per-length table of
+//    cost model, 1..32), each lane folding its position-domain words four at a
+//    time, then one XOR over the team; the corrections flip bits in the stage.  (3) Every output word from a per-length table of
 //    output-word offsets: a funnel shift (and, for short codewords, a merge at
 //    the word's checksum position), lane-strided so stage reads are
 //    conflict-free and stores coalesced.  (4) The words that hold a codeword's
 //    first 26 data bits or cross into the next codeword, per codeword.  (5) For
 //    long codewords, the few words that hold a checksum position.
-//  * k_short_small (n <= 255): warp tiles of 32 codewords straight from global
+//  * k_short_small (below): warp tiles of 32 codewords straight from global
 //    memory, one codeword per lane.
 // The encoder is in hd_short_encode.cu.
 #include <algorithm>
@@ -29,17 +28,22 @@
 #include <mutex>
 #include <new>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "hd_device.cuh"
-#include "hd_generic.cuh"
 #include "hd_internal.h"
+#include "hd_lane.cuh"
 
 namespace hd {
 namespace {
 
 constexpr uint32_t kShortMaxN = 32767;  // r <= 15: syndromes fit 16 bits
 constexpr uint32_t kLongMinK = 64;      // k_short_tiles needs the first 58 data bits inside one codeword
+// Lengths below it are decoded one codeword per lane.  On GB300, 1 Gbit with u16
+// syndromes, lanes against tiles: n = 100 90/145 us, 250 54/91, 400 54/86, 544 57/75,
+// 650 63/71, 810 64/72, 900 70/79, 1000 76/64; 100,000 bits of n = 544 3.0/4.8.
+constexpr uint32_t kLaneMaxN = 960;
 
 __host__ __device__ inline uint32_t short_r(uint32_t n)
 {
@@ -49,15 +53,6 @@ __host__ __device__ inline uint32_t short_r(uint32_t n)
 }
 
 __device__ __forceinline__ uint32_t lowmask(uint32_t b) { return b >= 32 ? 0xFFFFFFFFu : (1u << b) - 1u; }
-
-// Low five syndrome bits from the XOR of a codeword's position-domain words:
-// bit i is the parity of the bits whose in-word index has bit i set.
-__device__ __forceinline__ uint32_t fold5(uint32_t f)
-{
-    return (__popc(f & 0xAAAAAAAAu) & 1u) | ((__popc(f & 0xCCCCCCCCu) & 1u) << 1) |
-           ((__popc(f & 0xF0F0F0F0u) & 1u) << 2) | ((__popc(f & 0xFF00FF00u) & 1u) << 3) |
-           ((__popc(f & 0xFFFF0000u) & 1u) << 4);
-}
 
 struct ShortArgs {
     const uint32_t *in;
@@ -75,6 +70,7 @@ struct ShortArgs {
     uint32_t ylast;     // valid-bit mask of the last position-domain word
     uint32_t tlog;      // log2 of the team size of the syndrome pass
     int syn_type;
+    bool direct;        // one CTA that overwrites the counters
     const void *table;      // output-word offsets (see output_table), tab_len entries of 2 or 4 bytes
     uint32_t tab_len;
     uint32_t nJ;            // data runs J >= 5 that end inside the codeword's data (D_J < k)
@@ -144,6 +140,40 @@ __device__ __forceinline__ uint32_t run_word(const uint32_t *st, uint32_t cb, ui
     return (__funnelshift_r(lo, hi, sh) & m) | (__funnelshift_rc(lo, hi, sh + 1u) & ~m);
 }
 
+// End of a decode kernel: the lanes' counts to the counters.  direct: this CTA is
+// the whole grid and overwrites them (nothing cleared them); else they are added
+// to.  Warp w leaves its counts at base + w * stride (two words of shared memory of
+// its own).  Every thread of the CTA calls it.
+__device__ __forceinline__ void add_counts(bool direct, unsigned long long *err, unsigned long long *det, uint32_t errs,
+                                           uint32_t dets, uint32_t *base, uint32_t stride)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    errs = __reduce_add_sync(0xFFFFFFFFu, errs);
+    dets = __reduce_add_sync(0xFFFFFFFFu, dets);
+    if (!direct) {
+        if (lane == 0) {
+            grid_dep_wait();  // the counters' clear ahead of a programmatic dependent launch
+            if (err && errs) atomicAdd(err, (unsigned long long)errs);
+            if (det && dets) atomicAdd(det, (unsigned long long)dets);
+        }
+        return;
+    }
+    if (lane == 0) {
+        base[warp * stride] = errs;
+        base[warp * stride + 1] = dets;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long e = 0, d = 0;
+        for (uint32_t w = 0; w < blockDim.x / 32; ++w) {
+            e += base[w * stride];
+            d += base[w * stride + 1];
+        }
+        if (err) *err = e;
+        if (det) *det = d;
+    }
+}
+
 template <int W, int S, int SB, bool TAB_SMEM, bool SPLIT>
 __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
 {
@@ -179,8 +209,6 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
     // syndrome teams: T lanes per codeword, G codewords per round
     const uint32_t tlog = a.tlog, T = 1u << tlog, tl = lane & (T - 1u), team = lane >> tlog, G = 32u >> tlog;
     const uint32_t n = a.n, k = a.k, Ym1 = a.Y - 1u;
-    const uint32_t tl_last = Ym1 & (T - 1u);
-    const bool wide = ((a.Y + T - 1u) >> tlog) > 32u;  // a lane reads more than 32 words of a codeword
     const int32_t stage_bits = 8 * SB;  // reads past the data stay inside the stage's slack
     uint32_t errs = 0, dets = 0, it = 0;
     bool aborted = false;
@@ -207,77 +235,72 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             }
         }
 
-        // 1. syndromes.  Lane tl of a team reads position-domain words j = tl + T*i (at most
-        //    64); the low syndrome bits come from the XOR of all words, the high bits from the
-        //    XOR of the indices j of the odd-parity words: bit i of pm0 (i < 32) or of pm1
-        //    (i - 32) is the parity of word tl + T*i.
+        // 1. syndromes.  Lane tl of a team reads position-domain words j = tl + T*i, four at a
+        //    time (i = 4q + u): x is the XOR of all of them, A and B the XORs of those with bit 0
+        //    and bit 1 of u set, hq the XOR of the q whose four words have odd parity, so that
+        //    one popcount serves four words.  The low syndrome bits are parities of x, the high
+        //    ones the XOR of the indices j of the odd-parity words.
         for (uint32_t cbase = 0; cbase < gcnt; cbase += G) {
             const uint32_t c = cbase + team;
-            uint32_t x = 0, pm0 = 0, pm1 = 0;
+            uint32_t x = 0, A = 0, B = 0, hq = 0;
             if (c < gcnt) {
-                const int32_t q0 = (int32_t)(off0 + c * n) - 1 + 32 * (int32_t)tl;  // position 0 is bit -1 of c
+                const int32_t q0 = (int32_t)(off0 + c * n) - 1;  // position 0 is bit -1 of c (the guard word for c = 0)
                 const uint32_t sh = (uint32_t)q0 & 31u;
-                int32_t wi = q0 >> 5;  // -1 reads the guard word
-                uint32_t cnt = tl < Ym1 ? ((Ym1 - 1u - tl) >> tlog) + 1u : 0u;  // words before the last one
-                const uint32_t n0 = min(cnt, 32u), n1 = cnt - n0;
-                // a word's parity bit is shifted in (bit order reversed below)
-                auto take = [&](uint32_t y, uint32_t &pm) {
-                    x ^= y;
-                    pm = (pm << 1) | (__popc(y) & 1u);
+                const uint32_t *ad = st + (q0 >> 5) + (int32_t)tl;
+                auto take = [&](const uint32_t (&v)[4], uint32_t q) {
+                    A ^= v[1] ^ v[3];
+                    B ^= v[2] ^ v[3];
+                    const uint32_t b = v[0] ^ v[1] ^ v[2] ^ v[3];
+                    x ^= b;
+                    hq ^= q & (0u - (__popc(b) & 1u));
                 };
-                uint32_t lo = 0;  // only words of this codeword are read
-                // plain shared-memory loads, so that the compiler issues the unrolled
-                // iterations' loads ahead of their uses
-                const uint32_t *ad = st + wi;
-                if (T == 1) {  // one lane per codeword: each word is the next one's low half
-                    lo = ad[0];
-#pragma unroll 4
-                    for (uint32_t i = 0; i < n0; ++i, ++ad) {
-                        const uint32_t hi = ad[1];
-                        take(__funnelshift_r(lo, hi, sh), pm0);
-                        lo = hi;
-                    }
-#pragma unroll 4
-                    for (uint32_t i = 0; i < n1; ++i, ++ad) {
-                        const uint32_t hi = ad[1];
-                        take(__funnelshift_r(lo, hi, sh), pm1);
-                        lo = hi;
+                uint32_t j = tl, q = 0;
+                // plain shared-memory loads, so that the compiler issues an unrolled
+                // iteration's loads ahead of their uses
+                if (T == 1u) {  // a lane's words are neighbours: each one's high half is the next one's low half
+                    uint32_t lo = ad[0];
+#pragma unroll 2
+                    for (; j + 3u < Ym1; j += 4u, ++q, ad += 4) {
+                        uint32_t v[4];
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u) {
+                            const uint32_t hi = ad[u + 1];
+                            v[u] = __funnelshift_r(lo, hi, sh);
+                            lo = hi;
+                        }
+                        take(v, q);
                     }
                 } else {
-#pragma unroll 4
-                    for (uint32_t i = 0; i < n0; ++i, ad += T) take(__funnelshift_r(ad[0], ad[1], sh), pm0);
-#pragma unroll 4
-                    for (uint32_t i = 0; i < n1; ++i, ad += T) take(__funnelshift_r(ad[0], ad[1], sh), pm1);
-                    if (tl == tl_last) lo = ad[0];
+#pragma unroll 2
+                    for (; j + 3u * T < Ym1; j += 4u * T, ++q, ad += 4u * T) {
+                        uint32_t v[4];
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u) v[u] = __funnelshift_r(ad[u * T], ad[u * T + 1], sh);
+                        take(v, q);
+                    }
                 }
-                if (tl == tl_last) {  // the last word holds positions up to n only
-                    const uint32_t y = __funnelshift_r(lo, ad[1], sh) & a.ylast;
-                    if (cnt < 32u)
-                        take(y, pm0);
-                    else
-                        take(y, pm1);
-                    ++cnt;
+                if (j <= Ym1) {  // the last one to four words; word Ym1 holds positions up to n only
+                    uint32_t v[4];
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) {
+                        const uint32_t ju = j + u * T;
+                        v[u] = ju <= Ym1 ? __funnelshift_r(ad[u * T], ad[u * T + 1], sh) : 0u;
+                        if (ju == Ym1) v[u] &= a.ylast;
+                    }
+                    take(v, q);
                 }
-                const uint32_t m0 = min(cnt, 32u), m1 = cnt - m0;
-                pm0 = m0 ? __brev(pm0) >> (32u - m0) : 0u;
-                if (wide) pm1 = m1 ? __brev(pm1) >> (32u - m1) : 0u;
             }
-            // indices i of the odd-parity words (those of pm1 are 32 + their bit index;
-            // pm1 is used only when a lane reads more than 32 words)
-            uint32_t fi = fold5(pm0), par = __popc(pm0);
-            if (wide) {
-                const uint32_t par1 = __popc(pm1) & 1u;
-                fi ^= fold5(pm1) ^ (par1 << 5);
-                par ^= par1;
-            }
-            uint32_t h = ((par & 1u) ? tl : 0u) ^ (fi << tlog);
-            // XOR over the team: butterfly steps stay inside aligned groups of T lanes
-            for (uint32_t o = T >> 1; o > 0; o >>= 1) {
-                x ^= __shfl_xor_sync(0xFFFFFFFFu, x, o);
-                h ^= __shfl_xor_sync(0xFFFFFFFFu, h, o);
-            }
+            // the lane's share in one word: the low bits' parities on bits 1, 2, 4, 8, 16 of x's
+            // transform, the index bits from 17 up; XOR over the team (butterfly steps stay
+            // inside aligned groups of T lanes)
+            const uint32_t hi = hq << 2 | (__popc(B) & 1u) << 1 | (__popc(A) & 1u);
+            uint32_t z = (superset_xor<5>(x) & 0x00010116u) | ((hi << tlog) ^ ((__popc(x) & 1u) ? tl : 0u)) << 17;
+            if (T == 32u)
+                z = __reduce_xor_sync(0xFFFFFFFFu, z);
+            else
+                for (uint32_t o = T >> 1; o > 0; o >>= 1) z ^= __shfl_xor_sync(0xFFFFFFFFu, z, o);
             if (tl == 0 && c < gcnt) {
-                const uint32_t syn = (h << 5) | fold5(x);
+                const uint32_t syn = (z >> 17) << 5 | ((z >> 1) & 3u) | ((z >> 2) & 4u) | ((z >> 5) & 8u) | ((z >> 12) & 16u);
                 if (syn != 0) {
                     ++errs;
                     if (syn <= n) {
@@ -413,94 +436,112 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             if (tj < a.ntiles) (void)mbar_wait_bounded(&bar[j % S], (j / S) & 1u);
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        errs += __shfl_xor_sync(0xFFFFFFFFu, errs, o);
-        dets += __shfl_xor_sync(0xFFFFFFFFu, dets, o);
-    }
-    if (lane == 0) {
-        grid_dep_wait();  // the counters' clear ahead of a programmatic dependent launch
-        if (a.err && errs) atomicAdd(a.err, (unsigned long long)errs);
-        if (a.det && dets) atomicAdd(a.det, (unsigned long long)dets);
-    }
+    add_counts(a.direct, a.err, a.det, errs, dets, reinterpret_cast<uint32_t *>(smem), warp_bytes / 4);
 }
 
 // ---------------------------------------------------------------------------
-// Short segments (n <= 255): warp tiles of 32 codewords, one per lane.
-// 32 codewords of any length n fill exactly n input words and k output words.
+// Segments of at most WY position-domain words (n < 32 * WY): warp tiles of 32
+// codewords, one per lane, straight from global memory.  32 codewords of any
+// length n fill exactly n input words and k output words.  The data runs move to
+// constant places (positions past n are 0); the lanes OR theirs into the tile's k
+// output words in shared memory, which costs neither a division nor a loop over a
+// word's pieces.
+// Bound: the integer ALU (61 % busy at n = 70, 170 instructions a tile) below n = 150,
+// then the L1's wavefronts of the lanes' strided reads.  The per-lane kernel it
+// replaces (k < 64 only; bits moved a run at a time through shared memory) took 1296
+// us at n = 16 and 427 at n = 70 for 1 Gbit, this one 312 and 109; from n = 71 on see
+// kLaneMaxN.
 // ---------------------------------------------------------------------------
 constexpr int kSmallWarps = 8;
 
+template <int WY>
 __global__ void __launch_bounds__(kSmallWarps * 32)
     k_short_small(const uint32_t *__restrict__ in, uint64_t in_words, uint32_t n, uint32_t r, uint64_t num_cw,
                   uint32_t *__restrict__ out, uint64_t out_words, void *__restrict__ syn, int syn_type,
-                  unsigned long long *__restrict__ err, unsigned long long *__restrict__ det)
+                  unsigned long long *__restrict__ err, unsigned long long *__restrict__ det, bool direct)
 {
-    __shared__ uint32_t sy[kSmallWarps][kWarpSlotWords];
-    __shared__ uint32_t sd[kSmallWarps][kWarpSlotWords];
+    constexpr uint32_t kMerged = 32u * WY + WY + 1u;  // k words, and spill words for the last lane
+    __shared__ uint32_t merged[kSmallWarps][kMerged];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    uint32_t *my_y = &sy[wp][lane * kSlot];
-    uint32_t *my_d = &sd[wp][lane * kSlot];
+    uint32_t *m = merged[wp];
     const uint32_t k = n - r;
-    const uint32_t wy = (n + 32) >> 5;  // ceil((n + 1) / 32)
-    const uint32_t ylast = lowmask(n + 1 - 32 * (wy - 1));
     const uint64_t tiles = (num_cw + 31) / 32;
+    // position p of the lane's codeword is tile bit lane * n + p - 1
+    const int32_t bit = lane * (int32_t)n - 1, a0 = bit >> 5;
+    const uint32_t sh = (uint32_t)bit & 31u;
+    const uint32_t ob = (uint32_t)lane * k, os = ob & 31u, oe = (os + k + 31u) >> 5;  // the data bits' place in the tile
+    uint32_t *mine = m + (ob >> 5);
+    uint32_t mask[WY];  // valid positions (bit 0 of the first word is none)
+#pragma unroll
+    for (uint32_t w = 0; w < WY; ++w) mask[w] = n >= 32u * w ? lowmask(n + 1u - 32u * w) : 0u;
+    mask[0] &= ~1u;
     uint32_t errs = 0, dets = 0;
     for (uint64_t t = (uint64_t)blockIdx.x * kSmallWarps + wp; t < tiles; t += (uint64_t)gridDim.x * kSmallWarps) {
         const uint64_t i = t * 32 + lane;
         const bool valid = i < num_cw;
-        uint32_t y[8];
+        const uint32_t *src = in + t * n;
+        const uint32_t have = (uint32_t)min((uint64_t)n, in_words - t * n);  // words of the tile
+        uint32_t raw[WY + 1], y[WY];
 #pragma unroll
-        for (uint32_t w = 0; w < 8; ++w)
-            y[w] = (valid && w < wy) ? load_window(in, in_words, (int64_t)(i * n) - 1 + 32 * (int64_t)w) : 0u;
-        y[0] &= ~1u;
+        for (int w = 0; w <= WY; ++w) raw[w] = valid && (uint32_t)(a0 + w) < have ? src[a0 + w] : 0u;
 #pragma unroll
-        for (uint32_t w = 0; w < 8; ++w)
-            if (w == wy - 1) y[w] &= ylast;
-        const uint32_t s = syndrome_y(y, wy);
-        const uint32_t fix = s <= n ? s : 0u;  // a syndrome past n names no position
+        for (uint32_t w = 0; w <= WY; ++w)
+            if (32u * w + lane < kMerged) m[32u * w + lane] = 0u;
+        uint32_t x = 0, s = 0;
 #pragma unroll
-        for (uint32_t w = 0; w < 8; ++w)
-            if (w < wy) y[w] ^= shl_clamp(fix != 0 ? 1u : 0u, fix - 32u * w);
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            my_y[w] = y[w];
-            my_d[w] = 0;
+        for (int w = 0; w < WY; ++w) {
+            y[w] = __funnelshift_r(raw[w], raw[w + 1], sh) & mask[w];
+            x ^= y[w];
         }
-        my_y[8] = 0;
-        my_d[8] = 0;
-        // data run j: positions 2^j + 1 .. min(2^(j+1) - 1, n)
-        for (uint32_t j = 1; j < r; ++j) {
-            const uint32_t first = (1u << j) + 1u, last = min((2u << j) - 1u, n);
-            if (last >= first) copy_bits(my_y, first, my_d, (1u << j) - j - 1u, last - first + 1u);
+#pragma unroll
+        for (int b = 0; (1 << b) < WY; ++b) {
+            uint32_t g = 0;
+#pragma unroll
+            for (int w = 0; w < WY; ++w)
+                if ((w >> b) & 1) g ^= y[w];
+            s |= (__popc(g) & 1u) << (5 + b);
         }
-        __syncwarp();
-        for (uint32_t q = lane; q < k; q += 32) {
-            const uint64_t g = t * k + q;
-            if (g >= out_words) break;
-            uint32_t c = (32u * q) / k, o = 32u * q - c * k, v = 0, filled = 0;
-            while (filled < 32 && c < 32) {
-                const uint32_t avail = k - o, take = avail < 32 - filled ? avail : 32 - filled;
-                v |= get_bits(&sd[wp][c * kSlot], o, take) << filled;
-                filled += take;
-                ++c;
-                o = 0;
-            }
-            out[g] = v;
+        const uint32_t z = superset_xor<5>(x);
+        s |= ((z >> 1) & 3u) | ((z >> 2) & 4u) | ((z >> 5) & 8u) | ((z >> 12) & 16u);
+        const uint32_t fix = s <= n ? s : 0u;  // a syndrome past n names no position; bit 0 is dropped again
+#pragma unroll
+        for (int w = 0; w < WY; ++w) y[w] ^= shl_clamp(1u, fix - 32u * (uint32_t)w);
+        // the data bits, packed: 26 of the first word, then 31 or 32 a word
+        uint32_t d[WY + 1];
+        d[0] = compress_runs<5>(y[0] & ~1u);
+#pragma unroll
+        for (int w = 1; w <= WY; ++w) d[w] = 0u;
+        int at = 26;
+#pragma unroll
+        for (int w = 1; w < WY; ++w) {
+            const bool chk = (w & (w - 1)) == 0;  // position 32w is a checksum position
+            const uint32_t v = chk ? y[w] >> 1 : y[w];
+            d[at / 32] |= v << (at % 32);
+            if (at % 32 != 0) d[at / 32 + 1] |= v >> (32 - at % 32);
+            at += chk ? 31 : 32;
         }
+        __syncwarp();  // the tile's words are cleared
         if (valid) {
+            uint32_t lo = 0;
+#pragma unroll
+            for (uint32_t w = 0; w <= WY; ++w) {
+                if (w < oe) atomicOr(&mine[w], __funnelshift_l(lo, d[w], os));
+                lo = d[w];
+            }
             if (syn_type == 1) static_cast<uint8_t *>(syn)[i] = (uint8_t)s;
             if (syn_type == 2) static_cast<uint16_t *>(syn)[i] = (uint16_t)s;
         }
         errs += __popc(__ballot_sync(0xFFFFFFFFu, valid && s != 0));
         dets += __popc(__ballot_sync(0xFFFFFFFFu, valid && s > n));
         __syncwarp();
+        uint32_t *o = out + t * k;
+        const uint32_t words = (uint32_t)min((uint64_t)k, out_words - t * k);
+#pragma unroll
+        for (uint32_t w = 0; w < WY; ++w)
+            if (32u * w + lane < words) o[32u * w + lane] = m[32u * w + lane];
+        __syncwarp();  // the next tile clears the words
     }
-    if (lane == 0) {
-        grid_dep_wait();  // the counters' clear ahead of a programmatic dependent launch
-        if (err && errs) atomicAdd(err, (unsigned long long)errs);
-        if (det && dets) atomicAdd(det, (unsigned long long)dets);
-    }
+    add_counts(direct, err, det, lane == 0 ? errs : 0u, lane == 0 ? dets : 0u, merged[0], kMerged);
 }
 
 // ---------------------------------------------------------------------------
@@ -604,8 +645,8 @@ int short_blocks_per_sm(int v, int tsm, uint32_t smem)
     return bps;
 }
 
-// The configuration for length n: a pinned one, else the autotuner's, else the built-in default.
-int current_short_variant(uint32_t n)
+// The configuration chosen for length n: a pinned one, else the autotuner's, else -1.
+int chosen_short_variant(uint32_t n)
 {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -614,9 +655,10 @@ int current_short_variant(uint32_t n)
     if (g_short_choice[dev] > 0) return g_short_choice[dev] - 1;
     for (const TunedEntry &e : g_short_tuned[dev])
         if (e.n == n && e.v >= 0) return e.v;
-    return 0;
+    return -1;
 }
 
+// v < 0 forgets the length.
 void remember_short_variant(uint32_t n, int v)
 {
     int dev = 0;
@@ -631,27 +673,26 @@ void remember_short_variant(uint32_t n, int v)
         }
         if (!slot && e.v < 0) slot = &e;
     }
+    if (v < 0 && (!slot || slot->n != n)) return;
     if (!slot) slot = &g_short_tuned[dev][n % 64];  // table full: overwrite one entry
     slot->n = n;
     slot->v = v;
 }
 
 // Team size of the syndrome pass: a team of T lanes reads a codeword's Y
-// position-domain words, ceil(Y / T) per lane (at most 64: one bit each in the
-// two parity masks), and a tile's codewords take ceil(g / (32 / T)) rounds.
-// Each round ends in a chain of dependent steps (the reductions, the
-// butterfly over the team, the correction), which on GB300 measured as long as
-// about 31 word steps (the paper's (M, t) grid: 3 rounds of 13 words took 139
-// µs where 1 round of 32 took 111), plus a little per butterfly step.  Pick
-// the T with the lowest cost per tile.
+// position-domain words, ceil(Y / 4T) blocks of four per lane, and a tile's
+// codewords take ceil(g / (32 / T)) rounds, each of which ends in a chain of
+// dependent steps (the transform, the butterfly over the team, the correction).
+// The weights follow the times of every T at 18 lengths on GB300 (1 Gbit, T = 1 ..
+// 16: n = 1078 65/73/87/107/146 us, n = 3212 71/59/64/67/76, n = 8013
+// 128/91/73/66/75); the pick is the fastest at all of them.
 uint32_t team_log(uint32_t Y, uint32_t g)
 {
     uint32_t best = 5;
     uint64_t best_cost = ~0ull;
     for (uint32_t lg = 0; lg <= 5; ++lg) {
-        const uint32_t T = 1u << lg, G = 32u >> lg, per_lane = (Y + T - 1) / T;
-        if (per_lane > 64) continue;
-        const uint64_t cost = (uint64_t)((g + G - 1) / G) * (per_lane * 10u + 310u + 30u * lg);
+        const uint32_t T = 1u << lg, G = 32u >> lg;
+        const uint64_t cost = (uint64_t)((g + G - 1) / G) * ((Y + 4 * T - 1) / (4 * T) * 40 + 160 + 20 * lg);
         if (cost < best_cost) {
             best_cost = cost;
             best = lg;
@@ -799,9 +840,25 @@ void table_used(TableEntry *e, cudaStream_t st)
     else cudaEventRecord(e->last, st);
 }
 
+// Launch a decode whose counts start from zero: a grid of one CTA overwrites the
+// counters (*direct), any other is the programmatic dependent of their clear.
+// bare: the decode alone, added to counters nobody cleared (timing).
+template <class Launch>
+cudaError_t launch_counted(bool &direct, unsigned long long *err, unsigned long long *det, int grid, bool bare,
+                           cudaStream_t st, Launch launch)
+{
+    direct = grid == 1 && !bare;
+    const bool clear = (err || det) && !direct && !bare;
+    if (clear) {
+        const cudaError_t e = launch_zero_counts(err, det, st);
+        if (e != cudaSuccess) return e;
+    }
+    return launch(clear);
+}
+
 cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t num_cw, uint32_t *out, void *syn,
                                int syn_type, unsigned long long *err, unsigned long long *det, cudaStream_t st,
-                               const void *table, uint32_t tab_len, bool pdl = false)
+                               const void *table, uint32_t tab_len, bool bare)
 {
     const ShortVariant &v = kShortVariants[vi];
     const uint32_t r = short_r(n), k = n - r;
@@ -820,11 +877,9 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     a.k = k;
     a.g = std::min<uint32_t>((8u * v.SB - 256u) / n, TileGeom<4096>::max_g);  // as tile_codewords<SB>
     if (a.g == 0) return cudaErrorInvalidValue;  // the caller picks a configuration whose stage holds a codeword
-    a.ntiles = (num_cw + a.g - 1) / a.g;
     a.Y = (n + 32) / 32;
     const uint32_t lastbits = n + 1 - 32 * (a.Y - 1);
     a.ylast = lastbits >= 32 ? 0xFFFFFFFFu : (1u << lastbits) - 1u;
-    a.tlog = team_log(a.Y, a.g);
     a.table = table;
     a.tab_len = tab_len;
     if (!a.table) return cudaErrorInvalidValue;
@@ -839,10 +894,46 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     if (split) a.nJ = 0;  // no per-codeword pass for checksum words
     const int bps = short_blocks_per_sm(vi, tsm, smem);
     if (bps <= 0) return cudaErrorInvalidConfiguration;
-    const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
-    const uint64_t want = (a.ntiles + v.W - 1) / v.W;
-    const int grid = decode_grid(want, cap);
-    return v.launch[tsm](a, grid, smem, st, pdl);
+    const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps, warps = cap * (uint64_t)v.W;
+    // Even tiles: no more codewords per tile than give every resident warp as many tiles
+    // (160,000 segments of n = 3212: 16,000 tiles of 10 were 4.4 rounds of 3648 warps), down
+    // to one codeword per tile for short streams, which then spread over the whole GPU.
+    const uint64_t rounds = (num_cw + a.g * warps - 1) / (a.g * warps);
+    a.g = (uint32_t)((num_cw + rounds * warps - 1) / (rounds * warps));
+    a.ntiles = (num_cw + a.g - 1) / a.g;
+    a.tlog = team_log(a.Y, a.g);
+    const int grid = decode_grid((a.ntiles + v.W - 1) / v.W, cap);
+    return launch_counted(a.direct, err, det, grid, bare, st, [&](bool pdl) {
+        return v.launch[tsm](a, grid, smem, st, pdl);
+    });
+}
+
+// One codeword per lane: n < kLaneMaxN.  The kernel of the first word count that
+// holds n (even counts above 16).
+template <size_t... I>
+void (*lane_kernel(uint32_t words, std::index_sequence<I...>))(const uint32_t *, uint64_t, uint32_t, uint32_t, uint64_t,
+                                                               uint32_t *, uint64_t, void *, int, unsigned long long *,
+                                                               unsigned long long *, bool)
+{
+    static const decltype(&k_short_small<1>) kernels[] = {&k_short_small<(int)(I < 16 ? I + 1 : (I + 2) / 2 * 2)>...};
+    return kernels[words - 1];
+}
+
+cudaError_t launch_short_lanes(const uint32_t *in, uint32_t n, uint64_t num_cw, uint32_t *out, void *syn, int syn_type,
+                               unsigned long long *err, unsigned long long *det, cudaStream_t st, bool bare)
+{
+    const uint32_t r = short_r(n);
+    const auto kern = lane_kernel(n / 32 + 1, std::make_index_sequence<kLaneMaxN / 32>());
+    const uint64_t tiles = (num_cw + 31) / 32;
+    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kern), kSmallWarps * 32, 0);
+    if (bps <= 0) return cudaErrorInvalidConfiguration;
+    const int grid = decode_grid((tiles + kSmallWarps - 1) / kSmallWarps, (uint64_t)num_sms() * (uint64_t)bps);
+    bool direct = false;
+    return launch_counted(direct, err, det, grid, bare, st, [&](bool pdl) {
+        return launch_kernel(kern, dim3((unsigned)grid), dim3(kSmallWarps * 32), 0, st, pdl, in,
+                             words_for_bits(num_cw * n), n, r, num_cw, out, words_for_bits(num_cw * (n - r)), syn,
+                             syn_type, err, det, direct);
+    });
 }
 
 }  // namespace
@@ -899,42 +990,33 @@ hd_status check_short_args(const uint32_t *stream, uint64_t in_bits, uint32_t n,
     return HD_OK;
 }
 
-// The decode itself, given the output-word table of n (unused for k < 64);
-// pdl: launched as the programmatic dependent of the counters' clear.
+// The decode itself, the counters' clear included, given the output-word table
+// of n (unused for k < 64).
 hd_status decode_short_with(const uint32_t *stream, uint64_t in_bits, uint32_t n, uint64_t num_codewords,
                             uint32_t *out_bits, void *syndromes, hd_syn_type syn_type,
                             unsigned long long *err_count, unsigned long long *detected_count, cudaStream_t st,
-                            const void *table, uint32_t tab_len, bool pdl)
+                            const void *table, uint32_t tab_len)
 {
+    if (num_codewords == 0) {
+        if (!err_count && !detected_count) return HD_OK;
+        return launch_zero_counts(err_count, detected_count, st) == cudaSuccess ? HD_OK : HD_ERR_CUDA;
+    }
     const uint32_t r = short_r(n), k = n - r;
     const int syn = syndromes ? (int)syn_type : 0;
-    if (k >= kLongMinK) {
-        int vi = current_short_variant(n);
-        if (kShortVariants[vi].SB * 8u < n + 256u) vi = largest_stage_variant();  // stage too small for a codeword
-        if (launch_short_tiles(vi, stream, n, num_codewords, out_bits, syndromes, syn, err_count, detected_count,
-                               st, table, tab_len, pdl) != cudaSuccess)
-            return HD_ERR_CUDA;
-        return HD_OK;
-    }
-    const uint64_t tiles = (num_codewords + 31) / 32;
-    const uint64_t want = (tiles + kSmallWarps - 1) / kSmallWarps, cap = (uint64_t)num_sms() * 8;
-    return launch_kernel(k_short_small, dim3((unsigned)decode_grid(want, cap)), dim3(kSmallWarps * 32), 0, st, pdl,
-                         stream, words_for_bits(in_bits), n, r, num_codewords, out_bits,
-                         words_for_bits(num_codewords * k), syndromes, syn, err_count, detected_count) == cudaSuccess
+    // the tiled kernel from kLaneMaxN on, and below it (k >= 64) where a configuration is
+    // pinned or the autotuner found one faster
+    int vi = k >= kLongMinK ? chosen_short_variant(n) : -1;
+    if (vi < 0 && n < kLaneMaxN)
+        return launch_short_lanes(stream, n, num_codewords, out_bits, syndromes, syn, err_count, detected_count, st,
+                                  false) == cudaSuccess
+                   ? HD_OK
+                   : HD_ERR_CUDA;
+    if (vi < 0) vi = 0;  // the built-in configuration
+    if (kShortVariants[vi].SB * 8u < n + 256u) vi = largest_stage_variant();  // stage too small for a codeword
+    return launch_short_tiles(vi, stream, n, num_codewords, out_bits, syndromes, syn, err_count, detected_count, st,
+                              table, tab_len, false) == cudaSuccess
                ? HD_OK
                : HD_ERR_CUDA;
-}
-
-// Clear the counters (a one-thread kernel the decode may overlap); true when
-// the decode is to be launched as its programmatic dependent.
-hd_status clear_counts(unsigned long long *err_count, unsigned long long *detected_count, cudaStream_t st,
-                       bool *pdl)
-{
-    *pdl = false;
-    if (!err_count && !detected_count) return HD_OK;
-    if (launch_zero_counts(err_count, detected_count, st) != cudaSuccess) return HD_ERR_CUDA;
-    *pdl = true;
-    return HD_OK;
 }
 
 }  // namespace
@@ -962,11 +1044,8 @@ hd_status hd_decode_short(const uint32_t *stream, uint64_t in_bits, uint32_t n, 
         if (te == cudaErrorStreamCaptureUnsupported) return HD_ERR_INVALID_ARG;  // build it outside the capture
         if (te != cudaSuccess) return HD_ERR_CUDA;
     }
-    bool pdl = false;
-    if ((rc = clear_counts(err_count, detected_count, st, &pdl)) != HD_OK) return rc;
-    if (num_codewords == 0) return HD_OK;
     rc = decode_short_with(stream, in_bits, n, num_codewords, out_bits, syndromes, syn_type, err_count,
-                           detected_count, st, e ? e->dev : nullptr, e ? e->len : 0, pdl);
+                           detected_count, st, e ? e->dev : nullptr, e ? e->len : 0);
     if (e && rc == HD_OK) table_used(e, st);
     return rc;
 }
@@ -1003,11 +1082,8 @@ hd_status hd_decode_short_plan(const hd_short_plan *plan, const uint32_t *stream
     if (cudaGetDevice(&dev) != cudaSuccess) return HD_ERR_CUDA;
     if (dev != plan->device) return HD_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    bool pdl = false;
-    if ((rc = clear_counts(err_count, detected_count, st, &pdl)) != HD_OK) return rc;
-    if (num_codewords == 0) return HD_OK;
     return decode_short_with(stream, in_bits, plan->n, num_codewords, out_bits, syndromes, syn_type, err_count,
-                             detected_count, st, plan->table, plan->tab_len, pdl);
+                             detected_count, st, plan->table, plan->tab_len);
 }
 
 void hd_short_plan_destroy(hd_short_plan *plan)
@@ -1067,7 +1143,7 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
         auto go = [&]() {
             return launch_short_tiles(v, static_cast<const uint32_t *>(din), n, num_codewords,
                                       static_cast<uint32_t *>(dout), dsyn, HD_SYN_U16, cnt, cnt + 1, st, tab->dev,
-                                      tab->len);
+                                      tab->len, true);
         };
         if (go() != cudaSuccess) {  // warm-up (also configures the kernel)
             rc = HD_ERR_CUDA;
@@ -1086,6 +1162,21 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
             best_ms = ms;
         }
     }
+    // below kLaneMaxN a configuration is kept only if it beats one codeword per lane
+    bool beaten = false;
+    if (rc == HD_OK && best >= 0 && n < kLaneMaxN) {
+        auto go = [&]() {
+            return launch_short_lanes(static_cast<const uint32_t *>(din), n, num_codewords, static_cast<uint32_t *>(dout),
+                                      dsyn, HD_SYN_U16, cnt, cnt + 1, st, true);
+        };
+        float ms = 0.f;
+        if (go() != cudaSuccess) rc = HD_ERR_CUDA;
+        cudaEventRecord(e0, st);
+        for (uint32_t i = 0; rc == HD_OK && i < reps; ++i) go();
+        cudaEventRecord(e1, st);
+        if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) rc = HD_ERR_CUDA;
+        beaten = ms <= best_ms;
+    }
     if (tab) table_used(tab, st);
     if (din) cudaFree(din);
     if (dout) cudaFree(dout);
@@ -1094,7 +1185,7 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (rc != HD_OK) return rc;
-    if (best >= 0) remember_short_variant(n, best);
+    if (best >= 0) remember_short_variant(n, beaten ? -1 : best);
     if (chosen) *chosen = best;
     return HD_OK;
 }
