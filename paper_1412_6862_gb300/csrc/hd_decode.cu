@@ -82,18 +82,39 @@ std::map<int, uint32_t *> g_status_ptr;
 // Built-in choice per (n, syndrome type or -1 for any, G, T, S, inplace,
 // decode table), measured on GB300; used until the autotuner or the caller
 // picks another configuration.  The first entry of n that matches the
-// syndrome type and is compiled for it wins (n = 15 with u16 syndromes: 512
-// threads in place, 18.4 µs at 2^24 codewords against 18.9 µs for the
-// 576-thread configuration with separate output buffers).
+// syndrome type and is compiled for it wins.  At 2^24 codewords: n = 15 with u16
+// syndromes 18.1 us in place against 18.9 for the 576-thread configuration with
+// separate output buffers; n = 31 with u16 syndromes 26.4 us with 16 codewords per
+// thread, 27.4 with 32; n = 63 with none / u8 / u16 syndromes 40.9 / 42.6 / 47.0 us
+// with separate output buffers (one CTA per SM, its four warps' loads a whole chunk
+// further ahead), 41.4 / 47.7 / 52.0 in place with three stages (two CTAs per SM);
+// at 2^26 codewords with u8 syndromes 169 against 186.
 struct DefaultCfg {
     uint32_t n;
     int syn, G, T, S, inplace, lut;
 };
 constexpr DefaultCfg kDefaults[] = {
     {7, -1, 32, 128, 4, 1, 1},  {15, 2, 32, 512, 2, 1, 1},   {15, -1, 32, 576, 2, 0, 1},
-    {15, -1, 32, 512, 2, 1, 1}, {31, -1, 32, 128, 3, 1, 0},  {63, -1, 32, 128, 3, 1, 0},
+    {15, -1, 32, 512, 2, 1, 1}, {31, 2, 16, 256, 3, 1, 0},   {31, -1, 32, 128, 3, 1, 0}, {63, -1, 32, 128, 3, 0, 0},
     {127, -1, 8, 256, 3, 1, 0}, {255, -1, 8, 128, 2, 1, 0},
 };
+
+// SECDED: the built-in arithmetic configuration, the first compiled one of n unless
+// listed here (2^24 codewords, u8 syndromes: n = 31 24.4 us with four stages of 128
+// threads against 26.1 with two of 256, n = 63 45.4 against 46.6 for 64 threads).
+constexpr DefaultCfg kSecdedDefaults[] = {
+    {31, -1, 32, 128, 4, 1, 0},
+    {63, -1, 32, 128, 3, 1, 0},
+};
+
+bool secded_default(const StreamVariant &x)
+{
+    for (const auto &d : kSecdedDefaults)
+        if (d.n == x.n && (d.syn < 0 || d.syn == x.syn) && d.G == x.G && d.T == x.T && d.S == x.S &&
+            d.inplace == x.inplace)
+            return true;
+    return false;
+}
 
 int find_variant(uint32_t n, int syn, int G, int T, int S, int inplace, int lut)
 {
@@ -240,7 +261,7 @@ cudaError_t launch_decode_secded(const DecodeJob &j, cudaStream_t st, bool pdl)
     for (const StreamVariant &x : secded_variants())
         if (x.n == j.n && x.syn == j.syn_type) {
             if (!x.lut) {
-                if (v == nullptr) v = &x;
+                if (v == nullptr || secded_default(x)) v = &x;
             } else if (vt == nullptr) {
                 vt = &x;
             }

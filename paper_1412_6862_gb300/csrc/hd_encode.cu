@@ -58,9 +58,9 @@ struct EncCfg {
     static_assert(smem <= 232448 && S >= 2 && S <= 8, "shared memory per CTA");
 };
 
+// (The buffers are kernel parameters of their own, so that the compiler knows
+// them for global memory.)
 struct EncArgs {
-    const uint32_t *data;
-    uint32_t *stream;
     uint64_t data_words, stream_words, num_cw;
     uint64_t nchunks;              // whole chunks encoded as such
     uint64_t tile_begin, tile_end;  // 32-codeword tiles for the per-lane path
@@ -68,7 +68,7 @@ struct EncArgs {
 };
 
 template <int N_, int T, int S, int G, int CH>
-__global__ void __launch_bounds__(T) k_encode_stream(const EncArgs a)
+__global__ void __launch_bounds__(T) k_encode_stream(const uint32_t *__restrict__ data, uint32_t *__restrict__ stream, const EncArgs a)
 {
     using Cfg = EncCfg<N_, T, S, G, CH>;
     using C = Code<N_>;
@@ -83,13 +83,13 @@ __global__ void __launch_bounds__(T) k_encode_stream(const EncArgs a)
 
     // the tail's tiles, from the grid's last warp on
     for (uint64_t t = a.tile_begin + (tw - 1 - gw); t < a.tile_end; t += tw)
-        encode_lane_tile<N_>(a.data, a.data_words, a.num_cw, t, a.stream, a.stream_words,
+        encode_lane_tile<N_>(data, a.data_words, a.num_cw, t, stream, a.stream_words,
                              reinterpret_cast<uint32_t *>(ring), lane);
     if (gw >= a.nchunks) return;
 
     auto load = [&](uint64_t c, int s) {
         mbar_arrive_expect_tx(&bar[s], Cfg::in_bytes);
-        bulk_g2s(ring + s * Cfg::stage_bytes, a.data + c * (uint64_t)Cfg::in_words, Cfg::in_bytes, &bar[s]);
+        bulk_g2s(ring + s * Cfg::stage_bytes, data + c * (uint64_t)Cfg::in_words, Cfg::in_bytes, &bar[s]);
     };
     fence_proxy_async_smem();  // the tiles above used the ring
     __syncwarp();
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(T) k_encode_stream(const EncArgs a)
             bulk_wait_read<0>();
             const uint64_t cn = c - tw + (uint64_t)S * tw;
             if (it > 0 && cn < a.nchunks) load(cn, (int)((it - 1) % S));
-            bulk_s2g(a.stream + c * (uint64_t)Cfg::out_words, stage, Cfg::out_bytes);
+            bulk_s2g(stream + c * (uint64_t)Cfg::out_words, stage, Cfg::out_bytes);
             bulk_commit();
         }
         __syncwarp();
@@ -170,18 +170,18 @@ __global__ void __launch_bounds__(T) k_encode_stream(const EncArgs a)
 constexpr int kLaneWarps = 8;
 
 template <int N_>
-__global__ void __launch_bounds__(kLaneWarps * 32) k_encode_lanes(const EncArgs a)
+__global__ void __launch_bounds__(kLaneWarps * 32) k_encode_lanes(const uint32_t *__restrict__ data, uint32_t *__restrict__ stream, const EncArgs a)
 {
     __shared__ uint32_t slots[kLaneWarps][32 * lane_slot_words(Code<N_>::Wy)];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     grid_dep_launch_dependents();
     grid_dep_wait();
     for (uint64_t t = (uint64_t)blockIdx.x * kLaneWarps + warp; t < a.tile_end; t += (uint64_t)gridDim.x * kLaneWarps)
-        encode_lane_tile<N_>(a.data, a.data_words, a.num_cw, t, a.stream, a.stream_words, slots[warp], lane);
+        encode_lane_tile<N_>(data, a.data_words, a.num_cw, t, stream, a.stream_words, slots[warp], lane);
 }
 
 template <int N_, int T, int S, int G, int CH = 1>
-cudaError_t launch_encode_stream(EncArgs a, cudaStream_t st)
+cudaError_t launch_encode_stream(const uint32_t *data, uint32_t *stream, EncArgs a, cudaStream_t st)
 {
     using Cfg = EncCfg<N_, T, S, G, CH>;
     a.tile_end = (a.num_cw + 31) / 32;
@@ -195,7 +195,8 @@ cudaError_t launch_encode_stream(EncArgs a, cudaStream_t st)
     // n = 255: 2.8 against 3.6 at 100,000, 4.8 against 4.4 at 200,000.
     if (a.tile_end <= (uint64_t)decode_grid(lane_cap, lane_cap) * kLaneWarps) {
         const int grid = decode_grid((a.tile_end + kLaneWarps - 1) / kLaneWarps, lane_cap);
-        return launch_kernel(k_encode_lanes<N_>, dim3((unsigned)grid), dim3(kLaneWarps * 32), 0, st, true, a);
+        return launch_kernel(k_encode_lanes<N_>, dim3((unsigned)grid), dim3(kLaneWarps * 32), 0, st, true,
+                             data, stream, a);
     }
     auto kern = k_encode_stream<N_, T, S, G, CH>;
     const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kern), T, Cfg::smem);
@@ -203,7 +204,7 @@ cudaError_t launch_encode_stream(EncArgs a, cudaStream_t st)
     a.nchunks = a.num_cw / Cfg::chunk_cw;
     a.tile_begin = a.nchunks * (Cfg::chunk_cw / 32);
     const int grid = decode_grid((a.nchunks + Cfg::WARPS - 1) / Cfg::WARPS, (uint64_t)num_sms() * (uint64_t)bps);
-    return launch_kernel(kern, dim3((unsigned)grid), dim3(T), Cfg::smem, st, true, a);
+    return launch_kernel(kern, dim3((unsigned)grid), dim3(T), Cfg::smem, st, true, data, stream, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -330,21 +331,19 @@ cudaError_t launch_encode(const uint32_t *data, uint64_t data_words, uint32_t n,
                           uint64_t stream_words, cudaStream_t st)
 {
     EncArgs a{};
-    a.data = data;
-    a.stream = stream;
     a.data_words = data_words;
     a.stream_words = stream_words;
     a.num_cw = num_cw;
     a.status = status_ptr();
     if (a.status == nullptr) return cudaErrorInvalidSymbol;
     switch (n) {
-        case 3: return launch_encode_stream<3, 128, 2, 32, 8>(a, st);
-        case 7: return launch_encode_stream<7, 128, 2, 32, 4>(a, st);
-        case 15: return launch_encode_stream<15, 256, 4, 32>(a, st);
-        case 31: return launch_encode_stream<31, 128, 3, 32>(a, st);
-        case 63: return launch_encode_stream<63, 128, 3, 32>(a, st);
-        case 127: return launch_encode_stream<127, 256, 3, 8>(a, st);
-        case 255: return launch_encode_stream<255, 128, 2, 8>(a, st);
+        case 3: return launch_encode_stream<3, 128, 2, 32, 8>(data, stream, a, st);
+        case 7: return launch_encode_stream<7, 128, 2, 32, 4>(data, stream, a, st);
+        case 15: return launch_encode_stream<15, 256, 4, 32>(data, stream, a, st);
+        case 31: return launch_encode_stream<31, 128, 3, 32>(data, stream, a, st);
+        case 63: return launch_encode_stream<63, 128, 3, 32>(data, stream, a, st);
+        case 127: return launch_encode_stream<127, 256, 3, 8>(data, stream, a, st);
+        case 255: return launch_encode_stream<255, 128, 2, 8>(data, stream, a, st);
         default: return cudaErrorInvalidValue;
     }
 }

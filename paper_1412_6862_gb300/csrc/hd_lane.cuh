@@ -15,25 +15,6 @@ namespace hd {
 // zero spare for the two-word reads, and an odd stride against bank conflicts.
 __host__ __device__ constexpr int lane_slot_words(int words) { return (words + 1) | 1; }
 
-// ---------------------------------------------------------------------------
-// Checksum bits by a superset XOR transform.  After the steps for the index
-// bits 0 .. M-1, bit j of the result is the XOR of the bits of y whose index
-// contains j (as a bit set), so bit 2^b is the parity of index set I_b: every
-// checksum bit lands on its own position.  Two operations a step (a shift and
-// one lop3) against a mask, a popcount and a gather per bit; and for codes
-// shorter than a word the same steps serve several codewords side by side.
-// ---------------------------------------------------------------------------
-template <int M>
-__device__ __forceinline__ uint32_t superset_xor(uint32_t y)
-{
-    y ^= (y >> 1) & 0x55555555u;
-    if constexpr (M >= 2) y ^= (y >> 2) & 0x33333333u;
-    if constexpr (M >= 3) y ^= (y >> 4) & 0x0F0F0F0Fu;
-    if constexpr (M >= 4) y ^= (y >> 8) & 0x00FF00FFu;
-    if constexpr (M >= 5) y ^= y >> 16;
-    return y;
-}
-
 // v repeated in every field of 2^M bits of a word.
 template <int M>
 __host__ __device__ constexpr uint32_t in_fields(uint32_t v)

@@ -55,11 +55,6 @@ __host__ __device__ inline uint32_t short_r(uint32_t n)
 __device__ __forceinline__ uint32_t lowmask(uint32_t b) { return b >= 32 ? 0xFFFFFFFFu : (1u << b) - 1u; }
 
 struct ShortArgs {
-    const uint32_t *in;
-    uint32_t *out;
-    void *syn;
-    unsigned long long *err;
-    unsigned long long *det;
     uint32_t *status;
     uint64_t num_cw;
     uint64_t in_words;
@@ -71,8 +66,7 @@ struct ShortArgs {
     uint32_t tlog;      // log2 of the team size of the syndrome pass
     int syn_type;
     bool direct;        // one CTA that overwrites the counters
-    const void *table;      // output-word offsets (see output_table), tab_len entries of 2 or 4 bytes
-    uint32_t tab_len;
+    uint32_t tab_len;       // entries of the output-word table (see output_table), 2 or 4 bytes each
     uint32_t nJ;            // data runs J >= 5 that end inside the codeword's data (D_J < k)
     uint32_t nJ_magic;      // ceil(2^32 / nJ) for nJ > 1: f / nJ = umulhi(f, nJ_magic) for the small f used
 };
@@ -92,6 +86,18 @@ inline uint32_t tile_codewords(uint32_t n)
     return std::min<uint32_t>(g, TileGeom<SB>::max_g);
 }
 
+// A decode's buffers: parameters of the kernels of their own, so that the
+// compiler knows them for global memory (a store through a struct's pointer
+// might alias the stage, and holds back the shared-memory loads behind it).
+struct ShortBuffers {
+    const uint32_t *in;
+    uint32_t *out;
+    void *syn;
+    unsigned long long *err;
+    unsigned long long *det;
+    const void *table;
+};
+
 // Bytes of tile t that a bulk copy brings in, and where they start.
 __device__ __forceinline__ void tile_span(const ShortArgs &a, uint64_t t, uint64_t &byte0, uint32_t &bytes,
                                           uint32_t &gcnt)
@@ -106,13 +112,14 @@ __device__ __forceinline__ void tile_span(const ShortArgs &a, uint64_t t, uint64
 }
 
 template <int SB>
-__device__ __forceinline__ void issue_tile(const ShortArgs &a, uint64_t t, uint8_t *stage, uint64_t *bar)
+__device__ __forceinline__ void issue_tile(const ShortArgs &a, const uint32_t *in, uint64_t t, uint8_t *stage,
+                                           uint64_t *bar)
 {
     uint64_t byte0;
     uint32_t bytes, gcnt;
     tile_span(a, t, byte0, bytes, gcnt);
     mbar_arrive_expect_tx(bar, bytes);
-    if (bytes) bulk_g2s(stage + 16, reinterpret_cast<const uint8_t *>(a.in) + byte0, bytes, bar);
+    if (bytes) bulk_g2s(stage + 16, reinterpret_cast<const uint8_t *>(in) + byte0, bytes, bar);
 }
 
 // The first 32 data bits of the codeword whose position 1 is stage bit cb
@@ -175,7 +182,10 @@ __device__ __forceinline__ void add_counts(bool direct, unsigned long long *err,
 }
 
 template <int W, int S, int SB, bool TAB_SMEM, bool SPLIT>
-__global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
+__global__ void __launch_bounds__(W * 32)
+    k_short_tiles(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, void *__restrict__ syn,
+                  unsigned long long *__restrict__ err, unsigned long long *__restrict__ det,
+                  const void *__restrict__ table, const ShortArgs a)
 {
     using Geom = TileGeom<SB>;
     extern __shared__ __align__(128) uint8_t smem[];
@@ -185,7 +195,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
     // SPLIT: 32-bit entries that also say where a word's checksum position falls, resolved
     // in pass 3; otherwise 16-bit entries and pass 5 rewrites those words
     using Entry = typename std::conditional<SPLIT, uint32_t, uint16_t>::type;
-    const Entry *tab = static_cast<const Entry *>(a.table);
+    const Entry *tab = static_cast<const Entry *>(table);
     if constexpr (TAB_SMEM) {
         Entry *s_tab = reinterpret_cast<Entry *>(smem + W * warp_bytes);
         for (uint32_t i = threadIdx.x; i < a.tab_len; i += W * 32) s_tab[i] = tab[i];
@@ -201,7 +211,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
         fence_mbar_init();
         for (int s = 0; s < S; ++s) {
             const uint64_t t = gw + (uint64_t)s * tw;
-            if (t < a.ntiles) issue_tile<SB>(a, t, wbase + s * Geom::stage_stride, &bar[s]);
+            if (t < a.ntiles) issue_tile<SB>(a, in, t, wbase + s * Geom::stage_stride, &bar[s]);
         }
     }
     __syncwarp();
@@ -230,7 +240,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             const uint64_t w0 = byte0 >> 2, wb = (byte0 + bytes) >> 2;
             const uint64_t we = min(((c0 + gcnt) * n + 31) >> 5, a.in_words);
             if (wb < we) {
-                for (uint64_t w = wb + lane; w < we; w += 32) st[w - w0] = a.in[w];
+                for (uint64_t w = wb + lane; w < we; w += 32) st[w - w0] = in[w];
                 __syncwarp();
             }
         }
@@ -300,18 +310,18 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             else
                 for (uint32_t o = T >> 1; o > 0; o >>= 1) z ^= __shfl_xor_sync(0xFFFFFFFFu, z, o);
             if (tl == 0 && c < gcnt) {
-                const uint32_t syn = (z >> 17) << 5 | ((z >> 1) & 3u) | ((z >> 2) & 4u) | ((z >> 5) & 8u) | ((z >> 12) & 16u);
-                if (syn != 0) {
+                const uint32_t sv = (z >> 17) << 5 | ((z >> 1) & 3u) | ((z >> 2) & 4u) | ((z >> 5) & 8u) | ((z >> 12) & 16u);
+                if (sv != 0) {
                     ++errs;
-                    if (syn <= n) {
-                        const uint32_t b = off0 + c * n + syn - 1u;
+                    if (sv <= n) {
+                        const uint32_t b = off0 + c * n + sv - 1u;
                         atomicXor(&st[b >> 5], 1u << (b & 31u));
                     } else {
                         ++dets;
                     }
                 }
-                if (a.syn_type == 1) static_cast<uint8_t *>(a.syn)[c0 + c] = (uint8_t)syn;
-                if (a.syn_type == 2) static_cast<uint16_t *>(a.syn)[c0 + c] = (uint16_t)syn;
+                if (a.syn_type == 1) static_cast<uint8_t *>(syn)[c0 + c] = (uint8_t)sv;
+                if (a.syn_type == 2) static_cast<uint16_t *>(syn)[c0 + c] = (uint16_t)sv;
             }
         }
         __syncwarp();
@@ -334,7 +344,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             const int32_t idx0 = (int32_t)((cr * k) >> 5) + lane;
             int32_t sbw = (int32_t)off0 - (int32_t)(cr * n) + 32 * idx0;
             const Entry *tp = tab + idx0;
-            uint32_t *outp = a.out + F + lane;
+            uint32_t *outp = out + F + lane;
             // four words per lane per iteration, 32 apart.  Words past the tile come from
             // in-range entries and clamped stage bits and are never stored.
             for (int32_t w0 = lane; w0 <= whi; w0 += 128, outp += 128, tp += 128, sbw += 4096) {
@@ -382,7 +392,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             const uint32_t al = b & 31u;
             const uint32_t cb = off0 + c * n;  // stage bit of position 1
             const uint32_t head = head_word(st, cb);
-            uint32_t *o = a.out + F + ws;
+            uint32_t *o = out + F + ws;
             if (c == 0 && fs) {
                 const uint32_t own = ~lowmask(al), v = head << al;
                 atomicAnd(o, v | ~own);
@@ -402,7 +412,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             if (c == gcnt - 1 && (ob1 & 31u) != 0) {
                 const uint32_t rem = (uint32_t)(ob1 & 31u);
                 const uint32_t v = run_word(st, cb, k - rem) & lowmask(rem);
-                uint32_t *ol = a.out + L;
+                uint32_t *ol = out + L;
                 if (ls) {
                     atomicAnd(ol, v | ~lowmask(rem));
                     atomicOr(ol, v);
@@ -418,14 +428,14 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             const uint32_t b0 = (uint32_t)(ob0 & 31u) + c * k;   // tile bit of the codeword's data bit 0
             const uint32_t bd = b0 + (2u << J) - J - 2u;          // tile bit of data bit D_J
             const uint32_t dw = (bd & ~31u) - b0;                 // data bit at the start of its word (>= 26)
-            if ((bd & 31u) != 0 && dw + 32u <= k) a.out[F + (bd >> 5)] = run_word(st, off0 + c * n, dw);
+            if ((bd & 31u) != 0 && dw + 32u <= k) out[F + (bd >> 5)] = run_word(st, off0 + c * n, dw);
         }
         // the corrections wrote the stage through the generic proxy; the refill writes it through the async one
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
             const uint64_t tn = t + (uint64_t)S * tw;
-            if (tn < a.ntiles) issue_tile<SB>(a, tn, stage, &bar[s]);
+            if (tn < a.ntiles) issue_tile<SB>(a, in, tn, stage, &bar[s]);
         }
         __syncwarp();
     }
@@ -436,7 +446,7 @@ __global__ void __launch_bounds__(W * 32) k_short_tiles(ShortArgs a)
             if (tj < a.ntiles) (void)mbar_wait_bounded(&bar[j % S], (j / S) & 1u);
         }
     }
-    add_counts(a.direct, a.err, a.det, errs, dets, reinterpret_cast<uint32_t *>(smem), warp_bytes / 4);
+    add_counts(a.direct, err, det, errs, dets, reinterpret_cast<uint32_t *>(smem), warp_bytes / 4);
 }
 
 // ---------------------------------------------------------------------------
@@ -552,14 +562,14 @@ struct ShortVariant {
     uint32_t stage_smem;  // dynamic shared memory of the warps' stages
     // [0]: table in global memory; [1]: table in shared memory; [2]: shared, splits in pass 3
     const void *kernel[3];
-    cudaError_t (*launch[3])(const ShortArgs &, int grid, uint32_t smem, cudaStream_t, bool pdl);
+    cudaError_t (*launch[3])(const ShortBuffers &, const ShortArgs &, int grid, uint32_t smem, cudaStream_t, bool pdl);
 };
 
 template <int W, int S, int SB, bool TAB_SMEM, bool SPLIT>
-cudaError_t launch_tiles(const ShortArgs &a, int grid, uint32_t smem, cudaStream_t st, bool pdl)
+cudaError_t launch_tiles(const ShortBuffers &b, const ShortArgs &a, int grid, uint32_t smem, cudaStream_t st, bool pdl)
 {
     return launch_kernel(k_short_tiles<W, S, SB, TAB_SMEM, SPLIT>, dim3((unsigned)grid), dim3(W * 32), smem, st, pdl,
-                         a);
+                         b.in, b.out, b.syn, b.err, b.det, b.table, a);
 }
 
 template <int W, int S, int SB>
@@ -863,11 +873,7 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     const ShortVariant &v = kShortVariants[vi];
     const uint32_t r = short_r(n), k = n - r;
     ShortArgs a{};
-    a.in = in;
-    a.out = out;
-    a.syn = syn;
-    a.err = err;
-    a.det = det;
+    const ShortBuffers buf{in, out, syn, err, det, table};
     a.status = status_ptr();
     if (!a.status) return cudaErrorUnknown;
     a.num_cw = num_cw;
@@ -880,9 +886,8 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     a.Y = (n + 32) / 32;
     const uint32_t lastbits = n + 1 - 32 * (a.Y - 1);
     a.ylast = lastbits >= 32 ? 0xFFFFFFFFu : (1u << lastbits) - 1u;
-    a.table = table;
     a.tab_len = tab_len;
-    if (!a.table) return cudaErrorInvalidValue;
+    if (!table) return cudaErrorInvalidValue;
     a.syn_type = syn ? syn_type : 0;
     a.nJ = 0;
     for (uint32_t J = 5; (2u << J) - J - 2u < k; ++J) ++a.nJ;
@@ -904,7 +909,7 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     a.tlog = team_log(a.Y, a.g);
     const int grid = decode_grid((a.ntiles + v.W - 1) / v.W, cap);
     return launch_counted(a.direct, err, det, grid, bare, st, [&](bool pdl) {
-        return v.launch[tsm](a, grid, smem, st, pdl);
+        return v.launch[tsm](buf, a, grid, smem, st, pdl);
     });
 }
 

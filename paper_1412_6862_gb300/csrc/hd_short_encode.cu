@@ -35,8 +35,6 @@ constexpr uint32_t kAreaWords = 1056;  // position-domain words a warp holds: n 
 constexpr uint32_t kMaxTile = 256;     // segments per tile
 
 struct EncShortArgs {
-    const uint32_t *data;
-    uint32_t *stream;
     uint64_t data_words, num_cw, ntiles;
     uint32_t *status;
     uint32_t n, k, g;          // segment length, message bits, segments per tile
@@ -130,7 +128,7 @@ __device__ __forceinline__ void fold_segment(const uint32_t *st, int32_t bit0, u
 
 // TLOG: log2 of the team size, so that a lane's word strides are constants.
 template <int TLOG>
-__global__ void __launch_bounds__(kWarps * 32) k_encode_short(const EncShortArgs a)
+__global__ void __launch_bounds__(kWarps * 32) k_encode_short(const uint32_t *__restrict__ data, uint32_t *__restrict__ stream, const EncShortArgs a)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -158,7 +156,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_encode_short(const EncShortArgs
         uint32_t bytes;
         span(t, byte0, bytes);
         mbar_arrive_expect_tx(bar, bytes);
-        if (bytes) bulk_g2s(stage, reinterpret_cast<const uint8_t *>(a.data) + byte0, bytes, bar);
+        if (bytes) bulk_g2s(stage, reinterpret_cast<const uint8_t *>(data) + byte0, bytes, bar);
     };
     const uint64_t tw = (uint64_t)gridDim.x * kWarps;
     uint64_t t = (uint64_t)blockIdx.x * kWarps + warp;
@@ -188,7 +186,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_encode_short(const EncShortArgs
             span(t, byte0, bytes);
             const uint64_t w0 = byte0 >> 2, wb = (byte0 + bytes) >> 2, we = ((c0 + gcnt) * k + 31) >> 5;
             if (wb < we) {
-                for (uint64_t w = wb + lane; w < we; w += 32) stage[w - w0] = a.data[w];
+                for (uint64_t w = wb + lane; w < we; w += 32) stage[w - w0] = data[w];
                 __syncwarp();
             }
         }
@@ -227,7 +225,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_encode_short(const EncShortArgs
         // pass 2: stream words, counted from the word holding the tile's first bit.  Segment c
         // covers the tile's bits [s, s + n), s = ob + c * n.
         const uint32_t ob = (uint32_t)bit_out & 31u;
-        uint32_t *out = a.stream + (bit_out >> 5);
+        uint32_t *out = stream + (bit_out >> 5);
         const bool last_tile = c0 + gcnt == a.num_cw;
         // words inside one segment: the shift is the segment's own
         for (uint32_t c = team; c < gcnt; c += G) {
@@ -281,8 +279,6 @@ cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, ui
                                 cudaStream_t st)
 {
     EncShortArgs a{};
-    a.data = data;
-    a.stream = stream;
     a.data_words = words_for_bits(num_cw * k);
     a.num_cw = num_cw;
     a.status = status_ptr();
@@ -293,7 +289,7 @@ cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, ui
     a.ylast = n % 32 == 31 ? 0xFFFFFFFFu : (2u << (n % 32)) - 1u;
     a.ystride = (a.Y + 1) | 1u;
     constexpr uint32_t smem = kWarps * kWarpBytes;
-    static void (*const kernels[6])(EncShortArgs) = {k_encode_short<0>, k_encode_short<1>, k_encode_short<2>,
+    static void (*const kernels[6])(const uint32_t *, uint32_t *, EncShortArgs) = {k_encode_short<0>, k_encode_short<1>, k_encode_short<2>,
                                                      k_encode_short<3>, k_encode_short<4>, k_encode_short<5>};
     // segments per tile: what the area holds, evened out so that every warp of a full
     // GPU (3 CTAs an SM) takes as many tiles (40,001 segments of n = 3212: tiles of 10
@@ -323,7 +319,8 @@ cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, ui
     if (bps <= 0) return cudaErrorInvalidConfiguration;
     a.ntiles = (num_cw + a.g - 1) / a.g;
     const int grid = decode_grid((a.ntiles + kWarps - 1) / kWarps, (uint64_t)num_sms() * (uint64_t)bps);
-    return launch_kernel(kernels[tlog], dim3((unsigned)grid), dim3(kWarps * 32), smem, st, true, a);
+    return launch_kernel(kernels[tlog], dim3((unsigned)grid), dim3(kWarps * 32), smem, st, true, data,
+                         stream, a);
 }
 
 }  // namespace hd

@@ -194,11 +194,12 @@ __device__ __forceinline__ void issue_chunk(const uint32_t *in, uint64_t c, uint
 }
 
 // The ragged tail's tiles t0, t0 + step, ... of a stream; returns the nonzero
-// syndromes | detected ones << 16 (a tail has at most 1024 codewords).  Out of line
-// from n = 63 up: the kernel's loop then keeps the registers it has without a tail
-// (SECDED n = 63, 2^24 codewords: 50.0 us against 51.9 inline; n = 127: 26.7 against
-// 27.4); the short codes' loops are better with it inline (n = 31, 20,000,003
-// codewords: 33.5 us against 34.5).
+// syndromes | detected ones << 16 (a tail has at most 1024 codewords).  Where the
+// kernels have it decides how well their loops compile, measured on GB300 at 2^24
+// (n = 127: 2^22) codewords: out of line and first from n = 63 up (SECDED n = 63
+// 50.0 us against 51.9 inline, SECDED n = 127 with u8 syndromes 24.4 against 25.3
+// after the loop); after the loop for the short codes (n = 7, u16 syndromes, 2^26
+// codewords: 43 us, 61 with it first), out of line with a decode table.
 template <int N_, int SYN, bool XH>
 __device__ __forceinline__ uint32_t tail_tiles(const uint32_t *in, uint64_t in_words, uint64_t num_cw, uint64_t t0,
                                                uint64_t t1, uint64_t step, uint32_t *out, uint64_t out_words,
@@ -218,15 +219,33 @@ __device__ __noinline__ uint32_t tail_tiles_call(const uint32_t *in, uint64_t in
     return tail_tiles<N_, SYN, XH>(in, in_words, num_cw, t0, t1, step, out, out_words, syn, slots, lane);
 }
 
-template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH = false, bool LUT = false>
-__global__ void __launch_bounds__(T)
-    k_decode_stream(const StreamArgs args)
+// The CTAs per SM a kernel's registers are chosen for: 0 leaves it to the compiler,
+// 1 asks for no more than the shared memory allows anyway, which lets the loop of
+// the kernels listed here keep more loads ahead (SECDED n = 31 / 127 at 2^24 / 2^22
+// codewords with u16 syndromes 27.3 / 24.1 us against 31.0 / 25.4); others lose by
+// it (n = 63 in place 48.1 us against 44.4).
+constexpr int min_ctas(int n, bool inplace, bool xh) { return (xh && n >= 31) || (n == 63 && !inplace) ? 1 : 0; }
+
+// TAIL: the stream may have a ragged tail.  The built-in table kernels and the n = 255
+// one have a second form without it, for whole chunks, whose loops the tail's code
+// costs up to 3 % (n = 7, 2^26 codewords without syndromes 26.9 us against 26.3, n = 15
+// 12.75 against 12.6, SECDED n = 15 18.2 against 17.9).
+constexpr bool has_tailless(int n, bool lut, int T, int S)
 {
+    return lut ? n == 7 || (S == 2 && (T == 512 || T == 576)) : n == 255 && T == 128 && S == 2;
+}
+
+template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH = false, bool LUT = false, bool TAIL = true>
+__global__ void __launch_bounds__(T, min_ctas(N_, INPLACE != 0, XH))
+    k_decode_stream(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, uint8_t *__restrict__ syn,
+                    unsigned long long *__restrict__ err, uint32_t *__restrict__ status, uint64_t nchunks,
+                    unsigned long long *__restrict__ det, const uint16_t *__restrict__ lut, uint64_t num_cw,
+                    uint64_t in_words, uint64_t out_words, uint64_t tile_begin, uint64_t tile_end)
+{
+    // pointers as parameters of their own: the compiler then knows them for global
+    // memory (members of a struct are generic, and a generic store of syndromes may
+    // alias the decode table in shared memory: n = 7 with u16 syndromes 59 us against 44)
     using Cfg = StreamCfg<N_, SYN, T, S, G, INPLACE, XH, LUT>;
-    const uint32_t *__restrict__ in = args.in;
-    uint32_t *__restrict__ out = args.out;
-    uint8_t *__restrict__ syn = static_cast<uint8_t *>(args.syn);
-    const uint64_t nchunks = args.nchunks;
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // Programmatic dependent launch, both ways: the next kernel of the stream
@@ -249,7 +268,7 @@ __global__ void __launch_bounds__(T)
             static_assert(Cfg::lut_bytes % piece == 0, "whole pieces");
 #pragma unroll
             for (uint32_t o = 0; o < Cfg::lut_bytes; o += piece)
-                bulk_g2s(smem + Cfg::off_lut + o, reinterpret_cast<const uint8_t *>(args.lut) + o, piece, lut_bar);
+                bulk_g2s(smem + Cfg::off_lut + o, reinterpret_cast<const uint8_t *>(lut) + o, piece, lut_bar);
         }
         __syncthreads();  // the barrier is initialised before any thread waits on it
     }
@@ -263,23 +282,25 @@ __global__ void __launch_bounds__(T)
 
     uint32_t errs = 0, dets = 0;  // this lane's counts
     // The ragged tail's tiles, one codeword per lane, by the grid's last warps (which
-    // hold the fewest chunks) before their first chunk: a launch of its own for them
-    // cost 4 to 5 us, the GPU drained on both sides of it.
-    if (args.tile_begin < args.tile_end) {
+    // hold the fewest chunks): a launch of its own for them cost 4 to 5 us, the GPU
+    // drained on both sides of it.
+    auto tail = [&]() {
         static_assert(Cfg::warp_bytes - Cfg::off_in >= 32u * kLaneDataSlot<N_> * 4u, "a tile's merge area");
-        const uint64_t t0 = args.tile_begin + (tw - 1 - gw);
+        const uint64_t t0 = tile_begin + (tw - 1 - gw);
         uint32_t *slots = reinterpret_cast<uint32_t *>(s_in);
         uint32_t c;
-        if constexpr (N_ >= 63)
-            c = tail_tiles_call<N_, SYN, XH>(in, args.in_words, args.num_cw, t0, args.tile_end, tw, out,
-                                             args.out_words, syn, slots, lane);
+        if constexpr (N_ >= 63 || LUT)
+            c = tail_tiles_call<N_, SYN, XH>(in, in_words, num_cw, t0, tile_end, tw, out, out_words, syn, slots, lane);
         else
-            c = tail_tiles<N_, SYN, XH>(in, args.in_words, args.num_cw, t0, args.tile_end, tw, out, args.out_words,
-                                        syn, slots, lane);
+            c = tail_tiles<N_, SYN, XH>(in, in_words, num_cw, t0, tile_end, tw, out, out_words, syn, slots, lane);
         if (lane == 0) {
-            errs = c & 0xFFFFu;
-            dets = c >> 16;
+            errs += c & 0xFFFFu;
+            dets += c >> 16;
         }
+    };
+    constexpr bool kTailFirst = N_ >= 63 || (XH && N_ == 31);
+    if (TAIL && kTailFirst && tile_begin < tile_end) {
+        tail();
         fence_proxy_async_smem();  // the tiles used the ring that the copies below fill
         __syncwarp();
     }
@@ -391,7 +412,7 @@ __global__ void __launch_bounds__(T)
     }
     if (lane == 0) {
         if (aborted) {
-            atomicOr(args.status, (uint32_t)HD_ERR_TIMEOUT);
+            atomicOr(status, (uint32_t)HD_ERR_TIMEOUT);
             // wait (bounded) for every load still in flight into this warp's ring
             // (after the first iteration in-place refills lag one iteration, so
             // one fewer is outstanding) and for the table
@@ -404,6 +425,10 @@ __global__ void __launch_bounds__(T)
         }
         bulk_wait_all<0>();
     }
+    if (TAIL && !kTailFirst && tile_begin < tile_end) {
+        __syncwarp();  // lane 0 has waited for the stores that read the ring
+        tail();
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) errs += __shfl_xor_sync(0xFFFFFFFFu, errs, o);
     if constexpr (XH) {
@@ -411,8 +436,8 @@ __global__ void __launch_bounds__(T)
         for (int o = 16; o > 0; o >>= 1) dets += __shfl_xor_sync(0xFFFFFFFFu, dets, o);
     }
     if (lane == 0) {
-        if (args.err != nullptr && errs != 0) atomicAdd(args.err, (unsigned long long)errs);
-        if (XH && args.det != nullptr && dets != 0) atomicAdd(args.det, (unsigned long long)dets);
+        if (err != nullptr && errs != 0) atomicAdd(err, (unsigned long long)errs);
+        if (XH && det != nullptr && dets != 0) atomicAdd(det, (unsigned long long)dets);
     }
 }
 
@@ -422,6 +447,8 @@ cudaError_t launch_stream_variant(const StreamArgs &a, cudaStream_t st, bool pdl
     using Cfg = StreamCfg<N_, SYN, T, S, G, INPLACE, XH, LUT>;
     if (LUT && a.lut == nullptr) return cudaErrorInvalidValue;
     auto kern = k_decode_stream<N_, SYN, T, S, G, INPLACE, XH, LUT>;
+    if constexpr (has_tailless(N_, LUT, T, S))
+        if (a.tile_begin == a.tile_end) kern = k_decode_stream<N_, SYN, T, S, G, INPLACE, XH, LUT, false>;
     const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kern), T, Cfg::smem);
     if (bps <= 0) return cudaErrorInvalidConfiguration;
     const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
@@ -430,7 +457,9 @@ cudaError_t launch_stream_variant(const StreamArgs &a, cudaStream_t st, bool pdl
     // with pdl the launch may overlap the kernel ahead of it (the counters'
     // clear, or a decode's drain); the kernel waits for it before its first
     // access to global memory
-    return launch_kernel(kern, dim3((unsigned)grid), dim3(T), Cfg::smem, st, pdl, a);
+    return launch_kernel(kern, dim3((unsigned)grid), dim3(T), Cfg::smem, st, pdl, a.in, a.out,
+                         static_cast<uint8_t *>(a.syn), a.err, a.status, a.nchunks, a.det, a.lut, a.num_cw, a.in_words,
+                         a.out_words, a.tile_begin, a.tile_end);
 }
 
 template <int N_, int SYN, int T, int S, int G, int INPLACE, bool XH = false, bool LUT = false>

@@ -68,6 +68,61 @@ __device__ __forceinline__ uint32_t compress_runs(uint32_t y)
     return d;
 }
 
+// ---------------------------------------------------------------------------
+// Checksum bits by a superset XOR transform.  After the steps for the index
+// bits 0 .. M-1, bit j of the result is the XOR of the bits of y whose index
+// contains j (as a bit set), so bit 2^b is the parity of index set I_b: every
+// checksum bit lands on its own position.  Two operations a step (a shift and
+// one lop3) against a mask, a popcount and a gather per bit; and for codes
+// shorter than a word the same steps serve several codewords side by side.
+// ---------------------------------------------------------------------------
+template <int M>
+__device__ __forceinline__ uint32_t superset_xor(uint32_t y)
+{
+    y ^= (y >> 1) & 0x55555555u;
+    if constexpr (M >= 2) y ^= (y >> 2) & 0x33333333u;
+    if constexpr (M >= 3) y ^= (y >> 4) & 0x0F0F0F0Fu;
+    if constexpr (M >= 4) y ^= (y >> 8) & 0x00FF00FFu;
+    if constexpr (M >= 5) y ^= y >> 16;
+    return y;
+}
+
+// Redundancy removal within a position-domain word as compress_runs<5>, but
+// with the 26 data bits at the top (bits 6..31) and whatever was there below:
+// the lower runs move up (run 3 by 1, run 2 by 2, run 1 by 3, in two binary
+// steps) and run 4 stays, so the shifts are multiplications beside the logic
+// operations and the shift by 3 falls away (two logic operations a word against
+// five; OutPacker::append_top masks the rest).
+__device__ __forceinline__ uint32_t compress_runs_top(uint32_t y)
+{
+    const uint32_t a = bitsel(~0x0001FC10u, y, fma_lo(y, 2u, 0u));  // runs 3, 1 to 10..16, 4
+    return bitsel(~0x000003C0u, a, fma_lo(a, 4u, 0u));             // runs 2, 1 to 7..9, 6
+}
+
+// The syndromes of four codewords at once, one byte each.  f[c] is the XOR of
+// codeword c's position-domain words.  Halves, then bytes of the four are packed
+// side by side and folded, so that each fold and transform step serves all
+// four: 8.5 operations a codeword and no popcounts, where masked popcounts and
+// their gather took 17 (5 of them popcounts, at half the logic operations' rate).
+// Byte c of the result: s0..s4 of f[c]; par: the parity of f[c] on bit 0 of byte
+// c, other bits undefined.
+__device__ __forceinline__ uint32_t quad_syndromes(const uint32_t (&f)[4], uint32_t &par)
+{
+    const uint32_t hab = __byte_perm(f[0], f[1], 0x7632), pab = __byte_perm(f[0], f[1], 0x5410) ^ hab;
+    const uint32_t hcd = __byte_perm(f[2], f[3], 0x7632), pcd = __byte_perm(f[2], f[3], 0x5410) ^ hcd;
+    const uint32_t qh = __byte_perm(pab, pcd, 0x7531);               // folded to 16 bits: the high bytes (bit 3)
+    const uint32_t q = superset_xor<3>(__byte_perm(pab, pcd, 0x6420) ^ qh);  // to 8 bits: bits 0..2
+    const uint32_t h = __byte_perm(hab, hcd, 0x7531) ^ __byte_perm(hab, hcd, 0x6420);  // the high halves (bit 4)
+    // parities of qh and h, four bits each in a byte, folded together
+    uint32_t p = bitsel(0x0F0F0F0Fu, qh ^ (qh >> 4), h ^ fma_lo(h, 16u, 0u));
+    p ^= p >> 2;
+    p ^= p >> 1;
+    par = q;
+    const uint32_t lo = bitsel(0x03030303u, q >> 1, q >> 2);             // bits 1, 2, 4 of q to 0, 1, 2
+    const uint32_t hi = bitsel(0x08080808u, fma_lo(p, 8u, 0u), p);       // bits 0, 4 of p to 3, 4
+    return bitsel(0x07070707u, lo, hi) & 0x1F1F1F1Fu;
+}
+
 // Syndrome gather for codes whose m checksum bits come from one 32-bit word:
 // the parity counts are summed into fields of F bits, the field LSBs kept, and
 // one multiply moves LSB j (bit F*j) to bit 32-m+j.  All partial products land
@@ -175,6 +230,21 @@ struct OutPacker {
         }
     }
 
+    // As append(), of the top `len` bits of v; the bits below them are ignored.
+    __device__ __forceinline__ void append_top(uint32_t v, int len)
+    {
+        const int up = pos - (32 - len);  // the piece's move, left when positive
+        const uint32_t w = up > 0 ? fma_lo(v, 1u << (up & 31), 0u) : v >> (-up & 31);
+        acc = pos == 0 ? w : bitsel((1u << (pos & 31)) - 1u, acc, w);
+        if (pos + len >= 32) {
+            emit(acc);
+            acc = up > 0 ? v >> ((32 - up) & 31) : 0u;
+            pos = pos + len - 32;
+        } else {
+            pos += len;
+        }
+    }
+
     // Flush the last partial local word and the spill into the next word.
     __device__ __forceinline__ void finish()
     {
@@ -212,27 +282,45 @@ struct SynPacker {
             w = s;
         else
             w = fma_lo(s, 1u << (slot * 8 * SB), w);  // w | (s << lane offset)
-        if (slot == PER - 1) {
-            if constexpr (!WIDE) {
-                // a lane is nonzero iff adding 0x7F..F carries into its top bit
-                if constexpr (SB == 1)
-                    cnt = fma_lo(__popc(fma_lo(w, 1u, 0x7F7F7F7Fu) & 0x80808080u), 1u, cnt);
+        if (slot == PER - 1) flush(c);
+    }
+
+    // The packed word w that ends with syndrome c is complete.
+    __device__ __forceinline__ void flush(int c)
+    {
+        if constexpr (!WIDE) {
+            // a lane is nonzero iff adding 0x7F..F carries into its top bit
+            if constexpr (SB == 1)
+                cnt = fma_lo(__popc(fma_lo(w, 1u, 0x7F7F7F7Fu) & 0x80808080u), 1u, cnt);
+            else
+                cnt = fma_lo(__popc(fma_lo(w, 1u, 0x7FFF7FFFu) & 0x80008000u), 1u, cnt);
+        }
+        if constexpr (STORE) {
+            const int wi = c / PER;  // word index within the part
+            pend.set(wi % VEC, w);
+            if (wi % VEC == VEC - 1) {
+                uint8_t *p = dst + 4 * (wi - (VEC - 1));
+                if constexpr (VEC == 4)
+                    *reinterpret_cast<uint4 *>(p) = make_uint4(pend.p0, pend.p1, pend.p2, pend.p3);
+                else if constexpr (VEC == 2)
+                    *reinterpret_cast<uint2 *>(p) = make_uint2(pend.p0, pend.p1);
                 else
-                    cnt = fma_lo(__popc(fma_lo(w, 1u, 0x7FFF7FFFu) & 0x80008000u), 1u, cnt);
+                    *reinterpret_cast<uint32_t *>(p) = pend.p0;
             }
-            if constexpr (STORE) {
-                const int wi = c / PER;  // word index within the part
-                pend.set(wi % VEC, w);
-                if (wi % VEC == VEC - 1) {
-                    uint8_t *p = dst + 4 * (wi - (VEC - 1));
-                    if constexpr (VEC == 4)
-                        *reinterpret_cast<uint4 *>(p) = make_uint4(pend.p0, pend.p1, pend.p2, pend.p3);
-                    else if constexpr (VEC == 2)
-                        *reinterpret_cast<uint2 *>(p) = make_uint2(pend.p0, pend.p1);
-                    else
-                        *reinterpret_cast<uint32_t *>(p) = pend.p0;
-                }
-            }
+        }
+    }
+
+    // Four syndromes c .. c + 3 (c a multiple of 4), a byte each.
+    __device__ __forceinline__ void put4(int c, uint32_t s)
+    {
+        if constexpr (SB == 1) {
+            w = s;
+            flush(c + 3);
+        } else {
+            w = __byte_perm(s, 0u, 0x4140);
+            flush(c + 1);
+            w = __byte_perm(s, 0u, 0x4342);
+            flush(c + 3);
         }
     }
 
@@ -342,6 +430,50 @@ __device__ __forceinline__ void decode_part(const uint32_t (&r)[R], OP &op, SP &
             const uint32_t sv = e[c] >> C::k;  // s, or for SECDED s | P << m
             if constexpr (XH) det += (sv - 1u < (1u << C::m) - 1u) ? 1u : 0u;  // P = 0 and s != 0
             sp.put(c, sv);
+        }
+    } else if constexpr (N_ == 31 || (N_ == 63 && XH)) {
+        // four codewords at a time (quad_syndromes)
+        static_assert(G % 4 == 0, "whole quads");
+#pragma unroll
+        for (int c = 0; c < G; c += 4) {
+            uint32_t y[4][C::Wy], f[4], par;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                for (int w = 0; w < C::Wy; ++w) y[i][w] = XH ? part_y_xh<N_, R>(r, c + i, w) : part_y<N_, R>(r, c + i, w);
+                f[i] = C::Wy == 1 ? y[i][0] : y[i][0] ^ y[i][C::Wy - 1];
+            }
+            uint32_t s = quad_syndromes(f, par);
+            if constexpr (N_ == 63) {
+                // bit 5: the parity of the second word, from popcounts summed into byte fields
+                uint32_t p5 = __popc(y[0][1]);
+#pragma unroll
+                for (int i = 1; i < 4; ++i) p5 = fma_lo(__popc(y[i][1]), 1u << (8 * i), p5);
+                s = fma_lo(p5 & 0x01010101u, 32u, s);
+            }
+            uint32_t val = s, odd = 0;
+            if constexpr (XH) {
+                odd = par & 0x01010101u;  // overall parity; even with s != 0 is a detected double error
+                val = fma_lo(odd, 1u << C::m, s);
+                det += __popc((s + 0x7F7F7F7Fu) & ~fma_lo(odd, 128u, 0u) & 0x80808080u);
+            }
+            sp.put4(c, val);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                // flip position s of codeword i (XH: when its overall parity is odd); the wrapping
+                // shift reads the low five bits of the byte
+                const uint32_t si = s >> (8 * i);
+                const uint32_t bit = __funnelshift_l(0u, XH ? (odd >> (8 * i)) & 1u : 1u, si);
+                if constexpr (C::Wy == 1) {
+                    y[i][0] ^= bit;
+                } else {
+                    const uint32_t second = 0u - ((si >> 5) & 1u);
+                    y[i][0] ^= bit & ~second;
+                    y[i][1] ^= bit & second;
+                }
+                op.append_top(compress_runs_top(y[i][0]), 26);
+                if constexpr (C::Wy == 2) op.append(y[i][1] >> 1, 31);  // position 32 is a checksum position
+            }
         }
     } else {
 #pragma unroll
