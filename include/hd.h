@@ -86,10 +86,11 @@ hd_status hd_decode(const uint32_t *stream, uint64_t in_bits, uint32_t n, uint64
 /* Several independent streams decoded concurrently.  Each job is one
  * hd_decode() call (arguments, layout, results and errors as there, with
  * in_bits = n * num_codewords).  The jobs' counters are cleared by one kernel
- * on `cuda_stream`, then the decodes run as concurrent branches forked from
- * `cuda_stream` onto library-owned streams (8 per device, created by the
- * first call on a device, which should come before any stream capture) and
- * joined back into it, largest stream first: work enqueued on `cuda_stream`
+ * on `cuda_stream`, then the decodes run as concurrent branches, the largest
+ * on `cuda_stream` itself, the others forked from it onto library-owned
+ * streams (8 per device, created by the first call on a device, which should
+ * come before any stream capture) and joined back into it, the short ones one
+ * behind another in a branch of their own: work enqueued on `cuda_stream`
  * after this call waits for every job.  Decoding the streams side by side lets
  * one decode's ramp-up and drain overlap another's steady state, the
  * pipelining of independent packets the paper applies to its transfers
@@ -109,7 +110,8 @@ hd_status hd_decode_streams(const hd_stream_job *jobs, uint32_t num_jobs, void *
 
 /* Decode from and to HOST memory with overlapped transfers -- the paper's
  * asynchronous data transfer (Sec. III-B, Fig. 5, Eq. 1).  The stream is cut
- * into chunks of `chunk_codewords` (a multiple of 128; 0 = 2^22) and each
+ * into chunks of `chunk_codewords` (a multiple of 128; 0 = 2^22, and four pieces of
+ * a stream that would be one chunk of 24 MB of copies or more) and each
  * chunk's host-to-device copy, decode and device-to-host copy run on one of
  * `depth` CUDA streams (0 = 4, at most 8), so copies in both directions
  * overlap with the decoding of neighbouring chunks.  Arguments and results are
@@ -358,7 +360,8 @@ typedef struct {
  * A plan is not thread-safe: launch it from one host thread at a time. */
 typedef struct hd_plan hd_plan;
 
-/* A plan decodes with one of num_variants configurations: variants
+/* A plan decodes with one of num_variants configurations, chosen by its size
+ * and code lengths until it is tuned or one is selected: variants
  * 0 .. num_variants - 3 launch one persistent kernel that decodes tiles of
  * every n; variant num_variants - 2 (the split configuration) launches one
  * kernel per code length present, each compiled for that n alone, as

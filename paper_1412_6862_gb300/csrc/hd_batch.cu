@@ -11,19 +11,20 @@
 // dealt round-robin by the single-n kernels), prefetch their tiles into its own shared-memory stages with 1-D bulk copies,
 // decodes full tiles with the same per-warp chunk decoder as the streaming
 // kernel, decodes tails with the chunk decoder too (copied in, zero-padded to a
-// chunk, copied back out; n = 3 tails use the generic warp-tile decoder), and
+// chunk, copied back out; n = 3 one codeword per lane), and
 // adds each tile's nonzero-syndrome count to its packet's error counter.
 // Cutting packets whose lengths span six orders of magnitude into bounded
 // tiles is what balances the load.
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <vector>
 
 #include "hd_batch_internal.h"
-#include "hd_generic.cuh"
 #include "hd_internal.h"
+#include "hd_lane.cuh"
 #include "hd_multi.cuh"
 #include "hd_stream.cuh"
 
@@ -99,13 +100,15 @@ struct PacketView {
     uint8_t *syn;
     uint64_t num_cw;
     uint32_t n, m, syn_type;
+    uint32_t index;  // in the packet table
 };
 
 // Emit the tiles of every packet of code length n, without allocating: full
 // tiles in packet order, with the packets' ragged tails spread evenly among
 // them (after each full tile, tails until their share matches), so that the
 // latency-bound tails overlap the streaming of full tiles instead of running
-// as a phase of their own.  view(i) describes packet i; emit(tile) takes a tile.
+// as a phase of their own.  view(i), i < num_packets, describes a packet (packets of
+// other lengths are skipped); emit(tile) takes a tile.
 template <class View, class Emit>
 void emit_code_tiles(uint32_t n, uint32_t num_packets, View view, Emit emit, bool big = false)
 {
@@ -134,7 +137,7 @@ void emit_code_tiles(uint32_t n, uint32_t num_packets, View view, Emit emit, boo
                 // so 16-byte aligned); the last words are loaded when it is decoded
                 const uint32_t cnt = (uint32_t)std::min<uint64_t>(kTailTile, p.num_cw - tc);
                 const uint32_t bulk = n == 3 ? 0u : (uint32_t)(((uint64_t)cnt * n + 31) / 32 * 4) & ~15u;
-                emit(make_tile(p.in, p.out, p.syn, p.num_cw, n, p.m, p.syn_type, ti, tc, cnt, bulk));
+                emit(make_tile(p.in, p.out, p.syn, p.num_cw, n, p.m, p.syn_type, p.index, tc, cnt, bulk));
                 tc += kTailTile;
                 return true;
             }
@@ -148,7 +151,7 @@ void emit_code_tiles(uint32_t n, uint32_t num_packets, View view, Emit emit, boo
         const uint64_t f = nfull_of(p);
         for (uint64_t j = 0; j < f; j += per) {
             const uint64_t c = std::min(per, f - j);
-            emit(make_tile(p.in, p.out, p.syn, p.num_cw, n, p.m, p.syn_type, i, j * chunk,
+            emit(make_tile(p.in, p.out, p.syn, p.num_cw, n, p.m, p.syn_type, p.index, j * chunk,
                            (uint32_t)(c * chunk) | kFullTile, (uint32_t)(c * chunk * n / 8)));
             ++done_full;
             while (done_tail * nf < done_full * nt && next_tail()) ++done_tail;
@@ -184,7 +187,7 @@ struct BatchCfg {
     static constexpr uint32_t off_lut_bar = off_lut15 + lut15_bytes;
     static constexpr uint32_t smem = off_lut_bar + 16;
     static_assert(S >= 2 && S <= 8, "refills lag one iteration: at least two stages");
-    static_assert(kWarpSlotWords * 4 * 2 <= kBatchStageBytes, "generic slots fit a stage");
+    static_assert(kBatchSynBytes >= 32 * lane_slot_words(8) * 4, "a lane tile's slots fit the syndrome buffer");
     static_assert(smem <= 232448, "shared memory per CTA");
 };
 
@@ -268,15 +271,18 @@ __global__ void __launch_bounds__(WARPS * 32)
 
     // lane 0: record claim t with descriptor d in stage s's slot and start its
     // load (tails are read by the whole warp later; past-the-end claims load nothing)
-    auto issue = [&](int s, uint32_t t, const DevTile &d) {
+    auto start = [&](int s, uint32_t t, const DevTile &d) {
         claim[s] = t;
-        if (t < num_tiles) desc[s] = d;
         if (t < num_tiles && d.bytes != 0) {
             mbar_arrive_expect_tx(&bar[s], d.bytes);
             bulk_g2s(s_stage + s * Cfg::stage_bytes, d.in + d.c0 * d.n / 32u, d.bytes, &bar[s]);
         } else {
             mbar_arrive(&bar[s]);
         }
+    };
+    auto issue = [&](int s, uint32_t t, const DevTile &d) {
+        if (t < num_tiles) desc[s] = d;
+        start(s, t, d);
     };
     // Which tile a warp takes next.  The single-n kernels (NSEL != 0) deal
     // tiles round-robin: warp gw takes tiles gw, gw + tw, gw + 2 tw, ... (tw
@@ -286,15 +292,21 @@ __global__ void __launch_bounds__(WARPS * 32)
     // that finished early takes more (measured: 250 µs claimed against 267 µs
     // dealt for it; 246 against 239 µs for the single-n kernels).  Either way the
     // next tile is claimed, and its descriptor fetched, one iteration ahead.
+    //
+    // The first tiles of the all-n kernel (its S stages and the one behind them) are
+    // dealt too, and the counter counts from there: S + 1 claims before the first load,
+    // each an atomic's round trip and its descriptor's, were 4 to 6 us of every launch
+    // (300 packets, 12-warp CTAs: 18.5 us with them, 12.7 without).
     const uint64_t gw = (uint64_t)blockIdx.x * WARPS + (uint64_t)warp, tw = (uint64_t)gridDim.x * WARPS;
+    constexpr uint32_t kDealt = S + 1;
     uint32_t seq = 0;  // lane 0: tiles dealt to this warp so far
     auto deal = [&]() -> uint32_t {
-        if constexpr (NSEL == 0) {
-            return atomicAdd(counter, 1u);
-        } else {
-            const uint64_t t = gw + (uint64_t)(seq++) * tw;
+        if (NSEL == 0 && seq >= kDealt) {
+            const uint64_t t = kDealt * tw + atomicAdd(counter, 1u);
             return t < (uint64_t)num_tiles ? (uint32_t)t : num_tiles;
         }
+        const uint64_t t = gw + (uint64_t)(seq++) * tw;
+        return t < (uint64_t)num_tiles ? (uint32_t)t : num_tiles;
     };
     // The single-n kernels fetch a descriptor two iterations before its tile
     // is issued (next_d is in registers when its refill is due, after_d is in
@@ -307,15 +319,27 @@ __global__ void __launch_bounds__(WARPS * 32)
 #pragma unroll
         for (int s = 0; s < S; ++s) mbar_init(&bar[s], 1);
         fence_mbar_init();
-        // the claim counter and the error counters are cleared by the kernel
-        // ahead of this one, which a programmatic dependent launch overlaps
-        grid_dep_wait();
+    }
+    // the claim counter and the error counters are cleared by the kernel
+    // ahead of this one, which a programmatic dependent launch overlaps
+    grid_dep_wait();
+    {
+        // the first S tiles' descriptors, a word a lane, their loads together
+        static_assert(sizeof(DevTile) == 64, "16 words");
+        uint32_t w[S];
+#pragma unroll
         for (int s = 0; s < S; ++s) {
-            const uint32_t t = deal();
-            DevTile d{};
-            if (t < num_tiles) d = tiles[t];
-            issue(s, t, d);
+            const uint64_t t = gw + (uint64_t)s * tw;
+            w[s] = t < num_tiles && lane < 16 ? reinterpret_cast<const uint32_t *>(tiles + t)[lane] : 0u;
         }
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+            if (lane < 16) reinterpret_cast<uint32_t *>(desc + s)[lane] = w[s];
+        __syncwarp();
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int s = 0; s < S; ++s) start(s, deal(), desc[s]);
         next_t = deal();
         if constexpr (kAhead2) {
             if (next_t < num_tiles) next_d = tiles[next_t];  // issued at the end of iteration 1
@@ -438,9 +462,12 @@ __global__ void __launch_bounds__(WARPS * 32)
             fence_proxy_async_smem();
             __syncwarp();
         } else {
-            // n = 3: generic warp tiles, the (unloaded) stage as slot memory
-            errs = generic_decode_tiles(p.in, p.in_words, p.n, p.m, p.num_cw, tl.c0 / 32, (tl.c0 + tl.count + 31) / 32,
-                                        1, p.out, p.out_words, p.syn, (int)p.syn_type, stage, stage + kWarpSlotWords);
+            // n = 3: one codeword per lane
+            uint32_t e = 0, unused = 0;
+            for (uint64_t t32 = tl.c0 / 32; t32 < (tl.c0 + tl.count + 31) / 32; ++t32)
+                decode_lane_tile<3, false>(p.in, p.in_words, p.num_cw, t32, p.out, p.out_words, p.syn,
+                                           (int)p.syn_type, stage, lane, e, unused);
+            errs = e;
             fence_proxy_async_smem();
             __syncwarp();
         }
@@ -557,8 +584,8 @@ SplitKernels make_split_kernels()
 
 static const std::vector<BatchVariant> &batch_variants()
 {
-    // index 0 is the built-in choice (and the serving and allocation-free
-    // paths' configuration); it holds no n = 15 table
+    // index 0 is the serving, one-shot and allocation-free paths' configuration; it
+    // holds no n = 15 table (see default_plan_variant for a plan's)
     static const std::vector<BatchVariant> v = {
         make_batch_variant<1, 3>(),        make_batch_variant<1, 2>(),        make_batch_variant<1, 4>(),
         make_batch_variant<2, 2>(),        make_batch_variant<4, 2>(),        make_batch_variant<8, 2, true>(),
@@ -616,6 +643,8 @@ constexpr int kMaxGroups = 18;
 
 using namespace hd;
 
+struct LaunchGeom;
+
 struct hd_plan {
     int device = 0;
     uint32_t num_packets = 0;
@@ -634,6 +663,8 @@ struct hd_plan {
     unsigned long long *graph_err = nullptr;
     bool graph_ok = false;
     uint64_t graph_kernels = 0;  // kernels one replay of the graph launches
+    std::unique_ptr<LaunchGeom> geom;  // what the launches resolved on their first call
+    bool geom_ok = false;
     // the split configuration: each code group's tile range (tiles are grouped
     // by n in kSplitOrder), a stream per group and the fork/join events
     uint32_t grp_begin[kSplitGroups] = {}, grp_end[kSplitGroups] = {};
@@ -655,6 +686,25 @@ struct hd_plan {
     uint32_t num_rest = 0;
     cudaStream_t mstream[kMaxGroups + 1] = {};  // [0]: the n = 3 tiles; [1 + g]: group g
     cudaEvent_t mjoin[kMaxGroups + 1] = {};
+};
+
+// Resolve everything that touches device state before a (possibly captured)
+// enqueue: kernel attributes, occupancy, the status word address and the
+// decode tables (filled on `st` on first use; `st` must not be capturing for
+// that, else the n = 7 tiles decode arithmetically and a configuration that
+// holds the n = 15 table gives way to the built-in one).
+struct LaunchGeom {
+    int variant;
+    int grid;
+    uint32_t *status;
+    const uint16_t *lut7, *lut15;
+    bool split = false;
+    const BatchVariant *gk[kSplitGroups] = {};  // split: the kernel of each code group
+    int ggrid[kSplitGroups] = {};
+    bool groups = false;                        // the stream-group configuration
+    const MultiVariant *mk[kMaxGroups] = {};    // its kernel per group
+    int mgrid[kMaxGroups] = {};
+    int rest_grid = 0;                          // the batch kernel's grid for the n = 3 tiles
 };
 
 namespace {
@@ -703,14 +753,23 @@ hd_status build_tables(const hd_packet *table, uint32_t num_packets, std::vector
     tiles.reserve(ntiles);
     // tiles grouped by n (long codes first), each code's tails among its full tiles
     uint32_t nfull_tiles = 0;
+    // the packets of each code length, so that its passes see no others (2000 packets:
+    // 21 passes over the whole table were half of a one-shot call's 86 us)
+    std::vector<uint32_t> by_code[kSplitGroups];
+    for (uint32_t i = 0; i < num_packets; ++i)
+        for (int gi = 0; gi < kSplitGroups; ++gi)
+            if (pk[i].n == kSplitOrder[gi]) by_code[gi].push_back(i);
+    auto view_of = [&](int gi) {
+        return [&, gi](uint32_t j) {
+            const uint32_t i = by_code[gi][j];
+            const DevPacket &d = pk[i];
+            return PacketView{d.in, d.out, d.syn, d.num_cw, d.n, d.m, d.syn_type, i};
+        };
+    };
     for (int gi = 0; gi < kSplitGroups; ++gi) {
         if (stats) stats->grp_begin[gi] = (uint32_t)tiles.size();
         emit_code_tiles(
-            kSplitOrder[gi], num_packets,
-            [&](uint32_t i) {
-                const DevPacket &d = pk[i];
-                return PacketView{d.in, d.out, d.syn, d.num_cw, d.n, d.m, d.syn_type};
-            },
+            kSplitOrder[gi], (uint32_t)by_code[gi].size(), view_of(gi),
             [&](const DevTile &t) {
                 tiles.push_back(t);
                 if (t.count & kFullTile) ++nfull_tiles;
@@ -725,11 +784,7 @@ hd_status build_tables(const hd_packet *table, uint32_t num_packets, std::vector
         for (int gi = 0; gi < kSplitGroups; ++gi) {
             if (stats) stats->grp_begin[gi] = (uint32_t)split->size();
             emit_code_tiles(
-                kSplitOrder[gi], num_packets,
-                [&](uint32_t i) {
-                    const DevPacket &d = pk[i];
-                    return PacketView{d.in, d.out, d.syn, d.num_cw, d.n, d.m, d.syn_type};
-                },
+                kSplitOrder[gi], (uint32_t)by_code[gi].size(), view_of(gi),
                 [&](const DevTile &t) { split->push_back(t); }, true);
             if (stats) stats->grp_end[gi] = (uint32_t)split->size();
         }
@@ -816,7 +871,7 @@ hd_status build_group_tables(const std::vector<DevPacket> &pk, std::vector<Multi
         3, np,
         [&](uint32_t i) {
             const DevPacket &d = pk[i];
-            return PacketView{d.in, d.out, d.syn, d.num_cw, d.n, d.m, d.syn_type};
+            return PacketView{d.in, d.out, d.syn, d.num_cw, d.n, d.m, d.syn_type, i};
         },
         [&](const DevTile &t) { rest.push_back(t); });
     if (rest.size() >= 0xFFFFFFF0ull) return HD_ERR_CAPACITY;
@@ -832,31 +887,45 @@ int batch_grid(const BatchVariant &v, uint32_t num_tiles)
     return decode_grid(want, cap);
 }
 
-// Resolve everything that touches device state before a (possibly captured)
-// enqueue: kernel attributes, occupancy, the status word address and the
-// decode tables (filled on `st` on first use; `st` must not be capturing for
-// that, else the n = 7 tiles decode arithmetically and a configuration that
-// holds the n = 15 table gives way to the built-in one).
-struct LaunchGeom {
-    int variant;
-    int grid;
-    uint32_t *status;
-    const uint16_t *lut7, *lut15;
-    bool split = false;
-    const BatchVariant *gk[kSplitGroups] = {};  // split: the kernel of each code group
-    int ggrid[kSplitGroups] = {};
-    bool groups = false;                        // the stream-group configuration
-    const MultiVariant *mk[kMaxGroups] = {};    // its kernel per group
-    int mgrid[kMaxGroups] = {};
-    int rest_grid = 0;                          // the batch kernel's grid for the n = 3 tiles
-};
-
 // Index of the first split configuration among a plan's configurations
 // (after the single-kernel ones), of the stream-group configuration (the
 // last), and the number of configurations.
 inline int split_variant() { return (int)batch_variants().size(); }
 inline int group_variant() { return split_variant() + (int)split_kernels().size(); }
 inline int plan_variants() { return group_variant() + 1; }
+
+// The configuration of a new plan, until it is tuned or selected.  On GB300, packets
+// of 64 bit .. 4 Mbit of mixed n with u8 syndromes (time of 1-warp CTAs with two
+// stages (1), 4-warp (4), 12- and 14-warp CTAs around the n = 15 table (6, 7), stream
+// groups (9)): 100 packets 13.4 / 9.5 / 10.4 / 10.4 / 15.4 us, 300 (3800 tiles) 16.6 /
+// 15.9 / 12.7 / 14.5 / 18.8, 1000 34.4 / 39.5 / 34.8 / 34.1 / 45.6, 3000 (0.3 GB moved)
+// 83.8 / 102.9 / 88.4 / 85.0 / 107.3, 10,000 (1 GB) 247 / 300 / 268 / 251 / 223.
+// Without n = 15 packets the table only takes room.
+int default_plan_variant(const hd_plan *p, bool has15)
+{
+    constexpr uint64_t kGroupBytes = 768ull << 20;  // the stream groups' ramps and drains pay off
+    if (p->groups_ok && p->in_bytes + p->out_bytes + p->syn_bytes >= kGroupBytes) return group_variant();
+    if (p->num_tiles < 2048) return 4;
+    if (!has15) return 1;
+    return p->num_tiles < 8192 ? 6 : 7;
+}
+
+// The streams and events that a configuration's branches and graph need, created when
+// it is first chosen (all 27 streams up front were most of hd_plan_create's time for
+// small plans: 10 packets 126 us, now 30).
+bool ensure_branches(hd_plan *p, int variant)
+{
+    auto branch = [](cudaStream_t *s, cudaEvent_t *e) {
+        return (*s != nullptr || cudaStreamCreateWithFlags(s, cudaStreamNonBlocking) == cudaSuccess) &&
+               (e == nullptr || *e != nullptr || cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess);
+    };
+    const bool groups = variant == group_variant() && p->groups_ok, split = variant >= split_variant() && !groups;
+    bool ok = !(groups || split) || branch(&p->capture, nullptr);
+    for (int gi = 0; ok && split && variant != group_variant() && gi < kSplitGroups; ++gi)
+        ok = branch(&p->gstream[gi], &p->join[gi]);
+    for (size_t b = 0; ok && groups && b <= p->groups.size(); ++b) ok = branch(&p->mstream[b], &p->mjoin[b]);
+    return ok;
+}
 
 cudaError_t prepare_plan(hd_plan *p, LaunchGeom *g, cudaStream_t st)
 {
@@ -1001,6 +1070,14 @@ void drop_graph(hd_plan *p)
     p->graph_ok = false;
 }
 
+// Forget the recorded graph and the resolved geometry (another configuration).
+void drop_plan(hd_plan *p)
+{
+    drop_graph(p);
+    p->geom.reset();
+    p->geom_ok = false;
+}
+
 }  // namespace
 
 namespace hd {
@@ -1055,6 +1132,8 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
     p->num_packets = num_packets;
     p->num_tiles = (uint32_t)tiles.size();
     p->num_rest = (uint32_t)rest.size();
+    p->variant = default_plan_variant(
+        p, std::any_of(pk.begin(), pk.end(), [](const DevPacket &d) { return d.n == 15 && d.num_cw != 0; }));
     auto rounded = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t tl_b = rounded(tiles.size() * sizeof(DevTile)), sp_b = rounded(split.size() * sizeof(DevTile));
     const size_t ru_b = rounded(runs.size() * sizeof(MultiRun)), re_b = rounded(rest.size() * sizeof(DevTile));
@@ -1075,14 +1154,8 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
               upload(p->d_split, split.data(), split.size() * sizeof(DevTile)) &&
               upload(p->d_runs, runs.data(), runs.size() * sizeof(MultiRun)) &&
               upload(p->d_rest, rest.data(), rest.size() * sizeof(DevTile)) &&
-              cudaStreamCreateWithFlags(&p->capture, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int gi = 0; ok && gi < kSplitGroups; ++gi)
-        ok = cudaStreamCreateWithFlags(&p->gstream[gi], cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&p->join[gi], cudaEventDisableTiming) == cudaSuccess;
-    for (size_t b = 0; ok && b <= p->groups.size(); ++b)
-        ok = cudaStreamCreateWithFlags(&p->mstream[b], cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&p->mjoin[b], cudaEventDisableTiming) == cudaSuccess;
+              cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming) == cudaSuccess &&
+              ensure_branches(p, p->variant);
     if (!ok) {
         hd_plan_destroy(p);
         return HD_ERR_CUDA;
@@ -1095,10 +1168,22 @@ hd_status hd_plan_launch(hd_plan *p, unsigned long long *err_counts, void *cuda_
 {
     if (!p) return HD_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    // The single-kernel configurations are two launches (the clear and the decode, its
+    // programmatic dependent): launched directly, with the geometry resolved once, as a
+    // graph's would be.
+    if (!p->geom_ok) {
+        p->geom = std::make_unique<LaunchGeom>();
+        if (prepare_plan(p, p->geom.get(), st) != cudaSuccess) return HD_ERR_CUDA;
+        p->geom_ok = true;
+    }
+    if (!p->geom->split && !p->geom->groups) {
+        if (enqueue_plan(p, *p->geom, err_counts, st) != cudaSuccess) return HD_ERR_CUDA;
+        if (p->num_tiles) count_launch();  // the clear is counted where it is enqueued
+        return HD_OK;
+    }
     if (!p->graph_ok || p->graph_err != err_counts) {
         drop_graph(p);
-        LaunchGeom geom;
-        if (prepare_plan(p, &geom, st) != cudaSuccess) return HD_ERR_CUDA;
+        const LaunchGeom &geom = *p->geom;
         if (cudaStreamBeginCapture(p->capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return HD_ERR_CUDA;
         const cudaError_t e = enqueue_plan(p, geom, err_counts, p->capture);
         g_launches.fetch_sub(1, std::memory_order_relaxed);  // the clear recorded here runs (and counts) per replay
@@ -1137,9 +1222,13 @@ hd_status hd_plan_autotune(hd_plan *p, uint32_t reps, void *cuda_stream, hd_plan
     // graph, then replayed (err_counts NULL: the counts are not part of the choice)
     for (int i = 0; i < plan_variants(); ++i) {
         p->variant = i;
+        if (!ensure_branches(p, i)) {
+            rc = HD_ERR_CUDA;
+            break;
+        }
         LaunchGeom geom;
         if (prepare_plan(p, &geom, st) != cudaSuccess || geom.variant != i) continue;
-        drop_graph(p);
+        drop_plan(p);
         if ((rc = hd_plan_launch(p, nullptr, st)) != HD_OK) break;  // records the graph and runs it once
         cudaEventRecord(e0, st);
         for (uint32_t r = 0; r < reps; ++r)
@@ -1161,7 +1250,7 @@ hd_status hd_plan_autotune(hd_plan *p, uint32_t reps, void *cuda_stream, hd_plan
     cudaEventDestroy(e1);
     p->variant = best >= 0 ? best : keep;
     p->tuned_us = best >= 0 ? best_us : -1.f;
-    drop_graph(p);
+    drop_plan(p);
     if (rc != HD_OK) return rc;
     if (chosen) return hd_plan_get_info(p, chosen);
     return HD_OK;
@@ -1205,8 +1294,9 @@ hd_status hd_plan_select(hd_plan *p, uint32_t variant)
 {
     if (!p) return HD_ERR_NULL;
     if (variant >= (uint32_t)plan_variants()) return HD_ERR_INVALID_ARG;
+    if (!ensure_branches(p, (int)variant)) return HD_ERR_CUDA;
     p->variant = (int)variant;
-    drop_graph(p);
+    drop_plan(p);
     return HD_OK;
 }
 
@@ -1399,7 +1489,7 @@ extern "C" hd_status hd_decode_batch_noalloc(const hd_packet *table, uint32_t nu
             [&](uint32_t i) {
                 const hd_packet &q = table[i];
                 return PacketView{q.in, q.out, static_cast<uint8_t *>(q.syndromes), q.num_codewords, q.n,
-                                  (uint32_t)code_m(q.n), q.syndromes ? q.syn_type : 0u};
+                                  (uint32_t)code_m(q.n), q.syndromes ? q.syn_type : 0u, i};
             },
             [&](const DevTile &tile) {
                 up.tiles[up.count++] = tile;
