@@ -91,13 +91,29 @@ struct Chunk {
 
 // The chunk schedule of a batch: every job cut into chunks of C codewords,
 // except that the first chunks of the batch ramp up (C/8, C/4, C/2) and the
-// last ones ramp down, so the pipeline fills and drains on small copies.
-std::vector<Chunk> schedule(const hd_host_job *jobs, uint32_t num, uint64_t C)
+// last ones ramp down, so the pipeline fills and drains on small copies.  With the
+// default chunk (`split_one`) a batch that is one chunk of 24 MB of copies or more is cut
+// into four equal pieces of whole 4 KB pages, so that its copies in and out overlap
+// (67 MB: 315 us against 373 in one piece; with the ramps 336; 17 MB: 124 against 116).
+std::vector<Chunk> schedule(const hd_host_job *jobs, uint32_t num, uint64_t C, bool split_one)
 {
     std::vector<Chunk> out;
     for (uint32_t j = 0; j < num; ++j)
         for (uint64_t c0 = 0; c0 < jobs[j].num_codewords; c0 += C)
             out.push_back({j, c0, std::min(C, jobs[j].num_codewords - c0)});
+    if (split_one && out.size() == 1) {
+        const Chunk all = out[0];
+        const hd_host_job &b = jobs[all.job];
+        const uint32_t k = b.n - (uint32_t)code_m(b.n);
+        const uint64_t bytes = all.cnt * (b.n + k) / 8 + all.cnt * (b.syn_type == HD_SYN_U16 ? 2u : b.syn_type == HD_SYN_U8);
+        const uint64_t page = 32768;  // codewords that fill whole 4 KB pages of input and output
+        const uint64_t piece = (all.cnt / 4 + page - 1) / page * page;
+        if (bytes >= 24ull << 20 && piece < all.cnt) {
+            out.clear();
+            for (uint64_t c0 = 0; c0 < all.cnt; c0 += piece) out.push_back({all.job, c0, std::min(piece, all.cnt - c0)});
+            return out;
+        }
+    }
     // split the first chunk into pieces of 1/8, 1/4, 1/2 and the rest, and the last chunk into the
     // rest, 1/2, 1/4, 1/8 (multiples of 128 codewords)
     auto ramp = [&](size_t at, bool up) {
@@ -140,7 +156,8 @@ extern "C" hd_status hd_decode_host_batch(const hd_host_job *jobs, uint32_t num_
 {
     if (num_jobs == 0) return HD_OK;
     if (!jobs) return HD_ERR_NULL;
-    if (chunk_codewords == 0) chunk_codewords = 1ull << 22;  // the fastest of 2^19..2^24 on GB300
+    const bool auto_chunk = chunk_codewords == 0;
+    if (auto_chunk) chunk_codewords = 1ull << 22;  // the fastest of 2^19..2^24 on GB300
     if (depth == 0) depth = 4;
     // chunks start on 16-byte boundaries of both the input and the output
     if (chunk_codewords % 128 != 0 || depth > kMaxDepth) return HD_ERR_INVALID_ARG;
@@ -163,7 +180,7 @@ extern "C" hd_status hd_decode_host_batch(const hd_host_job *jobs, uint32_t num_
         syn_max = std::max(syn_max, round256(Cj * sb + 16));
         C = std::max(C, Cj);
     }
-    const std::vector<Chunk> plan = schedule(jobs, num_jobs, chunk_codewords);
+    const std::vector<Chunk> plan = schedule(jobs, num_jobs, chunk_codewords, auto_chunk);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HD_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_pipe_mu);
@@ -195,8 +212,8 @@ extern "C" hd_status hd_decode_host_batch(const hd_host_job *jobs, uint32_t num_
                                   cudaMemcpyDeviceToHost, st) != cudaSuccess)
             return HD_ERR_CUDA;
     }
-    // gather the per-chunk error counts once every stream has finished
-    for (uint32_t s = 0; s < depth; ++s) {
+    // gather the per-chunk error counts once every stream used has finished
+    for (uint32_t s = 1; s < std::min<uint64_t>(depth, plan.size()); ++s) {
         cudaEventRecord(p.done[s], p.st[s]);
         cudaStreamWaitEvent(p.st[0], p.done[s], 0);
     }
