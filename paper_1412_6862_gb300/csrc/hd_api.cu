@@ -14,23 +14,17 @@ std::atomic<uint32_t> g_max_ctas{0};
 
 int num_sms()
 {
-    static std::mutex mu;
-    static int cached[64];
-    static bool init = false;
+    static std::atomic<int> cached[64];
     int dev = 0;
     cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lk(mu);
-    if (!init) {
-        for (int &c : cached) c = 0;
-        init = true;
-    }
     if (dev < 0 || dev >= 64) dev = 0;
-    if (cached[dev] == 0) {
-        int v = 0;
+    int v = cached[dev].load(std::memory_order_relaxed);
+    if (v == 0) {
         cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        cached[dev] = v > 0 ? v : 1;
+        cached[dev].store(v > 0 ? v : 1, std::memory_order_relaxed);
+        v = v > 0 ? v : 1;
     }
-    return cached[dev];
+    return v;
 }
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -201,25 +195,33 @@ hd_status hd_decode_streams(const hd_stream_job *jobs, uint32_t num_jobs, void *
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return HD_ERR_CUDA;
     }
-    if (cudaEventRecord(pool.fork, st) != cudaSuccess) return HD_ERR_CUDA;
-    const int used = (int)std::min<uint32_t>(num_jobs, kPoolStreams);
-    for (int i = 0; i < used; ++i)
-        if (cudaStreamWaitEvent(pool.s[i], pool.fork, 0) != cudaSuccess) return HD_ERR_CUDA;
     // the largest streams first, so that the shorter ones fill in around them
-    uint32_t order[kMaxStreamJobs];
-    for (uint32_t i = 0; i < num_jobs; ++i) order[i] = i;
-    std::sort(order, order + num_jobs, [&](uint32_t x, uint32_t y) {
+    uint32_t order[kMaxStreamJobs], count = 0;
+    for (uint32_t i = 0; i < num_jobs; ++i)
+        if (jobs[i].num_codewords != 0) order[count++] = i;
+    std::sort(order, order + count, [&](uint32_t x, uint32_t y) {
         return (uint64_t)jobs[x].n * jobs[x].num_codewords > (uint64_t)jobs[y].n * jobs[y].num_codewords;
     });
-    for (uint32_t r = 0; r < num_jobs; ++r) {
+    // One branch per stream that fills the GPU, the largest on the caller's stream itself;
+    // the short ones (one codeword per lane, 2 to 4 us each) share a branch, chained: an
+    // event wait, a record and a wait each cost more than running them one after another.
+    uint32_t big = 0;
+    while (big < count && !lanes_suffice(jobs[order[big]].n, false, jobs[order[big]].num_codewords)) ++big;
+    const uint32_t branches = big + (big < count ? 1u : 0u);
+    const int pooled = (int)std::min<uint32_t>(branches > 0 ? branches - 1 : 0, kPoolStreams);
+    if (pooled > 0 && cudaEventRecord(pool.fork, st) != cudaSuccess) return HD_ERR_CUDA;
+    for (int i = 0; i < pooled; ++i)
+        if (cudaStreamWaitEvent(pool.s[i], pool.fork, 0) != cudaSuccess) return HD_ERR_CUDA;
+    for (uint32_t r = 0; r < count; ++r) {
         const hd_stream_job &j = jobs[order[r]];
-        if (j.num_codewords == 0) continue;
+        const uint32_t branch = std::min(r, big);
+        const bool chained = r > big;  // behind another decode of this call
         if (launch_decode(decode_job(j.stream, j.n, j.num_codewords, j.out_bits, j.syndromes,
                                      static_cast<hd_syn_type>(j.syn_type), j.err_count),
-                          pool.s[r % kPoolStreams], false) != cudaSuccess)
+                          branch == 0 ? st : pool.s[(branch - 1) % kPoolStreams], chained) != cudaSuccess)
             return HD_ERR_CUDA;
     }
-    for (int i = 0; i < used; ++i)
+    for (int i = 0; i < pooled; ++i)
         if (cudaEventRecord(pool.join[i], pool.s[i]) != cudaSuccess ||
             cudaStreamWaitEvent(st, pool.join[i], 0) != cudaSuccess)
             return HD_ERR_CUDA;

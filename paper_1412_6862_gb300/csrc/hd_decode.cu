@@ -2,6 +2,7 @@
 // per-device launch setup, the configuration choice (built-in defaults or the
 // autotuner's measured pick) and the device status word.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -76,8 +77,6 @@ std::map<std::tuple<int, uint32_t, int>, int> g_choice;
 std::set<std::tuple<int, uint32_t, int>> g_pinned;
 // (device, n, syn) -> pinned SECDED configuration (index into secded_variants())
 std::map<std::tuple<int, uint32_t, int>, int> g_secded_choice;
-// device -> address of g_hd_status
-std::map<int, uint32_t *> g_status_ptr;
 
 // Built-in choice per (n, syndrome type or -1 for any, G, T, S, inplace,
 // decode table), measured on GB300; used until the autotuner or the caller
@@ -126,7 +125,7 @@ int find_variant(uint32_t n, int syn, int G, int T, int S, int inplace, int lut)
     return -1;
 }
 
-int default_variant(uint32_t n, int syn)
+int find_default_variant(uint32_t n, int syn)
 {
     for (const auto &d : kDefaults)
         if (d.n == n && (d.syn < 0 || d.syn == syn)) {
@@ -139,8 +138,29 @@ int default_variant(uint32_t n, int syn)
     return -1;
 }
 
+// The built-in configuration of (n, syn), looked up once.
+int default_variant(uint32_t n, int syn)
+{
+    struct Table {
+        int v[9][3];
+        Table()
+        {
+            for (int m = 0; m <= 8; ++m)
+                for (int t = 0; t < 3; ++t) v[m][t] = find_default_variant((1u << m) - 1u, t);
+        }
+    };
+    static const Table table;
+    const int m = code_m(n);
+    return m != 0 && syn >= 0 && syn < 3 ? table.v[m][syn] : -1;
+}
+
+// Whether any configuration was ever chosen (tuned or pinned) in this process:
+// until then every launch takes the built-in ones without a lock.
+std::atomic<bool> g_any_choice{false};
+
 int chosen_variant(uint32_t n, int syn)
 {
+    if (!g_any_choice.load(std::memory_order_acquire)) return default_variant(n, syn);
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = g_choice.find({current_device(), n, syn});
     if (it != g_choice.end()) return it->second;
@@ -166,15 +186,15 @@ int stream_blocks_per_sm(const void *kernel, int threads, uint32_t smem)
 
 uint32_t *status_ptr()
 {
+    static std::atomic<uint32_t *> cached[64];
     const int dev = current_device();
-    std::lock_guard<std::mutex> lk(g_mu);
-    uint32_t *&p = g_status_ptr[dev];
-    if (p == nullptr) {
-        void *a = nullptr;
-        if (cudaGetSymbolAddress(&a, g_hd_status) != cudaSuccess) return nullptr;
-        p = static_cast<uint32_t *>(a);
-    }
-    return p;
+    const bool in_range = dev >= 0 && dev < 64;
+    if (in_range)
+        if (uint32_t *p = cached[dev].load(std::memory_order_acquire)) return p;
+    void *a = nullptr;
+    if (cudaGetSymbolAddress(&a, g_hd_status) != cudaSuccess) return nullptr;
+    if (in_range) cached[dev].store(static_cast<uint32_t *>(a), std::memory_order_release);
+    return static_cast<uint32_t *>(a);
 }
 
 uint32_t read_clear_status_decode()
@@ -216,12 +236,14 @@ const StreamVariant *variant_n3(int syn)
 
 bool variant_pinned(uint32_t n, int syn)
 {
+    if (!g_any_choice.load(std::memory_order_acquire)) return false;
     std::lock_guard<std::mutex> lk(g_mu);
     return g_pinned.count({current_device(), n, syn}) != 0;
 }
 
 bool secded_variant_pinned(uint32_t n, int syn)
 {
+    if (!g_any_choice.load(std::memory_order_acquire)) return false;
     std::lock_guard<std::mutex> lk(g_mu);
     return g_secded_choice.count({current_device(), n, syn}) != 0;
 }
@@ -248,7 +270,7 @@ cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl)
 cudaError_t launch_decode_secded(const DecodeJob &j, cudaStream_t st, bool pdl)
 {
     int pinned = -1;
-    {
+    if (g_any_choice.load(std::memory_order_acquire)) {
         std::lock_guard<std::mutex> lk(g_mu);
         auto it = g_secded_choice.find({current_device(), j.n, j.syn_type});
         if (it != g_secded_choice.end()) pinned = it->second;
@@ -352,6 +374,7 @@ hd_status hd_variant_select(uint32_t n, hd_syn_type syn_type, int32_t ordinal)
         if (v[i].n == n && v[i].syn == (int)syn_type) {
             if (c == ordinal) {
                 g_choice[{dev, n, (int)syn_type}] = (int)i;
+                g_any_choice.store(true, std::memory_order_release);
                 g_pinned.insert({dev, n, (int)syn_type});
                 return HD_OK;
             }
@@ -429,6 +452,7 @@ hd_status hd_secded_variant_select(uint32_t n, hd_syn_type syn_type, int32_t ord
         if (v[i].n == n && v[i].syn == (int)syn_type) {
             if (c == ordinal) {
                 g_secded_choice[{dev, n, (int)syn_type}] = (int)i;
+                g_any_choice.store(true, std::memory_order_release);
                 return HD_OK;
             }
             ++c;
@@ -565,6 +589,7 @@ hd_status hd_autotune(uint32_t n, hd_syn_type syn_type, uint64_t num_codewords, 
     {
         std::lock_guard<std::mutex> lk(g_mu);
         g_choice[{current_device(), n, (int)syn_type}] = best;
+        g_any_choice.store(true, std::memory_order_release);
         g_pinned.erase({current_device(), n, (int)syn_type});
     }
     if (chosen) {

@@ -185,8 +185,8 @@ cudaError_t launch_encode_stream(const uint32_t *data, uint32_t *stream, EncArgs
 {
     using Cfg = EncCfg<N_, T, S, G, CH>;
     a.tile_end = (a.num_cw + 31) / 32;
-    const int lane_bps =
-        stream_blocks_per_sm(reinterpret_cast<const void *>(k_encode_lanes<N_>), kLaneWarps * 32, 0);
+    static BlocksPerSm lane_blocks, blocks;
+    const int lane_bps = lane_blocks.get(reinterpret_cast<const void *>(k_encode_lanes<N_>), kLaneWarps * 32, 0);
     const uint64_t lane_cap = (uint64_t)num_sms() * (uint64_t)std::max(lane_bps, 1);
     // At most one round of tiles on the CTAs the device holds at once (152 SMs:
     // 311,296 codewords, fewer for the long codes' wider kernels): the two paths cross
@@ -199,7 +199,7 @@ cudaError_t launch_encode_stream(const uint32_t *data, uint32_t *stream, EncArgs
                              data, stream, a);
     }
     auto kern = k_encode_stream<N_, T, S, G, CH>;
-    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kern), T, Cfg::smem);
+    const int bps = blocks.get(reinterpret_cast<const void *>(kern), T, Cfg::smem);
     if (bps <= 0) return cudaErrorInvalidConfiguration;
     a.nchunks = a.num_cw / Cfg::chunk_cw;
     a.tile_begin = a.nchunks * (Cfg::chunk_cw / 32);

@@ -76,6 +76,26 @@ cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, ui
 // (opted in to on first use), cached per device; <= 0 on failure.
 int stream_blocks_per_sm(const void *kernel, int threads, uint32_t smem);
 
+// stream_blocks_per_sm() of one kernel, kept per device without a lock: one static
+// instance per kernel (its threads and shared memory never change).
+class BlocksPerSm {
+    std::atomic<int> v_[64] = {};
+
+public:
+    int get(const void *kernel, int threads, uint32_t smem)
+    {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev < 0 || dev >= 64) return stream_blocks_per_sm(kernel, threads, smem);
+        int v = v_[dev].load(std::memory_order_relaxed);
+        if (v == 0) {
+            v = stream_blocks_per_sm(kernel, threads, smem);
+            if (v > 0) v_[dev].store(v, std::memory_order_relaxed);
+        }
+        return v;
+    }
+};
+
 // Launch `kern` on `st`, as the programmatic dependent of the kernel ahead of
 // it in the stream when pdl is set (it may then start before that kernel has
 // finished, and must wait for it before touching what that kernel writes).

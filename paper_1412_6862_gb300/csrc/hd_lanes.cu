@@ -59,8 +59,9 @@ __global__ void __launch_bounds__(WARPS * 32)
 template <int N_, bool XH>
 uint64_t lane_ctas()
 {
-    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(k_decode_lanes<N_, XH, kLaneWarps, false>),
-                                         kLaneWarps * 32, 0);
+    static BlocksPerSm blocks;
+    const int bps =
+        blocks.get(reinterpret_cast<const void *>(k_decode_lanes<N_, XH, kLaneWarps, false>), kLaneWarps * 32, 0);
     return (uint64_t)num_sms() * (uint64_t)std::max(bps, 1);
 }
 

@@ -10,6 +10,7 @@
 // kernel on first use per device (on the caller's stream, which that first
 // call then synchronises; a first call inside a stream capture falls back to
 // the arithmetic decoder).
+#include <atomic>
 #include <cstdint>
 #include <mutex>
 
@@ -66,6 +67,7 @@ __global__ void k_fill_lut_xh(uint16_t *lut, uint32_t n, uint32_t m)
 
 std::mutex g_lut_mu;
 bool g_lut_ready[64][4];
+std::atomic<const uint16_t *> g_lut_filled[64][4];  // a filled table's device address
 
 }  // namespace
 
@@ -77,6 +79,7 @@ const uint16_t *lut_ptr(uint32_t n, cudaStream_t st, bool xh)
     static const void *const syms[4] = {&g_lut7, &g_lut15, &g_lut7x, &g_lut15x};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (const uint16_t *t = g_lut_filled[dev][slot].load(std::memory_order_acquire)) return t;
     void *p = nullptr;
     if (cudaGetSymbolAddress(&p, syms[slot]) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lk(g_lut_mu);
@@ -92,6 +95,7 @@ const uint16_t *lut_ptr(uint32_t n, cudaStream_t st, bool xh)
         // kernels on other streams may use the table next: wait for it once
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return nullptr;
         g_lut_ready[dev][slot] = true;
+        g_lut_filled[dev][slot].store(static_cast<const uint16_t *>(p), std::memory_order_release);
     }
     return static_cast<const uint16_t *>(p);
 }

@@ -449,7 +449,8 @@ cudaError_t launch_stream_variant(const StreamArgs &a, cudaStream_t st, bool pdl
     auto kern = k_decode_stream<N_, SYN, T, S, G, INPLACE, XH, LUT>;
     if constexpr (has_tailless(N_, LUT, T, S))
         if (a.tile_begin == a.tile_end) kern = k_decode_stream<N_, SYN, T, S, G, INPLACE, XH, LUT, false>;
-    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kern), T, Cfg::smem);
+    static BlocksPerSm blocks[2];  // with and without the tail
+    const int bps = blocks[a.tile_begin == a.tile_end].get(reinterpret_cast<const void *>(kern), T, Cfg::smem);
     if (bps <= 0) return cudaErrorInvalidConfiguration;
     const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
     const uint64_t want = (a.nchunks + Cfg::WARPS - 1) / Cfg::WARPS;

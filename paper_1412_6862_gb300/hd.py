@@ -494,26 +494,61 @@ def hd_version() -> int:
 # ----------------------------------------------------------------------------
 # PyTorch marshalling
 # ----------------------------------------------------------------------------
+_CODES = {(1 << m) - 1: (m, (1 << m) - 1 - m) for m in range(2, 9)}
+
+
 def code_params(n: int) -> tuple[int, int]:
     """(m, k) for n = 2^m - 1, 2 <= m <= 8."""
-    for m in range(2, 9):
-        if n == (1 << m) - 1:
-            return m, n - m
-    raise HDError(HD_ERR_INVALID_N, f"n={n}")
+    try:
+        return _CODES[n]
+    except KeyError:
+        raise HDError(HD_ERR_INVALID_N, f"n={n}") from None
 
 
 def words_for(bits: int) -> int:
     return (int(bits) + 31) // 32
 
 
-def _stream_handle(stream=None) -> int:
+_raw_stream = None  # () -> handle of the current CUDA stream
+
+
+def _find_raw_stream():
+    """torch.cuda.current_stream() builds a Stream object per call, 3 us beside the
+    2 to 4 us of a decode's launches; the handle alone takes 0.2 us."""
+    global _raw_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    torch.cuda.current_stream()  # initialises CUDA
+    try:
+        get, dev = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        get(dev())
+        _raw_stream = lambda: get(dev())  # noqa: E731
+    except AttributeError:
+        _raw_stream = lambda: int(torch.cuda.current_stream().cuda_stream)  # noqa: E731
+
+
+def _stream_handle(stream=None) -> int:
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is None:
+        _find_raw_stream()
+    return _raw_stream()
 
 
 def _ptr(t) -> int | None:
-    return None if t is None else int(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _empty_for(words: int, syn_type: int, num_codewords: int, ncounts: int, device, out, syndromes, counts):
+    """The outputs of a decode that the caller did not give."""
+    import torch
+    if out is None:
+        out = torch.empty(words, dtype=torch.int32, device=device)
+    if syndromes is None and syn_type != SYN_NONE:
+        syndromes = torch.empty(num_codewords, dtype=torch.uint8 if syn_type == SYN_U8 else torch.int16,
+                                device=device)
+    if counts is None:
+        counts = torch.empty(ncounts, dtype=torch.int64, device=device)
+    return out, syndromes, counts
 
 
 def decode(stream_words, n: int, num_codewords: int, syn_type: int = SYN_U8, out=None, syndromes=None,
@@ -522,19 +557,13 @@ def decode(stream_words, n: int, num_codewords: int, syn_type: int = SYN_U8, out
 
     Returns (out_words int32 tensor, syndromes tensor or None, err_count int64
     tensor of one element).  Outputs are allocated when not given."""
-    import torch
     m, k = code_params(n)
-    dev = stream_words.device
-    if out is None:
-        out = torch.empty(max(1, words_for(num_codewords * k)), dtype=torch.int32, device=dev)
-    if syndromes is None and syn_type != SYN_NONE:
-        dt = torch.uint8 if syn_type == SYN_U8 else torch.int16
-        syndromes = torch.empty(max(1, num_codewords), dtype=dt, device=dev)
-    if err_count is None:
-        err_count = torch.empty(1, dtype=torch.int64, device=dev)
-    rc = hd_decode(_ptr(stream_words), n * num_codewords, n, num_codewords, _ptr(out),
-                   _ptr(syndromes) if syn_type != SYN_NONE else None, syn_type, _ptr(err_count),
-                   _stream_handle(cuda_stream))
+    if out is None or err_count is None or (syndromes is None and syn_type != SYN_NONE):
+        out, syndromes, err_count = _empty_for(max(1, words_for(num_codewords * k)), syn_type, max(1, num_codewords),
+                                               1, stream_words.device, out, syndromes, err_count)
+    rc = lib().hd_decode(stream_words.data_ptr(), n * num_codewords, n, num_codewords, out.data_ptr(),
+                         syndromes.data_ptr() if syn_type != SYN_NONE else None, syn_type, err_count.data_ptr(),
+                         _stream_handle(cuda_stream))
     check(rc, "hd_decode")
     return out, syndromes, err_count
 
@@ -588,19 +617,14 @@ def decode_short(stream_words, n: int, num_codewords: int, syn_type: int = SYN_U
 
     Returns (out_words, syndromes or None, counts) where counts is an int64
     tensor of two elements: [nonzero syndromes, syndromes past n]."""
-    import torch
-    r, k = hd_short_params(n)
-    dev = stream_words.device
-    if out is None:
-        out = torch.empty(max(4, words_for(num_codewords * k)), dtype=torch.int32, device=dev)
-    if syndromes is None and syn_type != SYN_NONE:
-        dt = torch.uint8 if syn_type == SYN_U8 else torch.int16
-        syndromes = torch.empty(max(16, num_codewords), dtype=dt, device=dev)
-    if counts is None:
-        counts = torch.empty(2, dtype=torch.int64, device=dev)
-    rc = hd_decode_short(_ptr(stream_words), n * num_codewords, n, num_codewords, _ptr(out),
-                         _ptr(syndromes) if syn_type != SYN_NONE else None, syn_type, _ptr(counts),
-                         _ptr(counts) + 8, _stream_handle(cuda_stream))
+    if out is None or counts is None or (syndromes is None and syn_type != SYN_NONE):
+        r, k = hd_short_params(n)
+        out, syndromes, counts = _empty_for(max(4, words_for(num_codewords * k)), syn_type, max(16, num_codewords), 2,
+                                            stream_words.device, out, syndromes, counts)
+    c = counts.data_ptr()
+    rc = lib().hd_decode_short(stream_words.data_ptr(), n * num_codewords, n, num_codewords, out.data_ptr(),
+                               syndromes.data_ptr() if syn_type != SYN_NONE else None, syn_type, c, c + 8,
+                               _stream_handle(cuda_stream))
     check(rc, "hd_decode_short")
     return out, syndromes, counts
 
@@ -613,23 +637,19 @@ class ShortPlan:
         h = _vp()
         check(lib().hd_short_plan_create(n, ctypes.byref(h)), "hd_short_plan_create")
         self.handle, self.n = h.value, n
+        self.k = hd_short_params(n)[1]
 
     def decode(self, stream_words, num_codewords: int, syn_type: int = SYN_U16, out=None, syndromes=None,
                counts=None, cuda_stream=None):
         """As decode_short(); returns (out_words, syndromes or None, counts)."""
-        import torch
-        r, k = hd_short_params(self.n)
-        dev = stream_words.device
-        if out is None:
-            out = torch.empty(max(4, words_for(num_codewords * k)), dtype=torch.int32, device=dev)
-        if syndromes is None and syn_type != SYN_NONE:
-            dt = torch.uint8 if syn_type == SYN_U8 else torch.int16
-            syndromes = torch.empty(max(16, num_codewords), dtype=dt, device=dev)
-        if counts is None:
-            counts = torch.empty(2, dtype=torch.int64, device=dev)
-        rc = lib().hd_decode_short_plan(self.handle, _ptr(stream_words), self.n * num_codewords, num_codewords,
-                                        _ptr(out), _ptr(syndromes) if syn_type != SYN_NONE else None, syn_type,
-                                        _ptr(counts), _ptr(counts) + 8, _stream_handle(cuda_stream))
+        if out is None or counts is None or (syndromes is None and syn_type != SYN_NONE):
+            out, syndromes, counts = _empty_for(max(4, words_for(num_codewords * self.k)), syn_type,
+                                                max(16, num_codewords), 2, stream_words.device, out, syndromes,
+                                                counts)
+        c = counts.data_ptr()
+        rc = lib().hd_decode_short_plan(self.handle, stream_words.data_ptr(), self.n * num_codewords, num_codewords,
+                                        out.data_ptr(), syndromes.data_ptr() if syn_type != SYN_NONE else None,
+                                        syn_type, c, c + 8, _stream_handle(cuda_stream))
         check(rc, "hd_decode_short_plan")
         return out, syndromes, counts
 
@@ -647,8 +667,8 @@ class ShortPlan:
 
 def encode_short(data_words, n: int, num_codewords: int, out=None, cuda_stream=None):
     """Encode a device tensor of packed messages into segments of length n."""
-    import torch
     if out is None:
+        import torch
         out = torch.empty(max(4, words_for(num_codewords * n)), dtype=torch.int32, device=data_words.device)
     check(hd_encode_short(_ptr(data_words), n, num_codewords, _ptr(out), _stream_handle(cuda_stream)),
           "hd_encode_short")
@@ -669,27 +689,22 @@ def decode_secded(stream_words, n: int, num_codewords: int, syn_type: int = SYN_
                   counts=None, cuda_stream=None):
     """Decode a device tensor of SECDED codewords (n + 1 bits each).  Returns
     (out_words, syndromes or None, counts) with counts = [nonzero syndromes, detected]."""
-    import torch
     m, k = code_params(n)
-    dev = stream_words.device
-    if out is None:
-        out = torch.empty(max(4, words_for(num_codewords * k)), dtype=torch.int32, device=dev)
-    if syndromes is None and syn_type != SYN_NONE:
-        dt = torch.uint8 if syn_type == SYN_U8 else torch.int16
-        syndromes = torch.empty(max(16, num_codewords), dtype=dt, device=dev)
-    if counts is None:
-        counts = torch.empty(2, dtype=torch.int64, device=dev)
-    rc = hd_decode_secded(_ptr(stream_words), (n + 1) * num_codewords, n, num_codewords, _ptr(out),
-                          _ptr(syndromes) if syn_type != SYN_NONE else None, syn_type, _ptr(counts),
-                          _ptr(counts) + 8, _stream_handle(cuda_stream))
+    if out is None or counts is None or (syndromes is None and syn_type != SYN_NONE):
+        out, syndromes, counts = _empty_for(max(4, words_for(num_codewords * k)), syn_type, max(16, num_codewords), 2,
+                                            stream_words.device, out, syndromes, counts)
+    c = counts.data_ptr()
+    rc = lib().hd_decode_secded(stream_words.data_ptr(), (n + 1) * num_codewords, n, num_codewords, out.data_ptr(),
+                                syndromes.data_ptr() if syn_type != SYN_NONE else None, syn_type, c, c + 8,
+                                _stream_handle(cuda_stream))
     check(rc, "hd_decode_secded")
     return out, syndromes, counts
 
 
 def encode_secded(data_words, n: int, num_codewords: int, out=None, cuda_stream=None):
     """Encode a device tensor of packed messages into SECDED codewords."""
-    import torch
     if out is None:
+        import torch
         out = torch.empty(max(4, words_for(num_codewords * (n + 1))), dtype=torch.int32, device=data_words.device)
     check(hd_encode_secded(_ptr(data_words), n, num_codewords, _ptr(out), _stream_handle(cuda_stream)),
           "hd_encode_secded")
@@ -698,8 +713,9 @@ def encode_secded(data_words, n: int, num_codewords: int, out=None, cuda_stream=
 
 def encode(data_words, n: int, num_codewords: int, out=None, cuda_stream=None):
     """Encode a device tensor of packed message bits; returns the stream words."""
-    import torch
     if out is None:
+        import torch
+        code_params(n)
         out = torch.empty(max(1, words_for(num_codewords * n)), dtype=torch.int32, device=data_words.device)
     check(hd_encode(_ptr(data_words), n, num_codewords, _ptr(out), _stream_handle(cuda_stream)), "hd_encode")
     return out
