@@ -230,8 +230,8 @@ hd_status hd_decode_short_plan(const hd_short_plan *plan, const uint32_t *stream
 /* Free a plan's tables (after the work that reads them has finished). */
 void hd_short_plan_destroy(hd_short_plan *plan);
 
-/* The tiled kernel is compiled in several configurations (warps per CTA,
- * pipeline stages, stage bytes).
+/* The tiled kernel has several configurations (warps per CTA, stage bytes);
+ * configuration 0 is the built-in choice by length and size.
  * hd_short_variant_select() pins one configuration for every length on the
  * current device (ordinal < 0 removes the pin); hd_short_autotune() times
  * every configuration on `num_codewords` all-zero segments of length n (reps

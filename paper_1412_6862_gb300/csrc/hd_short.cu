@@ -10,11 +10,12 @@
 // left as received.
 //
 // Two decoders:
-//  * k_short_tiles (n >= 960; any k >= 64 where a configuration is chosen): each warp streams tiles of g whole
-//    codewords through a ring of shared-memory stages filled by 1-D bulk
-//    copies.  Per tile: (1) syndromes, teams of T lanes per codeword (T from a
-//    cost model, 1..32), each lane folding its position-domain words four at a
-//    time, then one XOR over the team; the corrections flip bits in the stage.  (3) Every output word from a per-length table of
+//  * k_short_tiles (n >= 960; any k >= 64 where a configuration is chosen): each warp
+//    takes tiles of g whole codewords, one at a time, into a shared-memory stage of its
+//    own filled by a 1-D bulk copy (the next tile goes to L2 meanwhile).  Per tile:
+//    (1) syndromes, teams of T lanes per codeword (g, T and the warps from a cost model),
+//    each lane folding its stage words four at a time, then one XOR over the team; the
+//    corrections flip bits in the stage.  (3) Every output word from a per-length table of
 //    output-word offsets: a funnel shift (and, for short codewords, a merge at
 //    the word's checksum position), lane-strided so stage reads are
 //    conflict-free and stores coalesced.  (4) The words that hold a codeword's
@@ -62,41 +63,30 @@ struct ShortArgs {
     uint64_t ntiles;
     uint32_t n, k, g;   // code length, data bits, codewords per tile
     uint32_t Y;         // position-domain words per codeword: ceil((n + 1) / 32)
-    uint32_t ylast;     // valid-bit mask of the last position-domain word
     uint32_t tlog;      // log2 of the team size of the syndrome pass
     int syn_type;
     bool direct;        // one CTA that overwrites the counters
     uint32_t tab_len;       // entries of the output-word table (see output_table), 2 or 4 bytes each
     uint32_t nJ;            // data runs J >= 5 that end inside the codeword's data (D_J < k)
     uint32_t nJ_magic;      // ceil(2^32 / nJ) for nJ > 1: f / nJ = umulhi(f, nJ_magic) for the small f used
+    uint32_t stage;         // bytes of a warp's stage: the longest tile with its 16-byte rounding
 };
 
-template <int SB>
-struct TileGeom {
-    // stage: 16-byte guard word area (read as word -1), SB data bytes, 16 bytes of slack
-    static constexpr uint32_t stage_stride = SB + 32;
-    static constexpr uint32_t max_g = 256;
-};
+// A warp's shared memory: a 16-byte guard area (its last word is read as word -1), the
+// stage, 16 bytes of slack behind it, and the mbarrier.
+constexpr uint32_t kStageExtra = 48;
+constexpr uint32_t kMaxStage = 8192;
+constexpr int kTileWarps = 24;  // most warps of a CTA
+constexpr uint32_t kMaxTileCw = 256;
 
-// Codewords per tile: the tile's input plus 16-byte rounding at both ends fits SB bytes.
-template <int SB>
-inline uint32_t tile_codewords(uint32_t n)
+// Codewords per tile: the tile's input plus 16-byte rounding at both ends fits a stage.
+inline uint32_t tile_codewords(uint32_t stage, uint32_t n)
 {
-    const uint32_t g = (uint32_t)((8u * SB - 256u) / n);
-    return std::min<uint32_t>(g, TileGeom<SB>::max_g);
+    return std::min<uint32_t>((8u * stage - 256u) / n, kMaxTileCw);
 }
 
-// A decode's buffers: parameters of the kernels of their own, so that the
-// compiler knows them for global memory (a store through a struct's pointer
-// might alias the stage, and holds back the shared-memory loads behind it).
-struct ShortBuffers {
-    const uint32_t *in;
-    uint32_t *out;
-    void *syn;
-    unsigned long long *err;
-    unsigned long long *det;
-    const void *table;
-};
+// The stage of g codewords: their bits behind up to 127 others, in whole 16-byte pieces.
+inline uint32_t stage_bytes(uint32_t n, uint32_t g) { return (g * n + 254u) / 128u * 16u; }
 
 // Bytes of tile t that a bulk copy brings in, and where they start.
 __device__ __forceinline__ void tile_span(const ShortArgs &a, uint64_t t, uint64_t &byte0, uint32_t &bytes,
@@ -111,7 +101,6 @@ __device__ __forceinline__ void tile_span(const ShortArgs &a, uint64_t t, uint64
     bytes = byte1 > byte0 ? (uint32_t)(byte1 - byte0) : 0u;
 }
 
-template <int SB>
 __device__ __forceinline__ void issue_tile(const ShortArgs &a, const uint32_t *in, uint64_t t, uint8_t *stage,
                                            uint64_t *bar)
 {
@@ -181,59 +170,72 @@ __device__ __forceinline__ void add_counts(bool direct, unsigned long long *err,
     }
 }
 
-template <int W, int S, int SB, bool TAB_SMEM, bool SPLIT>
-__global__ void __launch_bounds__(W * 32)
+template <bool TAB_SMEM, bool SPLIT>
+__global__ void __launch_bounds__(kTileWarps * 32, 1)
     k_short_tiles(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, void *__restrict__ syn,
                   unsigned long long *__restrict__ err, unsigned long long *__restrict__ det,
                   const void *__restrict__ table, const ShortArgs a)
 {
-    using Geom = TileGeom<SB>;
     extern __shared__ __align__(128) uint8_t smem[];
-    constexpr uint32_t warp_bytes = S * Geom::stage_stride + 16 * S;
+    const uint32_t warp_bytes = a.stage + kStageExtra, W = blockDim.x >> 5;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the output-word table, copied once per CTA when it fits next to the stages
     // SPLIT: 32-bit entries that also say where a word's checksum position falls, resolved
     // in pass 3; otherwise 16-bit entries and pass 5 rewrites those words
     using Entry = typename std::conditional<SPLIT, uint32_t, uint16_t>::type;
     const Entry *tab = static_cast<const Entry *>(table);
-    if constexpr (TAB_SMEM) {
-        Entry *s_tab = reinterpret_cast<Entry *>(smem + W * warp_bytes);
-        for (uint32_t i = threadIdx.x; i < a.tab_len; i += W * 32) s_tab[i] = tab[i];
-        __syncthreads();
-        tab = s_tab;
-    }
     uint8_t *wbase = smem + warp * warp_bytes;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(wbase + S * Geom::stage_stride);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(wbase + a.stage + 32);
+    uint32_t *st = reinterpret_cast<uint32_t *>(wbase + 16);
     const uint64_t gw = (uint64_t)blockIdx.x * W + warp, tw = (uint64_t)gridDim.x * W;
 
     if (lane == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(&bar[s], 1);
+        mbar_init(bar, 1);
         fence_mbar_init();
-        for (int s = 0; s < S; ++s) {
-            const uint64_t t = gw + (uint64_t)s * tw;
-            if (t < a.ntiles) issue_tile<SB>(a, in, t, wbase + s * Geom::stage_stride, &bar[s]);
+        if (gw < a.ntiles) issue_tile(a, in, gw, wbase, bar);
+    }
+    // the output-word table next to the stages where it fits: one bulk copy per CTA, behind the
+    // first tiles and waited for before the first output words
+    uint64_t *tbar = nullptr;
+    if constexpr (TAB_SMEM) {
+        uint8_t *s_tab = smem + W * warp_bytes;
+        const uint32_t tab_bytes = (a.tab_len * (uint32_t)sizeof(Entry) + 15u) & ~15u;
+        tbar = reinterpret_cast<uint64_t *>(s_tab + tab_bytes);
+        if (threadIdx.x == 0) {
+            mbar_init(tbar, 1);
+            fence_mbar_init();
+            mbar_arrive_expect_tx(tbar, tab_bytes);
+            bulk_g2s(s_tab, table, tab_bytes, tbar);
         }
+        __syncthreads();
+        tab = reinterpret_cast<const Entry *>(s_tab);
     }
     __syncwarp();
 
     // syndrome teams: T lanes per codeword, G codewords per round
     const uint32_t tlog = a.tlog, T = 1u << tlog, tl = lane & (T - 1u), team = lane >> tlog, G = 32u >> tlog;
-    const uint32_t n = a.n, k = a.k, Ym1 = a.Y - 1u;
-    const int32_t stage_bits = 8 * SB;  // reads past the data stay inside the stage's slack
+    const uint32_t n = a.n, k = a.k;
+    const int32_t stage_bits = 8 * (int32_t)a.stage;  // reads past the data stay inside the stage's slack
     uint32_t errs = 0, dets = 0, it = 0;
     bool aborted = false;
     for (uint64_t t = gw; t < a.ntiles; t += tw, ++it) {
-        const int s = (int)(it % S);
-        const bool ok = mbar_wait_bounded(&bar[s], (it / S) & 1u);
+        bool ok = mbar_wait_bounded(bar, it & 1u);
+        if (TAB_SMEM && it == 0) ok = ok && mbar_wait_bounded(tbar, 0);
         if (__any_sync(0xFFFFFFFFu, !ok)) {
             aborted = true;
             break;
         }
-        uint8_t *stage = wbase + s * Geom::stage_stride;
-        uint32_t *st = reinterpret_cast<uint32_t *>(stage + 16);
         uint64_t byte0;
         uint32_t bytes, gcnt;
         tile_span(a, t, byte0, bytes, gcnt);
+        if (TAB_SMEM && lane == 0 && t + tw < a.ntiles) {
+            // the warp's next tile comes into the one stage when this one is done: into L2 meanwhile
+            // (n = 8013, 1 Gbit 45.3 -> 43.1 us; no gain with the table in global memory, 54.1/55.4)
+            uint64_t nb;
+            uint32_t nbytes, ncw;
+            tile_span(a, t + tw, nb, nbytes, ncw);
+            if (nbytes) bulk_prefetch_l2(reinterpret_cast<const uint8_t *>(in) + nb, nbytes);
+        }
         const uint64_t c0 = t * a.g;
         const uint32_t off0 = (uint32_t)((c0 * n) & 127u);
         {  // words past the last 16-byte boundary of the input arrive by plain loads
@@ -245,66 +247,57 @@ __global__ void __launch_bounds__(W * 32)
             }
         }
 
-        // 1. syndromes.  Lane tl of a team reads position-domain words j = tl + T*i, four at a
-        //    time (i = 4q + u): x is the XOR of all of them, A and B the XORs of those with bit 0
-        //    and bit 1 of u set, hq the XOR of the q whose four words have odd parity, so that
-        //    one popcount serves four words.  The low syndrome bits are parities of x, the high
-        //    ones the XOR of the indices j of the odd-parity words.
+        // 1. syndromes.  Lane tl of a team reads stage words r = tl + T*i of its codeword, four
+        //    at a time (i = 4q + u), as they lie: bit b of word r is position 32*r + b - sh, so the
+        //    word's bits from sh up belong to position-domain word r and those below to r - 1.
+        //    x is the XOR of all of the lane's words (rotated by sh at the end: every word's
+        //    rotation is the same), A and B the XORs of those with bit 0 and bit 1 of u set, hq
+        //    the XOR of the q whose four words have odd parity, so that one popcount serves four
+        //    words.  For tl > 0 word r - 1 has the same i, and only the low part of the index
+        //    differs; for tl = 0 the bits below sh count for i - 1 (mask lm).  The low syndrome
+        //    bits are parities of x, the high ones the XOR of the indices of the odd-parity words.
+        //    One load and no shift per word: with two loads and a funnel shift (position-domain
+        //    words) 900 Mbit of n = 3212 took 52.2 us, 49.6 so.
         for (uint32_t cbase = 0; cbase < gcnt; cbase += G) {
             const uint32_t c = cbase + team;
-            uint32_t x = 0, A = 0, B = 0, hq = 0;
+            uint32_t x = 0, A = 0, B = 0, hq = 0, lo = 0, lm = 0, sh = 0;
             if (c < gcnt) {
                 const int32_t q0 = (int32_t)(off0 + c * n) - 1;  // position 0 is bit -1 of c (the guard word for c = 0)
-                const uint32_t sh = (uint32_t)q0 & 31u;
+                sh = (uint32_t)q0 & 31u;
+                lo = (1u << sh) - 1u;
+                lm = tl == 0 ? lo : 0u;
+                const uint32_t rl = (n + sh) >> 5, last = 0xFFFFFFFFu >> (31u - ((n + sh) & 31u));  // last word, its bits
                 const uint32_t *ad = st + (q0 >> 5) + (int32_t)tl;
-                auto take = [&](const uint32_t (&v)[4], uint32_t q) {
-                    A ^= v[1] ^ v[3];
-                    B ^= v[2] ^ v[3];
-                    const uint32_t b = v[0] ^ v[1] ^ v[2] ^ v[3];
+                auto take = [&](uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, uint32_t v4, uint32_t q) {
+                    A ^= v1 ^ v3;
+                    B ^= v2 ^ v3;
+                    const uint32_t b = v0 ^ v1 ^ v2 ^ v3;
                     x ^= b;
-                    hq ^= q & (0u - (__popc(b) & 1u));
+                    hq ^= q & (0u - (__popc(b ^ ((v0 ^ v4) & lm)) & 1u));
                 };
-                uint32_t j = tl, q = 0;
+                // word r without the bits past position n
+                auto end = [&](uint32_t r, const uint32_t *p) { return r < rl ? *p : r == rl ? *p & last : 0u; };
+                uint32_t r = tl, q = 0;
+                uint32_t v0 = end(r, ad) & ~lm;  // not the bits before the codeword
                 // plain shared-memory loads, so that the compiler issues an unrolled
                 // iteration's loads ahead of their uses
-                if (T == 1u) {  // a lane's words are neighbours: each one's high half is the next one's low half
-                    uint32_t lo = ad[0];
 #pragma unroll 2
-                    for (; j + 3u < Ym1; j += 4u, ++q, ad += 4) {
-                        uint32_t v[4];
-#pragma unroll
-                        for (uint32_t u = 0; u < 4; ++u) {
-                            const uint32_t hi = ad[u + 1];
-                            v[u] = __funnelshift_r(lo, hi, sh);
-                            lo = hi;
-                        }
-                        take(v, q);
-                    }
-                } else {
-#pragma unroll 2
-                    for (; j + 3u * T < Ym1; j += 4u * T, ++q, ad += 4u * T) {
-                        uint32_t v[4];
-#pragma unroll
-                        for (uint32_t u = 0; u < 4; ++u) v[u] = __funnelshift_r(ad[u * T], ad[u * T + 1], sh);
-                        take(v, q);
-                    }
+                for (; r + 4u * T < rl; r += 4u * T, ++q, ad += 4u * T) {
+                    const uint32_t v1 = ad[T], v2 = ad[2u * T], v3 = ad[3u * T], v4 = ad[4u * T];
+                    take(v0, v1, v2, v3, v4, q);
+                    v0 = v4;
                 }
-                if (j <= Ym1) {  // the last one to four words; word Ym1 holds positions up to n only
-                    uint32_t v[4];
-#pragma unroll
-                    for (uint32_t u = 0; u < 4; ++u) {
-                        const uint32_t ju = j + u * T;
-                        v[u] = ju <= Ym1 ? __funnelshift_r(ad[u * T], ad[u * T + 1], sh) : 0u;
-                        if (ju == Ym1) v[u] &= a.ylast;
-                    }
-                    take(v, q);
-                }
+                const uint32_t v1 = end(r + T, ad + T), v2 = end(r + 2u * T, ad + 2u * T);
+                const uint32_t v3 = end(r + 3u * T, ad + 3u * T), v4 = end(r + 4u * T, ad + 4u * T);
+                take(v0, v1, v2, v3, v4, q);
+                take(v4, 0u, 0u, 0u, 0u, q + 1u);
             }
             // the lane's share in one word: the low bits' parities on bits 1, 2, 4, 8, 16 of x's
             // transform, the index bits from 17 up; XOR over the team (butterfly steps stay
             // inside aligned groups of T lanes)
-            const uint32_t hi = hq << 2 | (__popc(B) & 1u) << 1 | (__popc(A) & 1u);
-            uint32_t z = (superset_xor<5>(x) & 0x00010116u) | ((hi << tlog) ^ ((__popc(x) & 1u) ? tl : 0u)) << 17;
+            const uint32_t hi = hq << 2 | (__popc(B ^ ((x ^ A) & lm)) & 1u) << 1 | (__popc(A ^ (x & lm)) & 1u);
+            const uint32_t tsum = (0u - (__popc(x & ~lo) & 1u) & tl) ^ (0u - (__popc(x & lo) & 1u) & (tl - 1u) & (T - 1u));
+            uint32_t z = (superset_xor<5>(__funnelshift_r(x, x, sh)) & 0x00010116u) | ((hi << tlog) ^ tsum) << 17;
             if (T == 32u)
                 z = __reduce_xor_sync(0xFFFFFFFFu, z);
             else
@@ -434,17 +427,15 @@ __global__ void __launch_bounds__(W * 32)
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-            const uint64_t tn = t + (uint64_t)S * tw;
-            if (tn < a.ntiles) issue_tile<SB>(a, in, tn, stage, &bar[s]);
+            const uint64_t tn = t + tw;
+            if (tn < a.ntiles) issue_tile(a, in, tn, wbase, bar);
         }
         __syncwarp();
     }
     if (lane == 0 && aborted) {
         atomicOr(a.status, (uint32_t)HD_ERR_TIMEOUT);
-        for (uint32_t j = it; j < it + S; ++j) {
-            const uint64_t tj = gw + (uint64_t)j * tw;
-            if (tj < a.ntiles) (void)mbar_wait_bounded(&bar[j % S], (j / S) & 1u);
-        }
+        (void)mbar_wait_bounded(bar, it & 1u);  // the copies in flight
+        if (TAB_SMEM) (void)mbar_wait_bounded(tbar, 0);
     }
     add_counts(a.direct, err, det, errs, dets, reinterpret_cast<uint32_t *>(smem), warp_bytes / 4);
 }
@@ -558,58 +549,25 @@ __global__ void __launch_bounds__(kSmallWarps * 32)
 // Variant table of the tile kernel (compiled configurations).
 // ---------------------------------------------------------------------------
 struct ShortVariant {
-    int W, S, SB;
-    uint32_t stage_smem;  // dynamic shared memory of the warps' stages
-    // [0]: table in global memory; [1]: table in shared memory; [2]: shared, splits in pass 3
-    const void *kernel[3];
-    cudaError_t (*launch[3])(const ShortBuffers &, const ShortArgs &, int grid, uint32_t smem, cudaStream_t, bool pdl);
+    uint32_t warps, stage;  // per CTA (fewer where shared memory does not hold them); bytes of a warp's stage
 };
 
-template <int W, int S, int SB, bool TAB_SMEM, bool SPLIT>
-cudaError_t launch_tiles(const ShortBuffers &b, const ShortArgs &a, int grid, uint32_t smem, cudaStream_t st, bool pdl)
-{
-    return launch_kernel(k_short_tiles<W, S, SB, TAB_SMEM, SPLIT>, dim3((unsigned)grid), dim3(W * 32), smem, st, pdl,
-                         b.in, b.out, b.syn, b.err, b.det, b.table, a);
-}
-
-template <int W, int S, int SB>
-ShortVariant make_short_variant()
-{
-    constexpr uint32_t warp_bytes = S * TileGeom<SB>::stage_stride + 16 * S;
-    return ShortVariant{W,
-                        S,
-                        SB,
-                        W * warp_bytes,
-                        {reinterpret_cast<const void *>(k_short_tiles<W, S, SB, false, false>),
-                         reinterpret_cast<const void *>(k_short_tiles<W, S, SB, true, false>),
-                         reinterpret_cast<const void *>(k_short_tiles<W, S, SB, true, true>)},
-                        {&launch_tiles<W, S, SB, false, false>, &launch_tiles<W, S, SB, true, false>,
-                         &launch_tiles<W, S, SB, true, true>}};
-}
-
-const ShortVariant kShortVariants[] = {
-    // the built-in choice: fastest over the paper's (M, t) grid on GB300 (the
-    // kernel waits on fixed-latency chains, so warps per SM count: two of these
-    // CTAs hold 24 warps, two 8-warp CTAs of 4 KB stages only 16)
-    make_short_variant<12, 2, 4096>(),
-    make_short_variant<8, 2, 4096>(),
-    make_short_variant<4, 2, 8192>(),
-    make_short_variant<4, 3, 4096>(),
-    make_short_variant<4, 4, 2048>(),
-    make_short_variant<16, 2, 2048>(),
-    make_short_variant<16, 2, 3072>(),
-};
+// [0]: the built-in choice.  One CTA of 24 warps shares one output-word table; where that stays in
+// global memory (n > about 18,500) two CTAs of 16 warps (n = 24,000, 900 Mbit: 54.5 us with 24
+// warps in one CTA, 49.4 with 16 in two).
+// A warp's tile costs the same few chains (wait, transform, butterfly, heads) whatever its
+// size, so one 8 KB stage beats two of 4 KB: 900 Mbit of n = 3212 in 52.2 us with two, n = 8013
+// in 55.9, n = 12,000 in 68.6, against 43.6, 44.5 and 51.1 with one.
+const ShortVariant kShortVariants[] = {{0, 0}, {24, 8192}, {24, 6144}, {16, 6144}, {16, 4096}, {12, 4096}, {8, 8192}};
+const ShortVariant kSharedTable = {24, 8192}, kGlobalTable = {16, 7168};
 constexpr int kNumShortVariants = sizeof(kShortVariants) / sizeof(kShortVariants[0]);
 
-// The configuration with the largest stages (the first of them), which holds a
-// codeword of every supported length.
-int largest_stage_variant()
-{
-    int best = 0;
-    for (int v = 1; v < kNumShortVariants; ++v)
-        if (kShortVariants[v].SB > kShortVariants[best].SB) best = v;
-    return best;
-}
+using TileKernel = void (*)(const uint32_t *, uint32_t *, void *, unsigned long long *, unsigned long long *,
+                            const void *, ShortArgs);
+// [0]: table in global memory; [1]: table in shared memory; [2]: shared, splits in pass 3
+const TileKernel kTileKernels[3] = {k_short_tiles<false, false>, k_short_tiles<true, false>, k_short_tiles<true, true>};
+
+constexpr uint32_t kSmemPerCta = 227u << 10;
 constexpr uint32_t kTabSmemMax = 40u << 10;  // larger tables stay in global memory
 
 std::mutex g_short_mu;
@@ -621,35 +579,34 @@ struct TunedEntry {
 TunedEntry g_short_tuned[64][64];  // per device: the autotuner's choice per length
 
 struct OccEntry {
-    int v = -1, tsm = 0;
-    uint32_t smem = 0;
+    int tsm = -1;
+    uint32_t warps = 0, smem = 0;
     int bps = 0;
 };
 OccEntry g_occ[64][32];
 
-// Resident CTAs per SM of configuration v with `smem` bytes of dynamic shared memory.
-int short_blocks_per_sm(int v, int tsm, uint32_t smem)
+// Resident CTAs per SM of tile kernel tsm with `warps` warps and `smem` bytes of dynamic shared memory.
+int short_blocks_per_sm(int tsm, uint32_t warps, uint32_t smem)
 {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
     std::lock_guard<std::mutex> lk(g_short_mu);
     for (const OccEntry &e : g_occ[dev])
-        if (e.v == v && e.tsm == tsm && e.smem == smem) return e.bps;
-    const ShortVariant &sv = kShortVariants[v];
+        if (e.tsm == tsm && e.warps == warps && e.smem == smem) return e.bps;
+    const void *kern = reinterpret_cast<const void *>(kTileKernels[tsm]);
     // the attribute is per kernel: allow the device's largest opt-in size once, never a smaller one
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         (uint32_t)optin < smem ||
-        cudaFuncSetAttribute(sv.kernel[tsm], cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
         return -1;
     int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, sv.kernel[tsm], sv.W * 32, smem) != cudaSuccess ||
-        bps <= 0)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, (int)warps * 32, smem) != cudaSuccess || bps <= 0)
         return -1;
     for (OccEntry &e : g_occ[dev])
-        if (e.v < 0) {
-            e = OccEntry{v, tsm, smem, bps};
+        if (e.tsm < 0) {
+            e = OccEntry{tsm, warps, smem, bps};
             break;
         }
     return bps;
@@ -689,26 +646,63 @@ void remember_short_variant(uint32_t n, int v)
     slot->v = v;
 }
 
-// Team size of the syndrome pass: a team of T lanes reads a codeword's Y
-// position-domain words, ceil(Y / 4T) blocks of four per lane, and a tile's
-// codewords take ceil(g / (32 / T)) rounds, each of which ends in a chain of
-// dependent steps (the transform, the butterfly over the team, the correction).
-// The weights follow the times of every T at 18 lengths on GB300 (1 Gbit, T = 1 ..
-// 16: n = 1078 65/73/87/107/146 us, n = 3212 71/59/64/67/76, n = 8013
-// 128/91/73/66/75); the pick is the fastest at all of them.
-uint32_t team_log(uint32_t Y, uint32_t g)
+// Syndrome pass of a tile of g codewords: a team of T = 2^lg lanes reads a codeword's Y
+// words, ceil(Y / 4T) blocks of four per lane, and the tile's codewords take
+// ceil(g / (32 / T)) rounds, each of which ends in a chain of dependent steps (the
+// transform, the butterfly over the team, the correction).  The weights follow the times
+// of every T at 18 lengths on GB300 (1 Gbit, T = 1 .. 16: n = 1078 65/73/87/107/146 us,
+// n = 3212 71/59/64/67/76, n = 8013 128/91/73/66/75); the least cost is the fastest at all
+// of them.
+uint64_t team_cost(uint32_t Y, uint32_t g, uint32_t *tlog)
 {
-    uint32_t best = 5;
-    uint64_t best_cost = ~0ull;
+    uint64_t best = ~0ull;
     for (uint32_t lg = 0; lg <= 5; ++lg) {
-        const uint32_t T = 1u << lg, G = 32u >> lg;
-        const uint64_t cost = (uint64_t)((g + G - 1) / G) * ((Y + 4 * T - 1) / (4 * T) * 40 + 160 + 20 * lg);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = lg;
+        const uint32_t rounds = (g + (32u >> lg) - 1) >> (5 - lg), blocks = (Y + (4u << lg) - 1) >> (lg + 2);
+        const uint64_t cost = (uint64_t)rounds * (blocks * 40 + 160 + 20 * lg);
+        if (cost < best) {
+            best = cost;
+            *tlog = lg;
         }
     }
     return best;
+}
+
+// How a stream is cut: codewords per tile (at most gmax), the team size for them, and the
+// warps per CTA (W, at most the configuration's; lowered in steps of two to w_min).  All
+// warps work through their tiles in step, so the last of the R rounds of tiles should be as
+// full as the others, g = ceil(num_cw / (R * warps)), and the g codewords should fill the
+// lanes of the syndrome teams (n = 3212: g = 20 takes two rounds of T = 2, g = 16 one).
+// The cost is R times a tile's, which grows with the warps that share the SM (0.2 + 0.8 W /
+// 24, fitted).  On GB300 at nine lengths of 961 .. 3212 and four sizes of 0.2 .. 0.5 Gbit the
+// pick is 5 % faster on average than 24 warps in the smallest R (n = 1100, 244,032
+// codewords: 24.9 -> 21.6 us; n = 1611, 124,146: 16.7 -> 14.2; at worst 1.8 % slower), and
+// the fastest choice of W and R 5.7 %.  A stream of one codeword per warp or less spreads over
+// the whole GPU.
+struct TileShape {
+    uint32_t g, tlog, warps;
+};
+
+TileShape tile_shape(uint32_t Y, uint32_t gmax, uint64_t num_cw, uint64_t ctas, uint32_t w_max, uint32_t w_min)
+{
+    TileShape pick{1, 0, w_max};
+    if (num_cw <= ctas * w_max) {
+        team_cost(Y, 1, &pick.tlog);
+        return pick;
+    }
+    uint64_t best = ~0ull;
+    for (int w = (int)w_max; w >= (int)w_min; w -= 2) {
+        const uint64_t warps = ctas * (uint32_t)w, r0 = (num_cw + gmax * warps - 1) / (gmax * warps);
+        for (uint64_t R = r0; R < r0 + 3; ++R) {
+            const uint32_t g = (uint32_t)((num_cw + R * warps - 1) / (R * warps));
+            uint32_t lg = 0;
+            const uint64_t cost = R * (team_cost(Y, g, &lg) + 100) * (uint32_t)(w + 6);
+            if (cost < best) {
+                best = cost;
+                pick = TileShape{g, lg, (uint32_t)w};
+            }
+        }
+    }
+    return pick;
 }
 
 // Output-word offsets: entry idx describes output word idx of a run of
@@ -752,8 +746,9 @@ bool split_in_pass3(uint32_t k) { return k < 1280; }
 cudaError_t build_short_table(uint32_t n, uint32_t k, void **dev, uint32_t *len)
 {
     // the longest tile of any configuration: the largest stage's codewords, plus a partial word
-    const uint32_t max_words = (uint32_t)(((uint64_t)tile_codewords<8192>(n) * k + 31) / 32) + 1;
-    const std::vector<uint32_t> full = output_table(n, k, max_words);
+    const uint32_t max_words = (uint32_t)(((uint64_t)tile_codewords(kMaxStage, n) * k + 31) / 32) + 1;
+    std::vector<uint32_t> full = output_table(n, k, max_words);
+    full.resize((full.size() + 7) / 8 * 8, 0);  // whole 16-byte pieces for the kernels' bulk copy
     const bool wide = split_in_pass3(k);
     std::vector<uint16_t> narrow;
     if (!wide)
@@ -870,24 +865,18 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
                                int syn_type, unsigned long long *err, unsigned long long *det, cudaStream_t st,
                                const void *table, uint32_t tab_len, bool bare)
 {
-    const ShortVariant &v = kShortVariants[vi];
     const uint32_t r = short_r(n), k = n - r;
     ShortArgs a{};
-    const ShortBuffers buf{in, out, syn, err, det, table};
     a.status = status_ptr();
     if (!a.status) return cudaErrorUnknown;
+    if (!table) return cudaErrorInvalidValue;
     a.num_cw = num_cw;
     a.in_words = words_for_bits(num_cw * n);
     a.bulk_end = (a.in_words * 4) >> 4 << 4;
     a.n = n;
     a.k = k;
-    a.g = std::min<uint32_t>((8u * v.SB - 256u) / n, TileGeom<4096>::max_g);  // as tile_codewords<SB>
-    if (a.g == 0) return cudaErrorInvalidValue;  // the caller picks a configuration whose stage holds a codeword
     a.Y = (n + 32) / 32;
-    const uint32_t lastbits = n + 1 - 32 * (a.Y - 1);
-    a.ylast = lastbits >= 32 ? 0xFFFFFFFFu : (1u << lastbits) - 1u;
     a.tab_len = tab_len;
-    if (!table) return cudaErrorInvalidValue;
     a.syn_type = syn ? syn_type : 0;
     a.nJ = 0;
     for (uint32_t J = 5; (2u << J) - J - 2u < k; ++J) ++a.nJ;
@@ -895,21 +884,30 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     const bool split = split_in_pass3(k);
     const uint32_t tab_bytes = (a.tab_len * (split ? 4u : 2u) + 15) & ~15u;
     const int tsm = split ? 2 : (tab_bytes <= kTabSmemMax ? 1 : 0);  // split tables are small
-    const uint32_t smem = v.stage_smem + (tsm ? tab_bytes : 0u);
     if (split) a.nJ = 0;  // no per-codeword pass for checksum words
-    const int bps = short_blocks_per_sm(vi, tsm, smem);
+    const uint32_t tab_smem = tsm ? tab_bytes + 16u : 0u;  // with its mbarrier
+    const ShortVariant v = vi > 0 ? kShortVariants[vi] : tsm ? kSharedTable : kGlobalTable;
+    const uint32_t gmax = tile_codewords(v.stage, n);
+    if (gmax == 0) return cudaErrorInvalidValue;  // the caller picks a configuration whose stage holds a codeword
+    a.stage = stage_bytes(n, gmax);
+    const uint32_t w_max = std::min(v.warps, (kSmemPerCta - tab_smem) / (a.stage + kStageExtra));
+    const int bps = short_blocks_per_sm(tsm, w_max, w_max * (a.stage + kStageExtra) + tab_smem);
     if (bps <= 0) return cudaErrorInvalidConfiguration;
-    const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps, warps = cap * (uint64_t)v.W;
-    // Even tiles: no more codewords per tile than give every resident warp as many tiles
-    // (160,000 segments of n = 3212: 16,000 tiles of 10 were 4.4 rounds of 3648 warps), down
-    // to one codeword per tile for short streams, which then spread over the whole GPU.
-    const uint64_t rounds = (num_cw + a.g * warps - 1) / (a.g * warps);
-    a.g = (uint32_t)((num_cw + rounds * warps - 1) / (rounds * warps));
+    const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
+    // the built-in choice for shared tables varies the warps, a pinned configuration does not
+    const TileShape shape = tile_shape(a.Y, gmax, num_cw, cap, w_max, vi > 0 || !tsm ? w_max : std::min(w_max, 14u));
+    uint32_t W = shape.warps;
+    a.g = shape.g;
+    a.tlog = shape.tlog;
     a.ntiles = (num_cw + a.g - 1) / a.g;
-    a.tlog = team_log(a.Y, a.g);
-    const int grid = decode_grid((a.ntiles + v.W - 1) / v.W, cap);
+    a.stage = stage_bytes(n, a.g);
+    // at most one tile per warp: the warps spread over all SMs, or stay in one CTA (direct counts)
+    if (a.ntiles > W) W = (uint32_t)std::min<uint64_t>(W, (a.ntiles + cap - 1) / cap);
+    const uint32_t smem = W * (a.stage + kStageExtra) + tab_smem;
+    const int grid = decode_grid((a.ntiles + W - 1) / W, cap);
     return launch_counted(a.direct, err, det, grid, bare, st, [&](bool pdl) {
-        return v.launch[tsm](buf, a, grid, smem, st, pdl);
+        return launch_kernel(kTileKernels[tsm], dim3((unsigned)grid), dim3(W * 32), smem, st, pdl, in, out, syn, err,
+                             det, table, a);
     });
 }
 
@@ -1017,7 +1015,7 @@ hd_status decode_short_with(const uint32_t *stream, uint64_t in_bits, uint32_t n
                    ? HD_OK
                    : HD_ERR_CUDA;
     if (vi < 0) vi = 0;  // the built-in configuration
-    if (kShortVariants[vi].SB * 8u < n + 256u) vi = largest_stage_variant();  // stage too small for a codeword
+    if (vi > 0 && kShortVariants[vi].stage * 8u < n + 256u) vi = 0;  // stage too small for a codeword
     return launch_short_tiles(vi, stream, n, num_codewords, out_bits, syndromes, syn, err_count, detected_count, st,
                               table, tab_len, false) == cudaSuccess
                ? HD_OK
@@ -1144,7 +1142,7 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
     TableEntry *tab = nullptr;
     if (rc == HD_OK && table_for(n, k, st, &tab) != cudaSuccess) rc = HD_ERR_CUDA;
     for (int v = 0; rc == HD_OK && v < kNumShortVariants; ++v) {
-        if (kShortVariants[v].SB * 8u < n + 256u) continue;
+        if (v > 0 && kShortVariants[v].stage * 8u < n + 256u) continue;
         auto go = [&]() {
             return launch_short_tiles(v, static_cast<const uint32_t *>(din), n, num_codewords,
                                       static_cast<uint32_t *>(dout), dsyn, HD_SYN_U16, cnt, cnt + 1, st, tab->dev,
