@@ -25,6 +25,7 @@
 //    memory, one codeword per lane.
 // The encoder is in hd_short_encode.cu.
 #include <algorithm>
+#include <array>
 #include <cstdint>
 #include <mutex>
 #include <new>
@@ -62,7 +63,6 @@ struct ShortArgs {
     uint64_t bulk_end;  // bytes of the input that 16-byte bulk copies may read
     uint64_t ntiles;
     uint32_t n, k, g;   // code length, data bits, codewords per tile
-    uint32_t Y;         // position-domain words per codeword: ceil((n + 1) / 32)
     uint32_t tlog;      // log2 of the team size of the syndrome pass
     int syn_type;
     bool direct;        // one CTA that overwrites the counters
@@ -646,6 +646,26 @@ void remember_short_variant(uint32_t n, int v)
     slot->v = v;
 }
 
+// Words of the fullest shared-memory bank when a warp's teams of 2^lg lanes read the same
+// word of their codewords, per lg (it depends on n modulo 32 words).
+using BankWays = std::array<uint8_t, 6>;
+
+const BankWays &bank_ways(uint32_t n)
+{
+    static const std::array<BankWays, 1024> table = [] {
+        std::array<BankWays, 1024> t{};
+        for (uint32_t m = 0; m < 1024; ++m)
+            for (uint32_t lg = 0; lg <= 5; ++lg) {
+                uint8_t words[32] = {}, most = 0;
+                for (uint32_t l = 0; l < 32; ++l)
+                    most = std::max(most, ++words[(((l >> lg) * (1024 + m) >> 5) + (l & ((1u << lg) - 1u))) & 31u]);
+                t[m][lg] = most;
+            }
+        return t;
+    }();
+    return table[n % 1024];
+}
+
 // Syndrome pass of a tile of g codewords: a team of T = 2^lg lanes reads a codeword's Y
 // words, ceil(Y / 4T) blocks of four per lane, and the tile's codewords take
 // ceil(g / (32 / T)) rounds, each of which ends in a chain of dependent steps (the
@@ -653,12 +673,18 @@ void remember_short_variant(uint32_t n, int v)
 // of every T at 18 lengths on GB300 (1 Gbit, T = 1 .. 16: n = 1078 65/73/87/107/146 us,
 // n = 3212 71/59/64/67/76, n = 8013 128/91/73/66/75); the least cost is the fastest at all
 // of them.
-uint64_t team_cost(uint32_t Y, uint32_t g, uint32_t *tlog)
+// A block's loads cost more than its arithmetic where the warp's 32 words share few banks
+// (codewords a multiple of 32 words apart): weight 10 per word of the fullest bank, fitted
+// to every T at 25 lengths, four of them so (1 Gbit of n = 1024: 171 us without the term, 89 with
+// it, 2047 134 / 73, 4095 99 / 58; lengths whose fullest bank has up to four words keep their T).
+uint64_t team_cost(uint32_t n, uint32_t g, uint32_t *tlog)
 {
+    const uint32_t Y = (n + 32) / 32;
+    const BankWays &ways = bank_ways(n);
     uint64_t best = ~0ull;
     for (uint32_t lg = 0; lg <= 5; ++lg) {
         const uint32_t rounds = (g + (32u >> lg) - 1) >> (5 - lg), blocks = (Y + (4u << lg) - 1) >> (lg + 2);
-        const uint64_t cost = (uint64_t)rounds * (blocks * 40 + 160 + 20 * lg);
+        const uint64_t cost = (uint64_t)rounds * (blocks * std::max(40u, 10u * ways[lg]) + 160 + 20 * lg);
         if (cost < best) {
             best = cost;
             *tlog = lg;
@@ -682,11 +708,11 @@ struct TileShape {
     uint32_t g, tlog, warps;
 };
 
-TileShape tile_shape(uint32_t Y, uint32_t gmax, uint64_t num_cw, uint64_t ctas, uint32_t w_max, uint32_t w_min)
+TileShape tile_shape(uint32_t n, uint32_t gmax, uint64_t num_cw, uint64_t ctas, uint32_t w_max, uint32_t w_min)
 {
     TileShape pick{1, 0, w_max};
     if (num_cw <= ctas * w_max) {
-        team_cost(Y, 1, &pick.tlog);
+        team_cost(n, 1, &pick.tlog);
         return pick;
     }
     uint64_t best = ~0ull;
@@ -695,7 +721,7 @@ TileShape tile_shape(uint32_t Y, uint32_t gmax, uint64_t num_cw, uint64_t ctas, 
         for (uint64_t R = r0; R < r0 + 3; ++R) {
             const uint32_t g = (uint32_t)((num_cw + R * warps - 1) / (R * warps));
             uint32_t lg = 0;
-            const uint64_t cost = R * (team_cost(Y, g, &lg) + 100) * (uint32_t)(w + 6);
+            const uint64_t cost = R * (team_cost(n, g, &lg) + 100) * (uint32_t)(w + 6);
             if (cost < best) {
                 best = cost;
                 pick = TileShape{g, lg, (uint32_t)w};
@@ -875,7 +901,6 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     a.bulk_end = (a.in_words * 4) >> 4 << 4;
     a.n = n;
     a.k = k;
-    a.Y = (n + 32) / 32;
     a.tab_len = tab_len;
     a.syn_type = syn ? syn_type : 0;
     a.nJ = 0;
@@ -895,7 +920,7 @@ cudaError_t launch_short_tiles(int vi, const uint32_t *in, uint32_t n, uint64_t 
     if (bps <= 0) return cudaErrorInvalidConfiguration;
     const uint64_t cap = (uint64_t)num_sms() * (uint64_t)bps;
     // the built-in choice for shared tables varies the warps, a pinned configuration does not
-    const TileShape shape = tile_shape(a.Y, gmax, num_cw, cap, w_max, vi > 0 || !tsm ? w_max : std::min(w_max, 14u));
+    const TileShape shape = tile_shape(n, gmax, num_cw, cap, w_max, vi > 0 || !tsm ? w_max : std::min(w_max, 14u));
     uint32_t W = shape.warps;
     a.g = shape.g;
     a.tlog = shape.tlog;
