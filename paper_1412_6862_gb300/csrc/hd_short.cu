@@ -10,7 +10,7 @@
 // left as received.
 //
 // Two decoders:
-//  * k_short_tiles (n >= 960; any k >= 64 where a configuration is chosen): each warp
+//  * k_short_tiles (n >= 960, large streams from n = 768; any k >= 64 where a configuration is chosen): each warp
 //    takes tiles of g whole codewords, one at a time, into a shared-memory stage of its
 //    own filled by a 1-D bulk copy (the next tile goes to L2 meanwhile).  Per tile:
 //    (1) syndromes, teams of T lanes per codeword (g, T and the warps from a cost model),
@@ -42,10 +42,13 @@ namespace {
 
 constexpr uint32_t kShortMaxN = 32767;  // r <= 15: syndromes fit 16 bits
 constexpr uint32_t kLongMinK = 64;      // k_short_tiles needs the first 58 data bits inside one codeword
-// Lengths below it are decoded one codeword per lane.  On GB300, 1 Gbit with u16
-// syndromes, lanes against tiles: n = 100 90/145 us, 250 54/91, 400 54/86, 544 57/75,
-// 650 63/71, 810 64/72, 900 70/79, 1000 76/64; 100,000 bits of n = 544 3.0/4.8.
+// Lengths below kLaneMaxN are decoded one codeword per lane, except large streams from
+// kLaneTileN on.  On GB300 with u16 syndromes, lanes against tiles: 1 Gbit of n = 400 55/76 us,
+// 544 58/68, 650 63/61, 700 60/66, 768 74/66, 850 67/62, 959 71/60; 256 Mbit of n = 768 24.5/23.5, 850
+// 23.0/21.5, 959 24.0/22.7; 32 Mbit of n = 900 5.8/6.6; 20,000 bits of n = 850 3.6/4.8.
 constexpr uint32_t kLaneMaxN = 960;
+constexpr uint32_t kLaneTileN = 768;
+constexpr uint64_t kLaneTileBits = 1ull << 28;
 
 __host__ __device__ inline uint32_t short_r(uint32_t n)
 {
@@ -1034,7 +1037,7 @@ hd_status decode_short_with(const uint32_t *stream, uint64_t in_bits, uint32_t n
     // the tiled kernel from kLaneMaxN on, and below it (k >= 64) where a configuration is
     // pinned or the autotuner found one faster
     int vi = k >= kLongMinK ? chosen_short_variant(n) : -1;
-    if (vi < 0 && n < kLaneMaxN)
+    if (vi < 0 && n < kLaneMaxN && (n < kLaneTileN || num_codewords * n < kLaneTileBits))
         return launch_short_lanes(stream, n, num_codewords, out_bits, syndromes, syn, err_count, detected_count, st,
                                   false) == cudaSuccess
                    ? HD_OK

@@ -49,9 +49,10 @@ def test_stream_lengths(n, N, cap):
 
 # the edges of the tiles: all codewords in one CTA or one tile per warp of every SM (24 | 25,
 # 3648 | 3649 codewords), more than one round, the last table in shared memory and the first in
-# global memory (18,600 | 18,700), two codewords per stage there or one (28,544 | 28,545)
+# global memory (18,600 | 18,700), lanes and tiles of a large stream (768), two codewords per stage there or one (28,544 | 28,545)
 @pytest.mark.parametrize("n,N", [(961, 24), (1023, 25), (1024, 3648), (1100, 40_001), (1500, 160_001), (2047, 3649),
                                  (2048, 7300), (4095, 7297), (4096, 20_011), (12_000, 3649), (18_600, 3649),
+                                 (768, 349_520), (768, 349_527), (959, 280_001),
                                  (1023, 70_001), (1536, 50_001), (2048, 40_001), (8191, 9001),
                                  (18_600, 4001), (18_700, 4001), (28_544, 5003), (28_545, 5003), (32_767, 4865)])
 def test_tile_shapes(n, N):
