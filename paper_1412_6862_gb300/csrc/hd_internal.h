@@ -2,6 +2,7 @@
 // libhd.so.  Not installed; the public interface is include/hd.h.
 #pragma once
 
+#include <array>
 #include <atomic>
 #include <cstdint>
 #include <utility>
@@ -68,6 +69,11 @@ cudaError_t launch_encode(const uint32_t *data, uint64_t data_words, uint32_t n,
                           uint64_t stream_words, cudaStream_t st);
 cudaError_t launch_encode_secded(const uint32_t *data, uint64_t data_words, uint32_t n, uint64_t num_cw,
                                  uint32_t *stream, cudaStream_t st);
+
+// Words of the fullest shared-memory bank when a warp's teams of 2^lg lanes read the same
+// word of segments `bits` apart, per lg.
+using BankWays = std::array<uint8_t, 6>;
+const BankWays &bank_ways(uint32_t bits);
 
 cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, uint64_t num_cw, uint32_t *stream,
                                 cudaStream_t st);

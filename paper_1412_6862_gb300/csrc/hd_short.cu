@@ -38,6 +38,24 @@
 #include "hd_lane.cuh"
 
 namespace hd {
+
+// It depends on the distance modulo 32 words.
+const BankWays &bank_ways(uint32_t bits)
+{
+    static const std::array<BankWays, 1024> table = [] {
+        std::array<BankWays, 1024> t{};
+        for (uint32_t m = 0; m < 1024; ++m)
+            for (uint32_t lg = 0; lg <= 5; ++lg) {
+                uint8_t words[32] = {}, most = 0;
+                for (uint32_t l = 0; l < 32; ++l)
+                    most = std::max(most, ++words[(((l >> lg) * (1024 + m) >> 5) + (l & ((1u << lg) - 1u))) & 31u]);
+                t[m][lg] = most;
+            }
+        return t;
+    }();
+    return table[bits % 1024];
+}
+
 namespace {
 
 constexpr uint32_t kShortMaxN = 32767;  // r <= 15: syndromes fit 16 bits
@@ -647,26 +665,6 @@ void remember_short_variant(uint32_t n, int v)
     if (!slot) slot = &g_short_tuned[dev][n % 64];  // table full: overwrite one entry
     slot->n = n;
     slot->v = v;
-}
-
-// Words of the fullest shared-memory bank when a warp's teams of 2^lg lanes read the same
-// word of their codewords, per lg (it depends on n modulo 32 words).
-using BankWays = std::array<uint8_t, 6>;
-
-const BankWays &bank_ways(uint32_t n)
-{
-    static const std::array<BankWays, 1024> table = [] {
-        std::array<BankWays, 1024> t{};
-        for (uint32_t m = 0; m < 1024; ++m)
-            for (uint32_t lg = 0; lg <= 5; ++lg) {
-                uint8_t words[32] = {}, most = 0;
-                for (uint32_t l = 0; l < 32; ++l)
-                    most = std::max(most, ++words[(((l >> lg) * (1024 + m) >> 5) + (l & ((1u << lg) - 1u))) & 31u]);
-                t[m][lg] = most;
-            }
-        return t;
-    }();
-    return table[n % 1024];
 }
 
 // Syndrome pass of a tile of g codewords: a team of T = 2^lg lanes reads a codeword's Y

@@ -16,10 +16,10 @@
 // one bulk copy into the warp's stage (plain loads spread over several segments
 // kept the L1 busy at 75 % of its wavefronts and took 1.4 to 2 times as long); the
 // stage is free once pass 1 has read it, so the next tile's copy runs behind pass
-// 2 and one stage a warp suffices: 27 warps an SM.  Measured on GB300, 512 Mbit of
-// segments, of the measured copy bandwidth: n = 100 / 544 / 1078 / 3212 / 16000 /
-// 32767: 0.34 / 0.45 / 0.43 / 0.49 / 0.65 / 0.78 (bit by bit before: 0.01); below
-// n = 64, where a stream word holds parts of several segments, 0.07 to 0.2.
+// 2 and one stage a warp suffices.  Measured on GB300, 512 Mbit of segments, of the measured
+// copy bandwidth: n = 100 / 544 / 1078 / 3212 / 16000 / 32767: 0.36 / 0.48 / 0.43 / 0.66 / 0.70 / 0.82
+// (bit by bit before: 0.01); below n = 64, where a stream word holds parts of several
+// segments, 0.08 to 0.23.
 #include <algorithm>
 #include <cstdint>
 
@@ -30,8 +30,8 @@
 namespace hd {
 namespace {
 
-constexpr int kWarps = 8;
-constexpr uint32_t kAreaWords = 1056;  // position-domain words a warp holds: n = 32767 fits
+constexpr uint32_t kWarps = 24;       // most warps of a CTA, one CTA per SM
+constexpr uint32_t kSmemPerCta = 227u << 10;
 constexpr uint32_t kMaxTile = 256;     // segments per tile
 
 struct EncShortArgs {
@@ -40,15 +40,22 @@ struct EncShortArgs {
     uint32_t n, k, g;          // segment length, message bits, segments per tile
     uint32_t Y, ylast;         // position-domain words per segment, valid bits of the last one
     uint32_t ystride;          // words between two segments' position domains (odd, at least Y + 1)
+    uint32_t off_area, warp_bytes;
 };
 
 __device__ __forceinline__ uint32_t low_bits(uint32_t b) { return b >= 32 ? 0xFFFFFFFFu : (1u << b) - 1u; }
 
-// Per-warp shared memory: the barrier, the message stage (a tile's bits plus the
-// rounding to 16 bytes at both ends) and the position-domain words.
-constexpr uint32_t kStageBytes = (kAreaWords * 4 + 32 + 15) / 16 * 16;
-constexpr uint32_t kOffStage = 16, kOffArea = kOffStage + kStageBytes + 16;  // slack for the last window
-constexpr uint32_t kWarpBytes = (kOffArea + kAreaWords * 4 + 15) / 16 * 16;
+// A warp's shared memory: the barrier, the message stage (a tile's bits behind up to 127
+// others, in whole 16-byte pieces, and slack for the last window) and the
+// position-domain words of g segments.
+constexpr uint32_t kOffStage = 16;
+
+inline uint32_t area_offset(uint32_t k, uint32_t g) { return kOffStage + (g * k + 254u) / 128u * 16u + 16u; }
+
+inline uint32_t warp_smem(uint32_t k, uint32_t ystride, uint32_t g)
+{
+    return (area_offset(k, g) + g * ystride * 4u + 15u) / 16u * 16u;
+}
 
 // Pass 1 for one segment per team: the lane's position-domain words tl + T*i
 // into `y` and their fold.  x is the XOR of the words; h the XOR of the
@@ -128,14 +135,14 @@ __device__ __forceinline__ void fold_segment(const uint32_t *st, int32_t bit0, u
 
 // TLOG: log2 of the team size, so that a lane's word strides are constants.
 template <int TLOG>
-__global__ void __launch_bounds__(kWarps * 32) k_encode_short(const uint32_t *__restrict__ data, uint32_t *__restrict__ stream, const EncShortArgs a)
+__global__ void __launch_bounds__(kWarps * 32, 1) k_encode_short(const uint32_t *__restrict__ data, uint32_t *__restrict__ stream, const EncShortArgs a)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint8_t *wbase = smem + warp * kWarpBytes;
+    uint8_t *wbase = smem + warp * a.warp_bytes;
     uint64_t *bar = reinterpret_cast<uint64_t *>(wbase);
     uint32_t *stage = reinterpret_cast<uint32_t *>(wbase + kOffStage);
-    uint32_t *area = reinterpret_cast<uint32_t *>(wbase + kOffArea);
+    uint32_t *area = reinterpret_cast<uint32_t *>(wbase + a.off_area);
     constexpr uint32_t T = 1u << TLOG, G = 32u >> TLOG;
     const uint32_t tl = lane & (T - 1u), team = lane >> TLOG;
     const uint32_t n = a.n, k = a.k, Y = a.Y, ys = a.ystride;
@@ -158,8 +165,9 @@ __global__ void __launch_bounds__(kWarps * 32) k_encode_short(const uint32_t *__
         mbar_arrive_expect_tx(bar, bytes);
         if (bytes) bulk_g2s(stage, reinterpret_cast<const uint8_t *>(data) + byte0, bytes, bar);
     };
-    const uint64_t tw = (uint64_t)gridDim.x * kWarps;
-    uint64_t t = (uint64_t)blockIdx.x * kWarps + warp;
+    const uint32_t W = blockDim.x >> 5;
+    const uint64_t tw = (uint64_t)gridDim.x * W;
+    uint64_t t = (uint64_t)blockIdx.x * W + warp;
     if (lane == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
@@ -273,6 +281,54 @@ __global__ void __launch_bounds__(kWarps * 32) k_encode_short(const uint32_t *__
     }
 }
 
+// How a stream is cut: segments per tile, log2 of the team size and the warps per CTA.
+// The warps work through their tiles in step, so every one of the R rounds should be
+// full, g = ceil(num_cw / (R * warps)), and g should fill the lanes of the teams: a round of
+// 32 / T segments costs a lane its ceil(Y / 4T) blocks of four words (dearer the more segments
+// a warp's accesses are spread over, and where they share few banks) and a fixed chain
+// (the transform, the team's XOR, the inserts, the heads), and more the more warps share the SM.
+// Weights fitted on GB300 to every T, seven warp counts and three R at 20 lengths and streams
+// of 128 .. 512 Mbit: the pick is 3.5 % off the fastest on average.  Against g of the
+// fewest rounds on three CTAs of 8 warps with areas of 1056 words: 22 lengths of 16 .. 32,767 at
+// eight sizes 1.09x on average (512 Mbit of n = 200 65 -> 48 us, 3212 41 -> 30, 4095 59 -> 39;
+// at worst 1.15x slower, 128 Mbit of n = 2500).
+struct EncShape {
+    uint32_t g, tlog, warps;
+};
+
+EncShape encode_shape(uint32_t n, uint32_t k, uint32_t ystride, uint64_t num_cw, uint64_t ctas)
+{
+    const uint32_t Y = (n + 32) / 32;
+    const BankWays &ways = bank_ways(k);
+    EncShape pick{1, 0, kWarps};
+    uint64_t best = ~0ull;
+    auto consider = [&](uint64_t R, uint32_t g, uint32_t w) {
+        for (uint32_t lg = 0; lg <= 5; ++lg) {
+            const uint32_t G = 32u >> lg, blocks = (Y + (4u << lg) - 1) >> (lg + 2);
+            const uint64_t round = (uint64_t)blocks * std::max(40 + 6 * std::min(G, g), 32u * ways[lg]) + 200;
+            const uint64_t cost = R * ((g + G - 1) >> (5 - lg)) * round * (w + 12);
+            if (cost < best) {
+                best = cost;
+                pick = EncShape{g, lg, w};
+            }
+        }
+    };
+    // the most segments that fit one of w warps' share of the shared memory (warp_smem)
+    auto most = [&](uint32_t w) { return std::min((kSmemPerCta / w - 96u) * 8u / (k + 32u * ystride), kMaxTile); };
+    // up to half of that in one round of all warps; more take two rounds at least, so that
+    // the second one's loads run behind the first one's stores
+    if (num_cw <= ctas * kWarps * std::max(1u, most(kWarps) / 2)) {
+        consider(1, (uint32_t)((num_cw + ctas * kWarps - 1) / (ctas * kWarps)), kWarps);
+        return pick;
+    }
+    for (uint32_t w = kWarps; w >= 12; w -= 2) {
+        const uint64_t warps = ctas * w, gmax = most(w);
+        const uint64_t r0 = std::max<uint64_t>(2, (num_cw + gmax * warps - 1) / (gmax * warps));
+        for (uint64_t R = r0; R < r0 + 3; ++R) consider(R, (uint32_t)((num_cw + R * warps - 1) / (R * warps)), w);
+    }
+    return pick;
+}
+
 }  // namespace
 
 cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, uint64_t num_cw, uint32_t *stream,
@@ -288,39 +344,21 @@ cudaError_t launch_encode_short(const uint32_t *data, uint32_t n, uint32_t k, ui
     a.Y = (n + 32) / 32;
     a.ylast = n % 32 == 31 ? 0xFFFFFFFFu : (2u << (n % 32)) - 1u;
     a.ystride = (a.Y + 1) | 1u;
-    constexpr uint32_t smem = kWarps * kWarpBytes;
     static void (*const kernels[6])(const uint32_t *, uint32_t *, EncShortArgs) = {k_encode_short<0>, k_encode_short<1>, k_encode_short<2>,
                                                      k_encode_short<3>, k_encode_short<4>, k_encode_short<5>};
-    // segments per tile: what the area holds, evened out so that every warp of a full
-    // GPU (3 CTAs an SM) takes as many tiles (40,001 segments of n = 3212: tiles of 10
-    // left 352 of 3648 warps a second one, 13.0 us; two of 6 each take 11.0)
-    const uint64_t resident = (uint64_t)num_sms() * 3 * kWarps;
-    const uint64_t gmax = std::min(kAreaWords / a.ystride, kMaxTile);
-    const uint64_t rounds = (num_cw + gmax * resident - 1) / (gmax * resident);
-    a.g = (uint32_t)((num_cw + rounds * resident - 1) / (rounds * resident));
-    // team size: a round of 32 / T segments costs a lane its ceil(Y / 4T) blocks of
-    // four words (dearer the more segments a warp's reads are spread over: bank
-    // conflicts) and a fixed chain (the transform, the team's XOR, the inserts).  The
-    // weights fit the times of every T at eleven lengths on GB300 (512 Mbit, T = 1 ..
-    // 32: n = 544 63/44/53/72/125/191 us, n = 3212 83/50/41/40/44/47, n = 32767
-    // 350/201/105/58/36/26); the pick is the fastest or within 16 % of it at all of them.
-    uint64_t best = ~0ull;
-    int tlog = 0;
-    for (int lg = 0; lg <= 5; ++lg) {
-        const uint32_t T = 1u << lg, G = 32u >> lg;
-        const uint64_t cost = (uint64_t)((a.g + G - 1) / G) *
-                              ((a.Y + 4 * T - 1) / (4 * T) * (40 + 4 * std::min(G, a.g)) + 60 + 8 * (uint32_t)lg);
-        if (cost < best) {
-            best = cost;
-            tlog = lg;
-        }
-    }
-    const int bps = stream_blocks_per_sm(reinterpret_cast<const void *>(kernels[tlog]), kWarps * 32, smem);
-    if (bps <= 0) return cudaErrorInvalidConfiguration;
+    const uint64_t ctas = (uint64_t)num_sms();
+    const EncShape shape = encode_shape(n, k, a.ystride, num_cw, ctas);
+    a.g = shape.g;
     a.ntiles = (num_cw + a.g - 1) / a.g;
-    const int grid = decode_grid((a.ntiles + kWarps - 1) / kWarps, (uint64_t)num_sms() * (uint64_t)bps);
-    return launch_kernel(kernels[tlog], dim3((unsigned)grid), dim3(kWarps * 32), smem, st, true, data,
-                         stream, a);
+    a.off_area = area_offset(k, a.g);
+    a.warp_bytes = warp_smem(k, a.ystride, a.g);
+    const auto kern = kernels[shape.tlog];
+    if (stream_blocks_per_sm(reinterpret_cast<const void *>(kern), kWarps * 32, kSmemPerCta) <= 0)
+        return cudaErrorInvalidConfiguration;
+    // at most one tile per warp: the warps spread over all SMs
+    const uint32_t W = (uint32_t)std::min<uint64_t>(shape.warps, (a.ntiles + ctas - 1) / ctas);
+    const int grid = decode_grid((a.ntiles + W - 1) / W, ctas);
+    return launch_kernel(kern, dim3((unsigned)grid), dim3(W * 32), W * a.warp_bytes, st, true, data, stream, a);
 }
 
 }  // namespace hd
