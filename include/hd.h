@@ -357,7 +357,11 @@ typedef struct {
 /* A plan: the packet table turned into a device tile table, owned by the
  * library (allocated by hd_plan_create, freed by hd_plan_destroy).  The
  * buffers the packets point to must stay valid while the plan is launched.
- * A plan is not thread-safe: launch it from one host thread at a time. */
+ * A plan is not thread-safe: launch it from one host thread at a time.  Its
+ * launches run in the order of their calls, on whatever streams: each begins
+ * when the one before has finished.  A launch recorded into a caller's graph is
+ * ordered by that graph alone: no other launch or replay of the same plan may
+ * run beside it. */
 typedef struct hd_plan hd_plan;
 
 /* A plan decodes with one of num_variants configurations, chosen by its size

@@ -663,6 +663,12 @@ struct hd_plan {
     unsigned long long *graph_err = nullptr;
     bool graph_ok = false;
     uint64_t graph_kernels = 0;  // kernels one replay of the graph launches
+    // Launches of one plan share its claim counters, and may share their error counts: each is
+    // followed by `done`, and one on another stream than the last waits for it (CUDA orders
+    // the launches of one executable graph by itself, kernels launched directly it does not).
+    cudaEvent_t done = nullptr;
+    unsigned long long last_stream = 0;  // cudaStreamGetId: not reused, as a handle may be
+    bool launched = false;
     std::unique_ptr<LaunchGeom> geom;  // what the launches resolved on their first call
     bool geom_ok = false;
     // the split configuration: each code group's tile range (tiles are grouped
@@ -1155,6 +1161,7 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
               upload(p->d_runs, runs.data(), runs.size() * sizeof(MultiRun)) &&
               upload(p->d_rest, rest.data(), rest.size() * sizeof(DevTile)) &&
               cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess &&
               ensure_branches(p, p->variant);
     if (!ok) {
         hd_plan_destroy(p);
@@ -1164,10 +1171,9 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
     return HD_OK;
 }
 
-hd_status hd_plan_launch(hd_plan *p, unsigned long long *err_counts, void *cuda_stream)
+// One launch of the plan on `st`, behind whatever `st` holds.
+static hd_status launch_plan(hd_plan *p, unsigned long long *err_counts, cudaStream_t st)
 {
-    if (!p) return HD_ERR_NULL;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     // The single-kernel configurations are two launches (the clear and the decode, its
     // programmatic dependent): launched directly, with the geometry resolved once, as a
     // graph's would be.
@@ -1205,6 +1211,23 @@ hd_status hd_plan_launch(hd_plan *p, unsigned long long *err_counts, void *cuda_
     if (cudaGraphLaunch(p->exec, st) != cudaSuccess) return HD_ERR_CUDA;
     count_launch(p->graph_kernels);
     return HD_OK;
+}
+
+hd_status hd_plan_launch(hd_plan *p, unsigned long long *err_counts, void *cuda_stream)
+{
+    if (!p) return HD_ERR_NULL;
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    // a launch that a graph records is ordered by that graph alone
+    if (stream_capturing(st)) return launch_plan(p, err_counts, st);
+    unsigned long long id = 0;
+    if (cudaStreamGetId(st, &id) != cudaSuccess) return HD_ERR_CUDA;
+    if (p->launched && id != p->last_stream && cudaStreamWaitEvent(st, p->done, 0) != cudaSuccess) return HD_ERR_CUDA;
+    hd_status rc = launch_plan(p, err_counts, st);
+    // behind a launch that failed half way too: its first kernel may be running
+    if (cudaEventRecord(p->done, st) != cudaSuccess && rc == HD_OK) rc = HD_ERR_CUDA;
+    p->last_stream = id;
+    p->launched = true;
+    return rc;
 }
 
 hd_status hd_plan_autotune(hd_plan *p, uint32_t reps, void *cuda_stream, hd_plan_info *chosen)
@@ -1314,6 +1337,7 @@ void hd_plan_destroy(hd_plan *p)
         if (p->mjoin[b]) cudaEventDestroy(p->mjoin[b]);
     }
     if (p->fork) cudaEventDestroy(p->fork);
+    if (p->done) cudaEventDestroy(p->done);
     if (p->dmem) cudaFree(p->dmem);
     delete p;
 }

@@ -102,6 +102,17 @@ public:
     }
 };
 
+// Whether `st` records into a graph.
+inline bool stream_capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs != cudaStreamCaptureStatusNone;
+}
+
 // Launch `kern` on `st`, as the programmatic dependent of the kernel ahead of
 // it in the stream when pdl is set (it may then start before that kernel has
 // finished, and must wait for it before touching what that kernel writes).

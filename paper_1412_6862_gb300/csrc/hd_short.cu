@@ -812,16 +812,6 @@ constexpr int kMaxTables = 32;
 TableEntry g_tables[64][kMaxTables];
 uint64_t g_table_clock = 0;
 
-bool stream_capturing(cudaStream_t st)
-{
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return cs != cudaStreamCaptureStatusNone;
-}
-
 // The cached table of length n for a launch on `st` (built on a miss, which a
 // capturing stream may not do: cudaErrorStreamCaptureUnsupported).
 cudaError_t table_for(uint32_t n, uint32_t k, cudaStream_t st, TableEntry **entry)
