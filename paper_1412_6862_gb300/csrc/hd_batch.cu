@@ -17,7 +17,6 @@
 // tiles is what balances the load.
 #include <algorithm>
 #include <cstring>
-#include <memory>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -643,7 +642,26 @@ constexpr int kMaxGroups = 18;
 
 using namespace hd;
 
-struct LaunchGeom;
+// Resolve everything that touches device state before a (possibly captured)
+// enqueue: kernel attributes, occupancy, the status word address and the
+// decode tables (filled on `st` on first use; `st` must not be capturing for
+// that, else the n = 7 tiles decode arithmetically and a configuration that
+// holds the n = 15 table gives way to the built-in one).
+struct LaunchGeom {
+    int variant = 0;
+    int grid = 0;
+    uint32_t *status = nullptr;
+    const uint16_t *lut7 = nullptr, *lut15 = nullptr;
+    bool tables = false;    // every decode table that the configuration reads was there
+    uint32_t max_ctas = 0;  // hd_set_max_ctas() when the grids were chosen
+    bool split = false;
+    const BatchVariant *gk[kSplitGroups] = {};  // split: the kernel of each code group
+    int ggrid[kSplitGroups] = {};
+    bool groups = false;                        // the stream-group configuration
+    const MultiVariant *mk[kMaxGroups] = {};    // its kernel per group
+    int mgrid[kMaxGroups] = {};
+    int rest_grid = 0;                          // the batch kernel's grid for the n = 3 tiles
+};
 
 struct hd_plan {
     int device = 0;
@@ -669,7 +687,7 @@ struct hd_plan {
     cudaEvent_t done = nullptr;
     unsigned long long last_stream = 0;  // cudaStreamGetId: not reused, as a handle may be
     bool launched = false;
-    std::unique_ptr<LaunchGeom> geom;  // what the launches resolved on their first call
+    LaunchGeom geom;  // what the launches resolved
     bool geom_ok = false;
     // the split configuration: each code group's tile range (tiles are grouped
     // by n in kSplitOrder), a stream per group and the fork/join events
@@ -692,25 +710,6 @@ struct hd_plan {
     uint32_t num_rest = 0;
     cudaStream_t mstream[kMaxGroups + 1] = {};  // [0]: the n = 3 tiles; [1 + g]: group g
     cudaEvent_t mjoin[kMaxGroups + 1] = {};
-};
-
-// Resolve everything that touches device state before a (possibly captured)
-// enqueue: kernel attributes, occupancy, the status word address and the
-// decode tables (filled on `st` on first use; `st` must not be capturing for
-// that, else the n = 7 tiles decode arithmetically and a configuration that
-// holds the n = 15 table gives way to the built-in one).
-struct LaunchGeom {
-    int variant;
-    int grid;
-    uint32_t *status;
-    const uint16_t *lut7, *lut15;
-    bool split = false;
-    const BatchVariant *gk[kSplitGroups] = {};  // split: the kernel of each code group
-    int ggrid[kSplitGroups] = {};
-    bool groups = false;                        // the stream-group configuration
-    const MultiVariant *mk[kMaxGroups] = {};    // its kernel per group
-    int mgrid[kMaxGroups] = {};
-    int rest_grid = 0;                          // the batch kernel's grid for the n = 3 tiles
 };
 
 namespace {
@@ -938,11 +937,14 @@ cudaError_t prepare_plan(hd_plan *p, LaunchGeom *g, cudaStream_t st)
     g->status = status_ptr();
     if (g->status == nullptr) return cudaErrorInvalidSymbol;
     g->variant = p->variant;
+    g->max_ctas = hd_get_max_ctas();
     g->lut7 = lut_ptr(7, st);
+    g->tables = g->lut7 != nullptr;
     if (g->variant == group_variant() && !p->groups_ok) g->variant = 0;
     if (g->variant == group_variant()) {
         g->groups = true;
         g->lut15 = lut_ptr(15, st);
+        g->tables = g->tables && g->lut15 != nullptr;
         g->grid = 0;
         if (p->num_rest != 0) {
             g->rest_grid = batch_grid(batch_variants()[0], p->num_rest);
@@ -966,6 +968,7 @@ cudaError_t prepare_plan(hd_plan *p, LaunchGeom *g, cudaStream_t st)
     if (g->variant >= split_variant()) {
         g->split = true;
         g->lut15 = lut_ptr(15, st);
+        g->tables = g->tables && g->lut15 != nullptr;
         g->grid = 0;
         const SplitKernels &sk = split_kernels()[g->variant - split_variant()];
         for (int gi = 0; gi < kSplitGroups; ++gi) {
@@ -979,7 +982,10 @@ cudaError_t prepare_plan(hd_plan *p, LaunchGeom *g, cudaStream_t st)
         return cudaSuccess;
     }
     g->lut15 = batch_variants()[g->variant].t15 ? lut_ptr(15, st) : nullptr;
-    if (batch_variants()[g->variant].t15 && g->lut15 == nullptr) g->variant = 0;
+    if (batch_variants()[g->variant].t15 && g->lut15 == nullptr) {
+        g->variant = 0;
+        g->tables = false;
+    }
     g->grid = batch_grid(batch_variants()[g->variant], p->num_tiles);
     return g->grid > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
@@ -1080,7 +1086,6 @@ void drop_graph(hd_plan *p)
 void drop_plan(hd_plan *p)
 {
     drop_graph(p);
-    p->geom.reset();
     p->geom_ok = false;
 }
 
@@ -1176,20 +1181,24 @@ static hd_status launch_plan(hd_plan *p, unsigned long long *err_counts, cudaStr
 {
     // The single-kernel configurations are two launches (the clear and the decode, its
     // programmatic dependent): launched directly, with the geometry resolved once, as a
-    // graph's would be.
-    if (!p->geom_ok) {
-        p->geom = std::make_unique<LaunchGeom>();
-        if (prepare_plan(p, p->geom.get(), st) != cudaSuccess) return HD_ERR_CUDA;
-        p->geom_ok = true;
+    // graph's would be.  It is resolved again where a decode table was missing (filled by
+    // the first launch that no capture records) and, unless a recorded graph is replayed,
+    // under another cap on the CTAs.
+    const bool recorded = p->graph_ok && p->graph_err == err_counts;
+    if (!p->geom_ok || (!recorded && p->geom.max_ctas != hd_get_max_ctas())) {
+        drop_plan(p);
+        p->geom = LaunchGeom{};
+        if (prepare_plan(p, &p->geom, st) != cudaSuccess) return HD_ERR_CUDA;
+        p->geom_ok = p->geom.tables;
     }
-    if (!p->geom->split && !p->geom->groups) {
-        if (enqueue_plan(p, *p->geom, err_counts, st) != cudaSuccess) return HD_ERR_CUDA;
+    if (!p->geom.split && !p->geom.groups) {
+        if (enqueue_plan(p, p->geom, err_counts, st) != cudaSuccess) return HD_ERR_CUDA;
         if (p->num_tiles) count_launch();  // the clear is counted where it is enqueued
         return HD_OK;
     }
     if (!p->graph_ok || p->graph_err != err_counts) {
         drop_graph(p);
-        const LaunchGeom &geom = *p->geom;
+        const LaunchGeom &geom = p->geom;
         if (cudaStreamBeginCapture(p->capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return HD_ERR_CUDA;
         const cudaError_t e = enqueue_plan(p, geom, err_counts, p->capture);
         g_launches.fetch_sub(1, std::memory_order_relaxed);  // the clear recorded here runs (and counts) per replay
