@@ -195,30 +195,39 @@ hd_status hd_decode_streams(const hd_stream_job *jobs, uint32_t num_jobs, void *
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return HD_ERR_CUDA;
     }
-    // the largest streams first, so that the shorter ones fill in around them
-    uint32_t order[kMaxStreamJobs], count = 0;
-    for (uint32_t i = 0; i < num_jobs; ++i)
-        if (jobs[i].num_codewords != 0) order[count++] = i;
-    std::sort(order, order + count, [&](uint32_t x, uint32_t y) {
-        return (uint64_t)jobs[x].n * jobs[x].num_codewords > (uint64_t)jobs[y].n * jobs[y].num_codewords;
+    // the streams that fill the GPU first, the largest ahead, so that the others fill in around
+    // them.  (By size alone a stream of few long codewords that the lanes decode may come ahead
+    // of one of many short codewords that they do not.)
+    struct Branched {
+        DecodeJob job;
+        bool lanes;
+    };
+    Branched order[kMaxStreamJobs];
+    uint32_t count = 0, big = 0;
+    for (uint32_t i = 0; i < num_jobs; ++i) {
+        const hd_stream_job &j = jobs[i];
+        if (j.num_codewords == 0) continue;
+        const DecodeJob d = decode_job(j.stream, j.n, j.num_codewords, j.out_bits, j.syndromes,
+                                       static_cast<hd_syn_type>(j.syn_type), j.err_count);
+        order[count] = Branched{d, decodes_by_lanes(d)};
+        big += !order[count++].lanes;
+    }
+    std::sort(order, order + count, [](const Branched &x, const Branched &y) {
+        return x.lanes != y.lanes ? y.lanes : x.job.n * x.job.num_cw > y.job.n * y.job.num_cw;
     });
     // One branch per stream that fills the GPU, the largest on the caller's stream itself;
     // the short ones (one codeword per lane, 2 to 4 us each) share a branch, chained: an
     // event wait, a record and a wait each cost more than running them one after another.
-    uint32_t big = 0;
-    while (big < count && !lanes_suffice(jobs[order[big]].n, false, jobs[order[big]].num_codewords)) ++big;
     const uint32_t branches = big + (big < count ? 1u : 0u);
     const int pooled = (int)std::min<uint32_t>(branches > 0 ? branches - 1 : 0, kPoolStreams);
     if (pooled > 0 && cudaEventRecord(pool.fork, st) != cudaSuccess) return HD_ERR_CUDA;
     for (int i = 0; i < pooled; ++i)
         if (cudaStreamWaitEvent(pool.s[i], pool.fork, 0) != cudaSuccess) return HD_ERR_CUDA;
     for (uint32_t r = 0; r < count; ++r) {
-        const hd_stream_job &j = jobs[order[r]];
         const uint32_t branch = std::min(r, big);
         const bool chained = r > big;  // behind another decode of this call
-        if (launch_decode(decode_job(j.stream, j.n, j.num_codewords, j.out_bits, j.syndromes,
-                                     static_cast<hd_syn_type>(j.syn_type), j.err_count),
-                          branch == 0 ? st : pool.s[(branch - 1) % kPoolStreams], chained) != cudaSuccess)
+        if (launch_decode(order[r].job, branch == 0 ? st : pool.s[(branch - 1) % kPoolStreams], chained) !=
+            cudaSuccess)
             return HD_ERR_CUDA;
     }
     for (int i = 0; i < pooled; ++i)

@@ -248,9 +248,11 @@ bool secded_variant_pinned(uint32_t n, int syn)
     return g_secded_choice.count({current_device(), n, syn}) != 0;
 }
 
-cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl)
+// The streaming configuration that decodes a plain-code job, or nullptr for one
+// codeword per lane.
+static const StreamVariant *stream_variant(const DecodeJob &j)
 {
-    if (!variant_pinned(j.n, j.syn_type) && lanes_suffice(j.n, j.xh, j.num_cw)) return launch_decode_lanes(j, false, st, pdl);
+    if (!variant_pinned(j.n, j.syn_type) && lanes_suffice(j.n, j.xh, j.num_cw)) return nullptr;
     const StreamVariant *v = nullptr;
     if (j.n == 3) {
         v = variant_n3(j.syn_type);
@@ -258,9 +260,17 @@ cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl)
         const int idx = chosen_variant(j.n, j.syn_type);
         if (idx >= 0) v = &variants()[idx];
     }
+    return v != nullptr && j.num_cw >= v->chunk_cw ? v : nullptr;  // at least one whole chunk
+}
+
+bool decodes_by_lanes(const DecodeJob &j) { return stream_variant(j) == nullptr; }
+
+cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl)
+{
+    const StreamVariant *v = stream_variant(j);
     const uint16_t *lut = v != nullptr && v->lut ? lut_ptr(j.n, st) : nullptr;
-    // no whole chunk, or no table yet (first call inside a capture)
-    if (v == nullptr || j.num_cw < v->chunk_cw || (v->lut && lut == nullptr)) return launch_decode_lanes(j, false, st, pdl);
+    // no table yet: first call inside a capture
+    if (v == nullptr || (v->lut && lut == nullptr)) return launch_decode_lanes(j, false, st, pdl);
     uint32_t *status = status_ptr();
     if (status == nullptr) return cudaErrorInvalidSymbol;
     return v->launch(stream_args(*v, j, status, lut), st, pdl);

@@ -158,6 +158,8 @@ cudaError_t launch_zero_counts(unsigned long long *a, unsigned long long *b, cud
 // its ragged tail, or one codeword per lane.  The counters are added to.  pdl:
 // launched as the programmatic dependent of the kernel ahead.
 cudaError_t launch_decode(const DecodeJob &j, cudaStream_t st, bool pdl);
+// Whether launch_decode takes a job one codeword per lane.
+bool decodes_by_lanes(const DecodeJob &j);
 cudaError_t launch_decode_secded(const DecodeJob &j, cudaStream_t st, bool pdl);
 
 // Whether the caller pinned a configuration (hd_variant_select, not the
