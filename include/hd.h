@@ -90,8 +90,8 @@ hd_status hd_decode(const uint32_t *stream, uint64_t in_bits, uint32_t n, uint64
  * on `cuda_stream` itself, the others forked from it onto library-owned
  * streams (8 per device, created by the first call on a device, which should
  * come before any stream capture) and joined back into it, the short ones one
- * behind another in a branch of their own: work enqueued on `cuda_stream`
- * after this call waits for every job.  Decoding the streams side by side lets
+ * behind another in a branch of their own (in a capture side by side as well):
+ * work enqueued on `cuda_stream` after this call waits for every job.  Decoding the streams side by side lets
  * one decode's ramp-up and drain overlap another's steady state, the
  * pipelining of independent packets the paper applies to its transfers
  * (Sec. III-B).  At most 32 jobs per call (HD_ERR_CAPACITY); the jobs' output

@@ -56,3 +56,11 @@ def test_pinned_short_stream_has_a_branch():
     finally:
         hd.hd_variant_select(63, hd.SYN_U8, -1)
     assert c.depth <= 3 and len(c.kernels) == 4
+
+
+def test_short_streams_side_by_side_when_captured():
+    # the caller's stream and eight branches: ten streams, the last one behind another
+    specs = [((7, 15, 31, 63)[i % 4], 20_000 - i) for i in range(10)]
+    c = _run(specs[:9])
+    assert c.depth == 2 and len(c.kernels) == 10
+    assert _run(specs).depth == 3
