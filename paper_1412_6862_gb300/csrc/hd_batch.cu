@@ -295,15 +295,14 @@ __global__ void __launch_bounds__(WARPS * 32)
     // The first tiles of the all-n kernel (its S stages and the one behind them) are
     // dealt too, and the counter counts from there: S + 1 claims before the first load,
     // each an atomic's round trip and its descriptor's, were 4 to 6 us of every launch
-    // (300 packets, 12-warp CTAs: 18.5 us with them, 12.7 without).
+    // (300 packets, 12-warp CTAs: 18.5 us with them, 12.7 without).  A claim stays as the
+    // atomic returned it until the next iteration, which adds that start: a sum right behind
+    // the atomic waits out its round trip in every iteration (8000 packets of n = 63, 1-warp
+    // CTAs: 154.2 us so, 146.2 now; 8000 of six codes 198 / 191).
     const uint64_t gw = (uint64_t)blockIdx.x * WARPS + (uint64_t)warp, tw = (uint64_t)gridDim.x * WARPS;
-    constexpr uint32_t kDealt = S + 1;
+    const uint32_t claim0 = (S + 1) * (uint32_t)tw;  // the first tile that is claimed
     uint32_t seq = 0;  // lane 0: tiles dealt to this warp so far
     auto deal = [&]() -> uint32_t {
-        if (NSEL == 0 && seq >= kDealt) {
-            const uint64_t t = kDealt * tw + atomicAdd(counter, 1u);
-            return t < (uint64_t)num_tiles ? (uint32_t)t : num_tiles;
-        }
         const uint64_t t = gw + (uint64_t)(seq++) * tw;
         return t < (uint64_t)num_tiles ? (uint32_t)t : num_tiles;
     };
@@ -366,10 +365,12 @@ __global__ void __launch_bounds__(WARPS * 32)
         if (lane == 0 && it > 0) {
             if constexpr (kAhead2) {
                 if (after_t < num_tiles) after_d = tiles[after_t];  // used at the end of the next iteration
+                later_t = deal();  // its descriptor is fetched next iteration
             } else {
+                if (it > 1) next_t += claim0;  // the first one was dealt
                 if (next_t < num_tiles) next_d = tiles[next_t];  // used at the end of this iteration
+                later_t = atomicAdd(counter, 1u);
             }
-            later_t = deal();  // its descriptor is fetched next iteration
         }
         const DevTile tl = desc[s];  // written by lane 0 before the stage's arrive
         // the single-n kernels know n at compile time: the per-tile index
