@@ -900,20 +900,59 @@ inline int split_variant() { return (int)batch_variants().size(); }
 inline int group_variant() { return split_variant() + (int)split_kernels().size(); }
 inline int plan_variants() { return group_variant() + 1; }
 
-// The configuration of a new plan, until it is tuned or selected.  On GB300, packets
-// of 64 bit .. 4 Mbit of mixed n with u8 syndromes (time of 1-warp CTAs with two
-// stages (1), 4-warp (4), 12- and 14-warp CTAs around the n = 15 table (6, 7), stream
-// groups (9)): 100 packets 13.4 / 9.5 / 10.4 / 10.4 / 15.4 us, 300 (3800 tiles) 16.6 /
-// 15.9 / 12.7 / 14.5 / 18.8, 1000 34.4 / 39.5 / 34.8 / 34.1 / 45.6, 3000 (0.3 GB moved)
-// 83.8 / 102.9 / 88.4 / 85.0 / 107.3, 10,000 (1 GB) 247 / 300 / 268 / 251 / 223.
-// Without n = 15 packets the table only takes room.
-int default_plan_variant(const hd_plan *p, bool has15)
+// The bytes a plan moves (inputs, outputs and syndromes), and those of some code lengths.
+struct PlanBytes {
+    uint64_t all = 0, n3 = 0, n7 = 0, n15 = 0, n127 = 0, n255 = 0;
+    bool u8 = false;  // some packet of n = 7 has u8 syndromes
+};
+
+PlanBytes plan_bytes(const std::vector<DevPacket> &pk)
 {
-    constexpr uint64_t kGroupBytes = 768ull << 20;  // the stream groups' ramps and drains pay off
-    if (p->groups_ok && p->in_bytes + p->out_bytes + p->syn_bytes >= kGroupBytes) return group_variant();
+    PlanBytes b;
+    for (const DevPacket &d : pk) {
+        const uint64_t bytes = d.num_cw * (2u * d.n - d.m) / 8 + d.num_cw * d.syn_type;
+        b.all += bytes;
+        if (d.n == 3) b.n3 += bytes;
+        if (d.n == 7) b.n7 += bytes, b.u8 = b.u8 || d.syn_type == 1;
+        if (d.n == 15) b.n15 += bytes;
+        if (d.n == 127) b.n127 += bytes;
+        if (d.n == 255) b.n255 += bytes;
+    }
+    return b;
+}
+
+// The configuration of a new plan, until it is tuned or selected: 1-warp CTAs with three
+// or two stages (0, 1), 4-warp (4), 12- and 14-warp CTAs around the n = 15 table (6, 7) or
+// the stream groups (9).  All on GB300; packets of 64 bit .. 4 Mbit, u8 syndromes unless said.
+//  * Few tiles.  Mixed n: 100 packets (1) 13.4 / (4) 9.5 / (6) 10.4 / (7) 10.4 / (9) 15.4 us, 300
+//    (3800 tiles) 16.6 / 15.9 / 12.7 / 14.5 / 18.8, 1000 34.4 / 39.5 / 34.8 / 34.1 / 45.6.
+//  * The stream groups from 768 MB on, where their ramps and drains pay off: six codes at 719 MB
+//    (0) 166 / (9) 174 us, 835 MB 187 / 190, 1025 MB 275 / 225.  They do not where n = 7
+//    makes up most of the bytes, unless n = 15 has its share: n = 7 alone at 878 MB 162 / 185,
+//    with n = 63 at 918 MB 169 / 187, with n = 15 at 854 MB 206 / 173.  With two fifths of n = 127
+//    from 512 MB on: on some buffers (not on others of the same size) the claiming kernels take
+//    up to twice their time for as long as they run, at full clocks, the groups do not (n = 127
+//    alone, 650 MB 120 .. 197 / 123 .. 135, 932 MB 157 .. 313 / 173; 472 MB 86 / 91).
+//  * Many tiles: three stages.  n = 63 alone, 90,000 tiles (0) 122 / (1) 129, 25,000 45.6 / 45.8; all
+//    but n = 15, 33,000 63.0 / 65.1, 25,000 51.5 / 50.3.  Two stages for n = 255 and 15 (62,000
+//    tiles, n = 255 with a tenth of 15, 144 / 139), n = 7 alone without u8 syndromes (59,000
+//    tiles u16 147 / 144, u8 101 / 105) and n = 3 (45,000 tiles 155 / 142).
+//  * The n = 15 table with many tiles for a quarter of n = 15 (by bytes; with n = 63, 63,000
+//    tiles: (7) 113 / (0) 134), and for an eighth of it, as a mix of six codes has, up to 36,864
+//    tiles (25,000 58 / 63, 33,000 74 / 76, 40,000 89 / 87, 61,000 127 / 122).  Below an eighth it
+//    only takes room (a tenth in n = 255, 13,700 tiles: (7) 41.4 / (1) 40.6, 25,600 70.1 / 65.0).
+int default_plan_variant(const hd_plan *p, const PlanBytes &b)
+{
+    constexpr uint64_t kMB = 1ull << 20;
+    constexpr uint32_t kManyTiles = 28 << 10, kMixedTable = 36 << 10;
+    if (p->groups_ok && ((b.all >= 768 * kMB && (2 * b.n7 <= b.all || 4 * b.n15 >= b.all)) ||
+                         (b.all >= 512 * kMB && 5 * b.n127 >= 2 * b.all)))
+        return group_variant();
     if (p->num_tiles < 2048) return 4;
-    if (!has15) return 1;
-    return p->num_tiles < 8192 ? 6 : 7;
+    const bool table = 8 * b.n15 >= b.all;
+    if (p->num_tiles < kManyTiles) return !table ? 1 : p->num_tiles < 8192 ? 6 : 7;
+    if (4 * b.n15 >= b.all || (table && p->num_tiles < kMixedTable)) return 7;
+    return 2 * (b.n15 + b.n255) >= b.all || 16 * b.n3 >= b.all || (b.n7 == b.all && !b.u8) ? 1 : 0;
 }
 
 // The streams and events that a configuration's branches and graph need, created when
@@ -1144,8 +1183,7 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
     p->num_packets = num_packets;
     p->num_tiles = (uint32_t)tiles.size();
     p->num_rest = (uint32_t)rest.size();
-    p->variant = default_plan_variant(
-        p, std::any_of(pk.begin(), pk.end(), [](const DevPacket &d) { return d.n == 15 && d.num_cw != 0; }));
+    p->variant = default_plan_variant(p, plan_bytes(pk));
     auto rounded = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t tl_b = rounded(tiles.size() * sizeof(DevTile)), sp_b = rounded(split.size() * sizeof(DevTile));
     const size_t ru_b = rounded(runs.size() * sizeof(MultiRun)), re_b = rounded(rest.size() * sizeof(DevTile));
