@@ -231,15 +231,15 @@ hd_status hd_decode_short_plan(const hd_short_plan *plan, const uint32_t *stream
 void hd_short_plan_destroy(hd_short_plan *plan);
 
 /* The tiled kernel has several configurations (warps per CTA, stage bytes);
- * configuration 0 is the built-in choice by length and size.
+ * configuration 0 is the built-in choice of these by length and size, and the
+ * last one decodes one segment per lane (n < 960; longer ones as configuration 0).
  * hd_short_variant_select() pins one configuration for every length on the
  * current device (ordinal < 0 removes the pin); hd_short_autotune() times
  * every configuration on `num_codewords` all-zero segments of length n (reps
  * launches each, 0 = 5; it allocates its own scratch buffers and synchronises
- * `cuda_stream`) and keeps the fastest for n on the current device, returned
- * in *chosen (-1 when n has a single kernel, k < 64); below n = 960 it is kept
- * only if it also beats decoding one segment per lane.  A configuration never
- * changes the result, only the speed. */
+ * `cuda_stream`) and keeps the fastest for n on the current device, for
+ * streams of any size, returned in *chosen (-1 when n has a single kernel,
+ * k < 64).  A configuration never changes the result, only the speed. */
 hd_status hd_short_variant_count(uint32_t *count);
 hd_status hd_short_variant_select(int32_t ordinal);
 hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, void *cuda_stream, int32_t *chosen);

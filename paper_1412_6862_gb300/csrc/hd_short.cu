@@ -582,6 +582,7 @@ struct ShortVariant {
 const ShortVariant kShortVariants[] = {{0, 0}, {24, 8192}, {24, 6144}, {16, 6144}, {16, 4096}, {12, 4096}, {8, 8192}};
 const ShortVariant kSharedTable = {24, 8192}, kGlobalTable = {16, 7168};
 constexpr int kNumShortVariants = sizeof(kShortVariants) / sizeof(kShortVariants[0]);
+constexpr int kLanes = kNumShortVariants;  // the configuration behind them: one codeword per lane, n < kLaneMaxN
 
 using TileKernel = void (*)(const uint32_t *, uint32_t *, void *, unsigned long long *, unsigned long long *,
                             const void *, ShortArgs);
@@ -646,7 +647,6 @@ int chosen_short_variant(uint32_t n)
     return -1;
 }
 
-// v < 0 forgets the length.
 void remember_short_variant(uint32_t n, int v)
 {
     int dev = 0;
@@ -661,7 +661,6 @@ void remember_short_variant(uint32_t n, int v)
         }
         if (!slot && e.v < 0) slot = &e;
     }
-    if (v < 0 && (!slot || slot->n != n)) return;
     if (!slot) slot = &g_short_tuned[dev][n % 64];  // table full: overwrite one entry
     slot->n = n;
     slot->v = v;
@@ -1025,7 +1024,8 @@ hd_status decode_short_with(const uint32_t *stream, uint64_t in_bits, uint32_t n
     // the tiled kernel from kLaneMaxN on, and below it (k >= 64) where a configuration is
     // pinned or the autotuner found one faster
     int vi = k >= kLongMinK ? chosen_short_variant(n) : -1;
-    if (vi < 0 && n < kLaneMaxN && (n < kLaneTileN || num_codewords * n < kLaneTileBits))
+    if (vi == kLanes && n >= kLaneMaxN) vi = 0;
+    if (vi == kLanes || (vi < 0 && n < kLaneMaxN && (n < kLaneTileN || num_codewords * n < kLaneTileBits)))
         return launch_short_lanes(stream, n, num_codewords, out_bits, syndromes, syn, err_count, detected_count, st,
                                   false) == cudaSuccess
                    ? HD_OK
@@ -1181,8 +1181,7 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
             best_ms = ms;
         }
     }
-    // below kLaneMaxN a configuration is kept only if it beats one codeword per lane
-    bool beaten = false;
+    // below kLaneMaxN a tile configuration is kept only if it beats one codeword per lane
     if (rc == HD_OK && best >= 0 && n < kLaneMaxN) {
         auto go = [&]() {
             return launch_short_lanes(static_cast<const uint32_t *>(din), n, num_codewords, static_cast<uint32_t *>(dout),
@@ -1194,7 +1193,7 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
         for (uint32_t i = 0; rc == HD_OK && i < reps; ++i) go();
         cudaEventRecord(e1, st);
         if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) rc = HD_ERR_CUDA;
-        beaten = ms <= best_ms;
+        if (ms <= best_ms) best = kLanes;
     }
     if (tab) table_used(tab, st);
     if (din) cudaFree(din);
@@ -1204,7 +1203,7 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (rc != HD_OK) return rc;
-    if (best >= 0) remember_short_variant(n, beaten ? -1 : best);
+    if (best >= 0) remember_short_variant(n, best);
     if (chosen) *chosen = best;
     return HD_OK;
 }
@@ -1212,13 +1211,13 @@ hd_status hd_short_autotune(uint32_t n, uint64_t num_codewords, uint32_t reps, v
 hd_status hd_short_variant_count(uint32_t *count)
 {
     if (!count) return HD_ERR_NULL;
-    *count = (uint32_t)kNumShortVariants;
+    *count = (uint32_t)kLanes + 1u;
     return HD_OK;
 }
 
 hd_status hd_short_variant_select(int32_t ordinal)
 {
-    if (ordinal >= kNumShortVariants) return HD_ERR_INVALID_ARG;
+    if (ordinal > kLanes) return HD_ERR_INVALID_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HD_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_short_mu);

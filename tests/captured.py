@@ -12,7 +12,8 @@ class _KernelParams(ctypes.Structure):
 
 
 class Captured:
-    """kernels: the grid size of every kernel node; depth: kernels on the longest chain."""
+    """kernels: the grid size of every kernel node; functions: their kernels; depth: kernels on
+    the longest chain."""
 
     def __init__(self, call):
         import torch
@@ -32,7 +33,7 @@ class Captured:
         check(rc)
         nodes, n = (ctypes.c_void_p * _HANDLES)(), ctypes.c_size_t(_HANDLES)
         check(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
-        grids = {}
+        grids, self.functions = {}, []
         for i in range(n.value):
             kind = ctypes.c_int()
             check(cu.cuGraphNodeGetType(ctypes.c_void_p(nodes[i]), ctypes.byref(kind)))
@@ -40,6 +41,7 @@ class Captured:
                 kp = _KernelParams()
                 check(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(nodes[i]), ctypes.byref(kp)))
                 grids[nodes[i]] = kp.grid[0]
+                self.functions.append((kp.func, kp.kern))
         src, dst, data = (ctypes.c_void_p * _HANDLES)(), (ctypes.c_void_p * _HANDLES)(), (ctypes.c_uint64 * _HANDLES)()
         e = ctypes.c_size_t(_HANDLES)
         check(cu.cuGraphGetEdges_v2(graph, src, dst, data, ctypes.byref(e)))
