@@ -501,7 +501,10 @@ def code_params(n: int) -> tuple[int, int]:
     """(m, k) for n = 2^m - 1, 2 <= m <= 8."""
     try:
         return _CODES[n]
-    except KeyError:
+    except (KeyError, TypeError):  # a tensor or array of one element: equal to its length, not found by hash
+        for length, code in _CODES.items():
+            if n == length:
+                return code
         raise HDError(HD_ERR_INVALID_N, f"n={n}") from None
 
 
