@@ -186,7 +186,6 @@ struct BatchCfg {
     static constexpr uint32_t off_lut_bar = off_lut15 + lut15_bytes;
     static constexpr uint32_t smem = off_lut_bar + 16;
     static_assert(S >= 2 && S <= 8, "refills lag one iteration: at least two stages");
-    static_assert(kBatchSynBytes >= 32 * lane_slot_words(8) * 4, "a lane tile's slots fit the syndrome buffer");
     static_assert(smem <= 232448, "shared memory per CTA");
 };
 

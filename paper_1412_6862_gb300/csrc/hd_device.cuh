@@ -34,13 +34,6 @@ __host__ __device__ constexpr uint32_t qmask(int n, int i)
     return mk;
 }
 
-// Data run j (j >= 1) covers positions 2^j + 1 .. 2^(j+1) - 1; in the compacted
-// data word it starts at bit 2^j - j - 1.  This is the mask of its bits there.
-__host__ __device__ constexpr uint32_t run_mask(int j)
-{
-    return (uint32_t)(((1ull << ((1 << j) - 1)) - 1ull) << ((1 << j) - j - 1));
-}
-
 // shl.b32 clamps shift amounts above 32 to 32, which yields 0: used for the
 // branch-free flip of a bit that may live in another word.
 __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t sh)
