@@ -403,18 +403,19 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
 
 /* Decode every packet of the plan on `cuda_stream`.  err_counts: device array
  * of num_packets elements, or NULL; element i is overwritten with packet i's
- * number of nonzero syndromes.  The first launch (and any launch with a
- * different err_counts pointer) records the launch as a CUDA graph; later
- * launches replay it.  n = 7 packets decode with a 256-byte table that the
- * first batched decode on a device fills on `cuda_stream` and then
- * synchronises it (a launch whose stream is capturing before that decodes
- * n = 7 arithmetically). */
+ * number of nonzero syndromes.  The configurations of one kernel are launched
+ * directly: the counters' clear and the decode.  The split and stream-group
+ * configurations are recorded as a CUDA graph by the first launch (and any
+ * launch with a different err_counts pointer) and replayed; they cannot be
+ * launched on a capturing stream (HD_ERR_CUDA).  n = 7 packets decode with a
+ * 256-byte table that the first batched decode on a device fills on
+ * `cuda_stream` and then synchronises it (a launch whose stream is capturing
+ * before that decodes n = 7 arithmetically, later ones with the table). */
 hd_status hd_plan_launch(hd_plan *plan, unsigned long long *err_counts, void *cuda_stream);
 
 /* Time every batch-kernel configuration on the plan's own packets as
- * hd_plan_launch() runs it (recorded as a CUDA graph, then `reps` replays,
- * 0 = 3; output buffers are overwritten, inputs only read), keep the fastest
- * and report it.  The next hd_plan_launch() records its graph anew.
+ * hd_plan_launch() runs it (one launch, then `reps` timed ones, 0 = 3; output
+ * buffers are overwritten, inputs only read), keep the fastest and report it.
  * Synchronises the stream. */
 hd_status hd_plan_autotune(hd_plan *plan, uint32_t reps, void *cuda_stream, hd_plan_info *chosen);
 
@@ -602,8 +603,9 @@ uint64_t hd_launch_count(void);
  * tiles to walk through; results never change.  Uses: leaving SMs free for
  * other kernels that run beside the decoder, and tests that make every warp's
  * staging ring wrap many times on inputs small enough for the CPU oracle.
- * Launch geometry already recorded in a CUDA graph (a plan's graph, recorded
- * on its first launch) keeps its grid.  Host only; always HD_OK. */
+ * Launch geometry already recorded in a CUDA graph (the caller's, or that of a
+ * split or stream-group plan until its err_counts pointer or configuration
+ * changes) keeps its grid.  Host only; always HD_OK. */
 hd_status hd_set_max_ctas(uint32_t max_ctas);
 
 /* The cap set by hd_set_max_ctas() (0 = none). */

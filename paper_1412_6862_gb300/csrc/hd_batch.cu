@@ -642,11 +642,11 @@ constexpr int kMaxGroups = 18;
 
 using namespace hd;
 
-// Resolve everything that touches device state before a (possibly captured)
-// enqueue: kernel attributes, occupancy, the status word address and the
-// decode tables (filled on `st` on first use; `st` must not be capturing for
-// that, else the n = 7 tiles decode arithmetically and a configuration that
-// holds the n = 15 table gives way to the built-in one).
+// What prepare_plan resolves before a (possibly captured) enqueue, everything that
+// touches device state: kernel attributes, occupancy, the status word address
+// and the decode tables (filled on the launching stream on first use; it must not
+// be capturing for that, else the n = 7 tiles decode arithmetically and a
+// configuration that holds the n = 15 table gives way to variant 0).
 struct LaunchGeom {
     int variant = 0;
     int grid = 0;
@@ -1288,8 +1288,8 @@ hd_status hd_plan_autotune(hd_plan *p, uint32_t reps, void *cuda_stream, hd_plan
     float best_us = 0.f;
     const int keep = p->variant;
     hd_status rc = HD_OK;
-    // every configuration timed as hd_plan_launch runs it: recorded as a CUDA
-    // graph, then replayed (err_counts NULL: the counts are not part of the choice)
+    // every configuration timed as hd_plan_launch runs it, directly or by replays of its
+    // graph (err_counts NULL: the counts are not part of the choice)
     for (int i = 0; i < plan_variants(); ++i) {
         p->variant = i;
         if (!ensure_branches(p, i)) {
@@ -1299,7 +1299,7 @@ hd_status hd_plan_autotune(hd_plan *p, uint32_t reps, void *cuda_stream, hd_plan
         LaunchGeom geom;
         if (prepare_plan(p, &geom, st) != cudaSuccess || geom.variant != i) continue;
         drop_plan(p);
-        if ((rc = hd_plan_launch(p, nullptr, st)) != HD_OK) break;  // records the graph and runs it once
+        if ((rc = hd_plan_launch(p, nullptr, st)) != HD_OK) break;  // resolves it, records a graph where it has one
         cudaEventRecord(e0, st);
         for (uint32_t r = 0; r < reps; ++r)
             if ((rc = hd_plan_launch(p, nullptr, st)) != HD_OK) break;

@@ -607,7 +607,7 @@ def hd_short_variant_select(ordinal: int) -> None:
 
 
 def hd_short_autotune(n: int, num_codewords: int, reps: int = 5, cuda_stream=None) -> int:
-    """Time every tile configuration for length n; returns the chosen ordinal (-1: single kernel)."""
+    """Time every configuration for length n; returns the chosen ordinal (-1: single kernel)."""
     chosen = _c.c_int32(-2)
     check(lib().hd_short_autotune(n, num_codewords, reps, _stream_handle(cuda_stream), ctypes.byref(chosen)),
           "hd_short_autotune")
