@@ -406,8 +406,8 @@ hd_status hd_plan_create(const hd_packet *table, uint32_t num_packets, hd_plan *
  * number of nonzero syndromes.  The configurations of one kernel are launched
  * directly: the counters' clear and the decode.  The split and stream-group
  * configurations are recorded as a CUDA graph by the first launch (and any
- * launch with a different err_counts pointer) and replayed; they cannot be
- * launched on a capturing stream (HD_ERR_CUDA).  n = 7 packets decode with a
+ * launch with a different err_counts pointer) and replayed; a capturing stream
+ * records their kernels as it does the others'.  n = 7 packets decode with a
  * 256-byte table that the first batched decode on a device fills on
  * `cuda_stream` and then synchronises it (a launch whose stream is capturing
  * before that decodes n = 7 arithmetically, later ones with the table). */

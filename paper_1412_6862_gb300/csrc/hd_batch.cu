@@ -1229,9 +1229,11 @@ static hd_status launch_plan(hd_plan *p, unsigned long long *err_counts, cudaStr
         if (prepare_plan(p, &p->geom, st) != cudaSuccess) return HD_ERR_CUDA;
         p->geom_ok = p->geom.tables;
     }
-    if (!p->geom.split && !p->geom.groups) {
+    // In a capture the others too: their forks and joins become edges of the caller's graph,
+    // where a graph of their own could not be launched.
+    if ((!p->geom.split && !p->geom.groups) || stream_capturing(st)) {
         if (enqueue_plan(p, p->geom, err_counts, st) != cudaSuccess) return HD_ERR_CUDA;
-        if (p->num_tiles) count_launch();  // the clear is counted where it is enqueued
+        count_launch(plan_kernels(p, p->geom) - 1);  // the clear is counted where it is enqueued
         return HD_OK;
     }
     if (!p->graph_ok || p->graph_err != err_counts) {
